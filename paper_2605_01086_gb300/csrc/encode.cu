@@ -14,23 +14,12 @@
 //                 computes again in FP64 (products and sums rounded
 //                 separately, in sample order, then scaled by 2/N, as the host
 //                 encoder does), one bin per lane, and quantizes from that.
-//   k_enc_ref     one thread per packing block of kPackBlock symbols: Alg. 1
-//                 on the block alone, entered with a word that starts at its
-//                 first symbol (the reference packing): the words it closes
-//                 and the state it ends in; then the next block of the stream
-//                 packed from that state beside the next block's reference
-//                 until the two start a word at the same symbol (from there
-//                 on they coincide): the next block's transfer.
-//   k_enc_scan    one warp per stream: the word counts added up block after
-//                 block (a block entered in another state is walked again
-//                 from the true one); each block's entry state; zeroes the
-//                 words two blocks share; the stream's word count, room and
-//                 code checks.
-//   k_enc_pack    one thread per block: Alg. 1 from the block's entry state,
-//                 whole words staged in shared memory and written out per
-//                 warp, the words shared with the previous or next block with
-//                 64-bit atomicOr (their codeword bits are disjoint), each
-//                 word's symbol count by the block that closes it.
+//   k_enc_starts  one warp per packing block of kPackBlock symbols: where
+//                 words start in it (Alg. 1), as a bitmap of its symbols.
+//   k_enc_scan    one warp per stream: the words before each block; the
+//                 stream's word count, room and code checks.
+//   k_enc_pack    one warp per 2048 symbols, one lane per word: the words'
+//                 codewords put together and written, with their counts.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -48,12 +37,12 @@
 namespace fptc {
 namespace {
 
-constexpr uint32_t kPackBlock = 8192;  // symbols per packing block
+constexpr uint32_t kPackBlock = 8192;            // symbols per packing block
+constexpr uint32_t kMaskWords = kPackBlock / 32;  // words of its bitmap of word starts
 
 struct EncDomain {
   uint32_t N, E, B1, B2;
   uint32_t cos_off;   // first entry of the E x N cosine tables (FP64 and FP32 copies)
-  uint32_t code_off;  // first entry of the 256 codewords / lengths
   // FP32 forms for the fast evaluation of the quantizer
   float A0f, A1f, muf, d1f, inv_A0f, inv_span1f, inv_log1pmuf;
   float slack0, slack1;  // per zone: an input width that covers the FP32 evaluation error
@@ -82,34 +71,13 @@ struct EncSeg {
   uint32_t pad;
 };
 
-// Alg. 1's state before the first symbol of a packing block.
-struct PackState {
-  uint64_t word;   // word of the stream being filled
-  uint32_t bits;   // bits used in it
-  uint32_t count;  // codewords in it
-};
-
 struct EncStatus {
   unsigned int flags;
   unsigned int pad;
   unsigned long long first_bad;
 };
 
-struct RefEnd {
-  uint32_t words;  // words the reference packing closes in the block (its last word stays open)
-  uint32_t bits;   // bits used in that open word
-  uint32_t count;  // its codewords
-  uint32_t bad;    // a level of the block has no codeword
-};
-
-// What Alg. 1 does over one packing block entered in a given state.
-struct BlockTrans {
-  int32_t adj;     // met: the words it closes are the reference's plus adj; else the words it closes
-  uint32_t bits;   // not met: the state it leaves the block in (bits of the open word
-  uint32_t count;  // and its codewords); met: the reference's end state
-  uint32_t flags;  // kTransMerged: it met the block's reference packing
-};
-constexpr uint32_t kTransMerged = 1u;
+struct PackRec;
 
 struct EncParams {
   const float *x;
@@ -121,15 +89,14 @@ struct EncParams {
   const EncDomain *doms;
   const double *cosv;
   const float *cosf;
-  const uint32_t *codes;
-  const uint8_t *lens;
-  PackState *blocks;
-  RefEnd *ref_end;       // per packing block: the reference packing's end state
-  BlockTrans *trans;     // per packing block: Alg. 1 over it from the state its predecessor's reference ends in
+  PackRec *recs;         // per packing block: its words and states
+  uint32_t *masks;       // per packing block: kMaskWords words, where words start in it
+  uint64_t *first_word;  // per packing block: the stream's words that start before it
   const uint32_t *block_seg;  // per packing block: its segment
-  const uint32_t *code_tab;   // per domain, 256 entries: codeword | length << 16
+  const uint32_t *code_tab;   // per domain, 256 entries: codeword << (32 - length) | length, 0: no codeword
   const uint32_t *lv_seg;     // k_enc_levels_w32: the segment of each warp's first window
   const long long *bound_keys;  // per domain: zone 0's, then zone 1's 255 level boundaries (order keys)
+  uint32_t n_doms;
   uint32_t *seg_bad;
   unsigned long long *fb_list;   // bins whose level the FP64 coefficient decides
   unsigned int *fb_count;
@@ -657,287 +624,438 @@ __global__ void __launch_bounds__(kLvThreads, 5) k_enc_levels_w32(EncParams p, u
   cp_async_wait_group<0>();
 }
 
-// ---- SymLen packing (Alg. 1) in parallel over blocks of kPackBlock symbols ----
-// Alg. 1 closes a word when the next codeword does not fit, so where words
-// start inside a block depends only on the state the block is entered with
-// (the bits already used in the open word).  Greedy packings entered with
-// different states soon start a word at the same symbol, and from there on
-// they coincide.  Call the packing of a block entered with a word that starts
-// at its first symbol the block's reference packing.  A block whose packing
-// meets its reference ends in the reference's end state, whatever state it
-// was entered with; so in the usual case every block but a stream's first is
-// entered in the state its predecessor's reference ends in.  k_enc_ref packs
-// block b as its reference does (the words it closes, the state it ends in),
-// then walks block b + 1 from that end state beside block b + 1's reference
-// until the two start a word at the same symbol: the transfer of block b + 1,
-// from the state it is entered in when block b met its reference.  k_enc_scan
-// adds the word counts up along each stream; a block whose predecessor never
-// met its reference (constant code lengths can do that) was entered in
-// another state, and the scan walks it again from the true one.
+// ---- SymLen packing (Alg. 1) in parallel ---------------------------------------
+// Alg. 1 starts a word at the first codeword that does not fit the open one,
+// so where words start in a run of symbols depends only on the bits u of the
+// open word that are used when the run is entered (1 .. 64; 64 also when no
+// word is open).  A codeword of c bits starts a word when u + c > 64, and u
+// becomes c, else u + c.  Held as s = u + kOff with kOff = 2^16 - 65 (or 2^32 -
+// 65), u + c > 64 is the carry out of s + c, so the step is
+// s = max(s + c, c + kOff) in modular arithmetic: one instruction, and one for
+// two packings at once in 16-bit halves.
+//
+// Where the first word of a run starts is the only thing its entry state
+// decides: at the symbol j whose codeword no longer fits, one of the (about
+// ten) symbols that begin in the run's first 64 bits.  So a run's effect on the
+// state is a small table: the run packed once for every such j, two packings
+// per instruction.  A run of kSub symbols per lane keeps the serial chain
+// short; the tables of 32 runs are put together step by step, again for every
+// first start at once (one per lane), which gives the table of the block of
+// kPackBlock symbols.  Packings of the same symbols from different states meet
+// sooner or later (on the trained codes the chance that two have not falls by
+// e every 900 symbols) and coincide from there on: the table of a block nearly
+// always gives one and the same state, which is then where the next block is
+// entered whatever came before.
+//   k_enc_starts  a warp per block: the tables, then, entered as the block
+//                 before it (of the same CTA, or packed along for this) says,
+//                 the word starts as a bitmap of the block's symbols.
+//   k_enc_scan    a warp per stream: the word starts added up block after
+//                 block; a block entered in another state than assumed is
+//                 walked again from the true one until the two packings meet.
+//   k_enc_pack    a warp per 2048 symbols, one lane per word: the word starts
+//                 give every word's symbols, so the words are put together
+//                 independently of one another and written once, consecutive
+//                 lanes to consecutive words.
+// All three are bound by instruction issue on large batches and by the length
+// of a run (256 symbols) on small ones.  With a block's packing done by one
+// thread twice (its reference, then the words) the chain was 16,384 symbols
+// and more: 43 M levels of a mixed batch took 1,112 us for the packing, now
+// 123 us (79 + 2 + 42); one stream of 32,768 levels 677 us, now 30 us.  Runs of
+// 2048 symbols by one thread without tables left 5 to 14 % of the blocks
+// unmet, and the scan that walked them took 380 us.
 
-// 16 levels from lv + i (zero past n) as one 16-byte vector.
-__device__ __forceinline__ uint4 load_raw16(const uint8_t *lv, uint64_t i, uint64_t n) {
-  if (i + 16 <= n && (reinterpret_cast<uintptr_t>(lv + i) & 15u) == 0) return *reinterpret_cast<const uint4 *>(lv + i);
+// What k_enc_starts leaves of a block.
+struct PackRec {
+  uint32_t starts;  // words that start in the block, entered as assumed
+  uint32_t u_in;    // the assumed state (64 at a stream's first block)
+  uint32_t u_out;   // the state it is left in then (not of a stream's last block)
+  uint32_t bad;     // a level of the block has no codeword
+};
+
+// A level's code length from the table of a domain (code << (32 - length) |
+// length per level, 0: no codeword); 64 for a level without one, which takes a
+// word of its own and shows in the OR of a block's lengths.
+__device__ __forceinline__ uint32_t entry_len(uint32_t e) { return e ? e & 31u : 64u; }
+
+// The code tables in shared memory (lengths in k_enc_starts, whole entries in
+// k_enc_pack), for encoders of at most kTabDomains domains; others read the
+// table in global memory.
+constexpr uint32_t kTabDomains = 16;
+
+// 16 levels from i (a multiple of 16, i < n) of the run of n at lv, zero past
+// n: one vector load where the run is 16-byte aligned, else aligned 4-byte
+// words put together (bytes at the run's ends, where a word would reach
+// outside it).
+__device__ __forceinline__ uint4 load_run16(const uint8_t *lv, uint32_t i, uint32_t n) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(lv + i);
+  if ((a & 15u) == 0 && i + 16 <= n) return __ldg(reinterpret_cast<const uint4 *>(a));
+  if (i != 0 && i + 20 <= n) {
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(a & ~uintptr_t(3));
+    const uint32_t s = (uint32_t)(a & 3u) * 8u;
+    const uint32_t w0 = __ldg(w), w1 = __ldg(w + 1), w2 = __ldg(w + 2), w3 = __ldg(w + 3), w4 = __ldg(w + 4);
+    return make_uint4(__funnelshift_r(w0, w1, s), __funnelshift_r(w1, w2, s), __funnelshift_r(w2, w3, s),
+                      __funnelshift_r(w3, w4, s));
+  }
   uint32_t t[4] = {0u, 0u, 0u, 0u};
-  for (uint32_t r = 0; r < 16 && i + r < n; ++r) t[r >> 2] |= (uint32_t)lv[i + r] << (8 * (r & 3));
+#pragma unroll
+  for (int r = 0; r < 16; ++r)
+    if (i + r < n) t[r >> 2] |= (uint32_t)__ldg(lv + i + r) << (8 * (r & 3));
   return make_uint4(t[0], t[1], t[2], t[3]);
 }
 
-// 64 levels from lv + i (zero past n) as four 16-byte vectors.
-__device__ __forceinline__ void load_raw64(const uint8_t *lv, uint64_t i, uint64_t n, uint4 (&v)[4]) {
+// fn(j, level) for the 16 levels of a vector.
+template <class F>
+__device__ __forceinline__ void each16(const uint4 &q, F fn) {
+  const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-  for (int q = 0; q < 4; ++q) v[q] = load_raw16(lv, i + 16 * q, n);
+  for (int j = 0; j < 16; ++j) fn(j, (w[j >> 2] >> (8 * (j & 3))) & 0xffu);
 }
 
-// Alg. 1 over 64 levels of the reference packing (FULL: all 64 exist).
-template <bool FULL>
-__device__ __forceinline__ void ref_step64(const uint4 (&v)[4], uint32_t i, uint32_t nb, const uint8_t *len,
-                                           uint32_t &words, uint32_t &bits, uint32_t &count, bool &bad) {
+constexpr uint32_t kSub = kPackBlock / 32;       // symbols of a lane's run
+constexpr uint32_t kOff16x2 = 0xFFBFFFBFu;       // 2^16 - 65 in both halves
+constexpr uint32_t kOff32 = 0xFFFFFFBFu;         // 2^32 - 65
+constexpr uint32_t kStartWarps = 8;              // blocks of a CTA of k_enc_starts; one more warp packs the block before
+constexpr uint32_t kExitPitch = 68;              // bytes per run: its exits by first start (64 at most), in separate banks
+constexpr uint32_t kSeqPitch = 33;               // bytes per first start: the states its 32 runs are entered in, exit
+constexpr uint32_t kStartWarpBytes = 32 * kExitPitch + 64 * kSeqPitch + 32 * 8;
+
+// The run packed from first starts base .. base + 2 R - 1 on (base a multiple
+// of 16, R <= 8): s[r] ends as the states of first starts base + 2 r and + 1.
+// c2: a level's code length in both halves.
+template <int R, class Len2>
+__device__ __forceinline__ void pack_run(const uint8_t *lv, uint32_t base, const Len2 &c2, uint32_t (&s)[R]) {
+#pragma unroll
+  for (int r = 0; r < R; ++r) s[r] = 0xFFFFFFFFu;  // a full word: the next symbol starts one
+  uint4 cur[4], nxt[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const uint32_t vw[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
-    uint32_t cl[16];
+    cur[q] = make_uint4(0u, 0u, 0u, 0u);
+    if (base + 16 * q < kSub) cur[q] = load_run16(lv, base + 16 * q, kSub);
+    nxt[q] = cur[q];
+  }
+  each16(cur[0], [&](int j, uint32_t level) {  // first start j begins at symbol base + j
+    const uint32_t c = c2(level), k = c + kOff16x2;
 #pragma unroll
-    for (int j = 0; j < 16; ++j) cl[j] = __ldg(len + ((vw[j >> 2] >> (8 * (j & 3))) & 0xffu));
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      if (!FULL && i + 16 * q + j >= nb) break;
-      const uint32_t c = cl[j];
-      bad = bad || c == 0u;
-      const bool start = count == 0u || bits + c > 64u;  // a word starts here
-      words += (start && count) ? 1u : 0u;
-      bits = (start ? 0u : bits) + c;
-      count = (start ? 0u : count) + 1u;
+    for (int r = 0; r < R; ++r) {
+      if (j >= 2 * r) s[r] = __viaddmax_u16x2(s[r], c, k);
+      if (j == 2 * r) s[r] |= 0xFFFF0000u;
     }
+  });
+  auto step = [&](const uint4 &v) {
+    each16(v, [&](int, uint32_t level) {
+      const uint32_t c = c2(level), k = c + kOff16x2;
+#pragma unroll
+      for (int r = 0; r < R; ++r) s[r] = __viaddmax_u16x2(s[r], c, k);
+    });
+  };
+#pragma unroll 1
+  for (uint32_t i = base; i < kSub; i += 64) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (i + 64 + 16 * q < kSub) nxt[q] = load_run16(lv, i + 64 + 16 * q, kSub);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if ((q || i != base) && i + 16 * q < kSub) step(cur[q]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) cur[q] = nxt[q];
   }
 }
 
-// One thread per packing block b: its reference packing, then the transfer
-// of block b + 1 (when it is in the same stream) entered in the state the
-// reference of b ends in.
-__global__ void __launch_bounds__(128) k_enc_ref(EncParams p) {
-  const uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= p.n_blocks) return;
-  const EncSeg sg = p.segs[p.block_seg[b]];
-  const EncDomain d = p.doms[sg.domain];
-  const uint64_t L = sg.n_windows * d.E;
-  const uint64_t i0 = (b - sg.block_base) * kPackBlock;
-  const uint32_t nb = (uint32_t)(L - i0 < kPackBlock ? L - i0 : kPackBlock);
-  const uint8_t *lv = p.levels + sg.level_offset + i0;
-  const uint8_t *len = p.lens + d.code_off;
-  uint32_t words = 0, bits = 0, count = 0;
-  bool bad = false;
-  // block b + 1 of the same stream, if any
-  const uint32_t nb2 = i0 + nb < L ? (uint32_t)(L - i0 - nb < kPackBlock ? L - i0 - nb : kPackBlock) : 0u;
-  // 64 levels per step, the next 64 in flight
-  uint4 v[4], vn[4];
-  load_raw64(lv, 0, nb, v);
-  for (uint32_t i = 0; i < nb; i += 64) {
-    if (i + 64 < nb) load_raw64(lv, i + 64, nb, vn);
-    if (i + 64 <= nb)
-      ref_step64<true>(v, i, nb, len, words, bits, count, bad);
-    else
-      ref_step64<false>(v, i, nb, len, words, bits, count, bad);
+// Exits of a run by first start into its row (bytes: the states' low bytes,
+// u - 65 mod 256), for the first starts base .. base + 2 R - 1.
+template <int R, class Len2>
+__device__ __forceinline__ void run_exits(const uint8_t *lv, uint32_t base, const Len2 &c2, uint8_t *row) {
+  uint32_t s[R];
+  pack_run<R>(lv, base, c2, s);
+  // byte 0 and byte 2 of two states
 #pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = vn[q];
+  for (int r = 0; r < R; r += 2)
+    *reinterpret_cast<uint32_t *>(row + base + 2 * r) = __byte_perm(s[r], r + 1 < R ? s[r + 1] : 0u, 0x6420);
+}
+
+// Index of the first start of a run entered with u bits used, from the
+// run's symbol boundaries in its first 63 bits (bit t - 1: one after t bits):
+// the symbols that fit the 64 - u bits left.
+__device__ __forceinline__ uint32_t first_start(uint64_t bounds, uint32_t u) {
+  return (uint32_t)__popcll(bounds & ((1ull << (64u - u)) - 1ull));
+}
+
+template <bool TAB>
+__global__ void __launch_bounds__((kStartWarps + 1) * 32, 3) k_enc_starts(EncParams p) {
+  extern __shared__ uint32_t starts_smem[];
+  // per block: what it is (bit 0: there is one, 1: its stream's first, 2: another follows it, 3: every first start
+  // gives one exit), the state it is entered in and which first start that is
+  __shared__ uint32_t what_s[kStartWarps + 1], in_s[kStartWarps + 1], cand_s[kStartWarps + 1];
+  const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+  uint32_t *const tab_s = starts_smem;  // TAB: [n_domains][256] code lengths, in both halves
+  uint8_t *const wbase = reinterpret_cast<uint8_t *>(starts_smem + (TAB ? p.n_doms * 256u : 0u)) + wid * kStartWarpBytes;
+  uint64_t *const bounds_s = reinterpret_cast<uint64_t *>(wbase);
+  uint8_t *const exits = wbase + 32 * 8;                         // [run][kExitPitch]
+  uint8_t *const seq = exits + 32 * kExitPitch;                  // [first start][kSeqPitch]
+  if (TAB) {
+    for (uint32_t i = threadIdx.x; i < p.n_doms * 256u; i += (kStartWarps + 1) * 32)
+      tab_s[i] = entry_len(__ldg(p.code_tab + i)) * 0x10001u;
+    __syncthreads();
   }
-  p.ref_end[b] = RefEnd{words, bits, count, bad ? 1u : 0u};
-  if (b == sg.block_base) p.trans[b] = BlockTrans{0, 0u, 0u, kTransMerged};  // a stream's first block packs as its reference
-  if (nb2 == 0) return;
-  // block b + 1: Alg. 1 from (bits, count) and from a fresh word side by side
-  const uint8_t *lv2 = lv + nb;
-  uint32_t rb = 0, rc = 0, closes = 0, r = 0;
-  bool met = false;
-  for (uint32_t i = 0; i < nb2 && !met; i += 16) {
-    const uint4 u = load_raw16(lv2, i, nb2);
-    const uint32_t vw[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      if (i + j >= nb2) break;
-      const uint32_t c = __ldg(len + ((vw[j >> 2] >> (8 * (j & 3))) & 0xffu));
-      const bool rs = rc == 0u || rb + c > 64u;  // the reference starts a word here
-      const bool ts = bits + c > 64u;            // so does the packing from (bits, count)
-      if (rs && ts) {
-        met = true;
-        break;
+  const uint64_t b = (uint64_t)blockIdx.x * kStartWarps + wid - 1;  // warp 0: the block before the CTA's (may wrap: none)
+  bool have = b < p.n_blocks;
+  const uint8_t *lv = p.levels;  // this lane's run
+  uint32_t dom = 0, nb = 0;
+  bool head = true, more = false;  // the stream's first block; it has another after it
+  if (have) {
+    const EncSeg &sg = p.segs[p.block_seg[b]];
+    const uint64_t i0 = (b - sg.block_base) * kPackBlock;
+    const uint64_t L = sg.n_windows * p.doms[sg.domain].E;
+    nb = (uint32_t)(L - i0 < kPackBlock ? L - i0 : kPackBlock);
+    lv = p.levels + sg.level_offset + i0 + lane * kSub;
+    dom = sg.domain;
+    head = i0 == 0;
+    more = i0 + nb < L;
+  }
+  uint32_t what = (have ? 1u : 0u) | (head ? 2u : 0u) | (more ? 4u : 0u);
+  if (wid == 0) have = have && more;  // only its exit is wanted
+  const uint32_t *const lt = tab_s + dom * 256u;
+  const uint32_t *const gt = p.code_tab + dom * 256u;
+  auto c2 = [&](uint32_t level) -> uint32_t { return TAB ? lt[level] : entry_len(__ldg(gt + level)) * 0x10001u; };
+  const uint32_t nsub = (nb + kSub - 1) / kSub;
+  uint32_t n_cand = 1;  // first starts of the block
+  if (have) {
+    // ---- the runs' tables.  A run needs one when another follows it (it is whole then)
+    const bool mine = (lane + 1 < nsub) || (lane + 1 == nsub && more);
+    uint32_t blo = 0, bhi = 0;
+    {
+      uint32_t sum = 0;
+#pragma unroll 1
+      for (uint32_t i = 0; i < 64; i += 16) {
+        if (!__any_sync(0xffffffffu, mine && sum < 64u)) break;
+        if (!mine) continue;
+        each16(load_run16(lv, i, kSub), [&](int, uint32_t level) {
+          sum += c2(level) & 0xffffu;
+          const uint32_t bit = 1u << ((sum - 1u) & 31u);
+          blo |= sum <= 32u ? bit : 0u;
+          bhi |= sum > 32u && sum <= 63u ? bit : 0u;
+        });
       }
-      r += rs ? 1u : 0u;
-      closes += ts ? 1u : 0u;
-      rb = (rs ? 0u : rb) + c;
-      rc = (rs ? 0u : rc) + 1u;
-      bits = (ts ? 0u : bits) + c;
-      count = (ts ? 0u : count) + 1u;
+    }
+    const uint64_t bounds = (uint64_t)bhi << 32 | blo;
+    bounds_s[lane] = bounds;
+    const uint32_t cands = mine ? (uint32_t)__popcll(bounds) + 1u : 0u;
+    const uint32_t most = __reduce_max_sync(0xffffffffu, cands);
+    uint8_t *const row = exits + lane * kExitPitch;
+#pragma unroll 1
+    for (uint32_t base = 0; base < most; base += 16) {
+      if (!mine) continue;
+      // as many packings as the warp's runs want (the instance is the warp's)
+      if (most - base > 12)
+        run_exits<8>(lv, base, c2, row);
+      else if (most - base > 8)
+        run_exits<6>(lv, base, c2, row);
+      else
+        run_exits<4>(lv, base, c2, row);
+    }
+    __syncwarp();
+    // ---- the block's: lane = first start, run after run
+    n_cand = (uint32_t)__popcll(bounds_s[0]) + 1u;
+    const uint32_t steps = more ? nsub : (nsub ? nsub - 1u : 0u);  // runs that are left for another
+    uint32_t same = 1u, last = 0u;
+    for (uint32_t j0 = 0; j0 < n_cand; j0 += 32) {
+      const uint32_t j = j0 + lane;
+      uint32_t u = 0;
+      if (j < n_cand) {
+        uint32_t at = j;
+#pragma unroll 1
+        for (uint32_t k = 0; k < steps; ++k) {
+          u = ((uint32_t)exits[k * kExitPitch + at] + 65u) & 0xffu;
+          seq[j * kSeqPitch + k + 1] = (uint8_t)u;
+          at = k + 1 < 32u ? first_start(bounds_s[k + 1], u) : 0u;
+        }
+      }
+      const uint32_t u0 = __shfl_sync(0xffffffffu, u, 0);
+      same &= __all_sync(0xffffffffu, j >= n_cand || u == u0) ? 1u : 0u;
+      if (j0) same &= u0 == last ? 1u : 0u;
+      last = u0;
+    }
+    what |= same << 3;
+  }
+  if (lane == 0) what_s[wid] = what;
+  __syncthreads();
+  // ---- the states the CTA's blocks are entered in
+  if (threadIdx.x == 0) {
+    uint32_t u = 64u;
+    for (uint32_t w = 0; w <= kStartWarps; ++w) {
+      const uint32_t f = what_s[w];
+      if (!(f & 1u)) continue;
+      const uint8_t *wb = wbase + w * kStartWarpBytes;  // thread 0 is of warp 0
+      if (f & 2u) u = 64u;
+      in_s[w] = u;
+      // warp 0's block stands for itself when its stream starts there or every first
+      // start gives one exit; else 64 is assumed, and k_enc_scan sees whether that is so
+      const uint32_t cand = w == 0 ? 0u : first_start(*reinterpret_cast<const uint64_t *>(wb), u);
+      cand_s[w] = cand;
+      if (f & 4u)
+        u = w == 0 && (f & 10u) == 0 ? 64u : (uint32_t)wb[32 * 8 + 32 * kExitPitch + cand * kSeqPitch + 32];
     }
   }
-  // met: the word open before the meeting symbol closes there, then come the
-  // reference's words but the r that start before it
-  p.trans[b + 1] = met ? BlockTrans{(int32_t)(closes + 1u) - (int32_t)r, 0u, 0u, kTransMerged}
-                       : BlockTrans{(int32_t)closes, bits, count, 0u};
+  __syncthreads();
+  if (wid == 0 || !have) return;
+  // ---- the word starts, each lane those of its run
+  uint32_t seen = 0, cnt = 0;
+  const uint32_t n = lane * kSub < nb ? (nb - lane * kSub < kSub ? nb - lane * kSub : kSub) : 0u;
+  const uint32_t u_in = in_s[wid];
+  uint32_t *const row = p.masks + b * kMaskWords + lane * (kSub / 32);
+  if (n) {
+    const uint32_t cand = cand_s[wid];
+    uint32_t s = (lane ? (uint32_t)seq[cand * kSeqPitch + lane] : u_in) + kOff32;
+    uint32_t m[kSub / 32];
+#pragma unroll
+    for (uint32_t q = 0; q < kSub / 32; ++q) m[q] = 0u;
+    uint4 cur[2], nxt[2];
+    cur[0] = load_run16(lv, 0, n);
+    cur[1] = 16u < n ? load_run16(lv, 16, n) : make_uint4(0u, 0u, 0u, 0u);
+    nxt[0] = nxt[1] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (uint32_t q = 0; q < kSub / 32; ++q) {
+      const uint32_t i = 32 * q;
+      if (i + 32 < n) nxt[0] = load_run16(lv, i + 32, n);
+      if (i + 48 < n) nxt[1] = load_run16(lv, i + 48, n);
+      if (i + 32 <= n) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          each16(cur[h], [&](int j, uint32_t level) {
+            const uint32_t c = c2(level) & 0xffffu, k = c + kOff32;
+            seen |= c;
+            s = __viaddmax_u32(s, c, k);
+            if (s == k) m[q] |= 1u << (16 * h + j);
+          });
+      } else if (i < n) {
+#pragma unroll 1
+        for (uint32_t j = 0; i + j < n; ++j) {
+          const uint32_t c = c2((uint32_t)__ldg(lv + i + j)) & 0xffffu, k = c + kOff32;
+          seen |= c;
+          s = __viaddmax_u32(s, c, k);
+          if (s == k) m[q] |= 1u << j;
+        }
+      }
+      cnt += __popc(m[q]);
+      cur[0] = nxt[0];
+      cur[1] = nxt[1];
+    }
+    static_assert(kSub == 256, "a run's bitmap is two 16-byte vectors");
+    reinterpret_cast<uint4 *>(row)[0] = make_uint4(m[0], m[1], m[2], m[3]);
+    reinterpret_cast<uint4 *>(row)[1] = make_uint4(m[4], m[5], m[6], m[7]);
+  }
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  seen = __reduce_or_sync(0xffffffffu, seen);
+  if (lane == 0)
+    p.recs[b] = PackRec{cnt, u_in, more ? (uint32_t)seq[cand_s[wid] * kSeqPitch + 32] : 64u, seen >> 6};
 }
 
-// Word starts of Alg. 1 among symbols from .. valid - 1 of a chunk of 32
-// (S: inclusive prefix of the chunk's code lengths, per lane), entered in
-// (bits, count); a word that starts at the chunk's first symbol because none
-// is open (count == 0) is one too.  One ballot per word start; the state is
-// carried over.
-__device__ __forceinline__ uint32_t chunk_starts(uint32_t S, uint32_t lane, uint32_t valid, uint32_t &bits,
-                                                 uint32_t &count) {
-  uint32_t mask = count == 0u ? 1u : 0u;
-  uint32_t from = 0;
+// Word starts of Alg. 1 among the first `valid` symbols of a chunk of 32 (S:
+// inclusive prefix of the chunk's code lengths, per lane), entered with v bits
+// left, which moves on.  One ballot per word start.
+__device__ __forceinline__ uint32_t chunk_starts(uint32_t S, uint32_t lane, uint32_t valid, uint32_t &v) {
+  uint32_t mask = 0, from = 0, pre = 0;
   while (true) {
-    const uint32_t pre = from ? __shfl_sync(0xffffffffu, S, from - 1) : 0u;
-    const uint32_t over = __ballot_sync(0xffffffffu, lane >= from && lane < valid && bits + (S - pre) > 64u);
+    const uint32_t over = __ballot_sync(0xffffffffu, lane >= from && lane < valid && S - pre > v);
     if (over == 0) {  // the rest of the chunk fits the open word
-      bits += __shfl_sync(0xffffffffu, S, valid - 1) - pre;
-      count += valid - from;
+      v -= __shfl_sync(0xffffffffu, S, valid - 1) - pre;
       return mask;
     }
     from = (uint32_t)(__ffs(over) - 1);  // a word starts at symbol from
     mask |= 1u << from;
-    bits = 0;
-    count = 0;
+    pre = from ? __shfl_sync(0xffffffffu, S, from - 1) : 0u;
+    v = 64u;
   }
 }
 
-// The transfer of block b entered in (bits, count > 0), by the whole warp:
-// Alg. 1 from that state and the block's reference side by side, 32 symbols
-// at a time (a warp scan of their code lengths; each word start one ballot),
-// until both start a word at the same symbol.  Levels arrive 128 per round
-// trip (a 4-byte load per lane), the next 128 in flight.
-__device__ BlockTrans walk_block(const EncParams &p, const EncSeg &sg, const EncDomain &d, uint64_t b, uint32_t bits,
-                                 uint32_t count, uint32_t lane) {
+// Block b again, entered with u bits used, by the whole warp, 32 symbols at a
+// time, until a start of its bitmap is met (its starts before that one are
+// replaced): the words that start in it and the state it is left in.
+__device__ void walk_block(const EncParams &p, const EncSeg &sg, const EncDomain &d, uint64_t b, uint32_t &u,
+                           uint32_t &starts, uint32_t u_out, uint32_t lane) {
   const uint64_t L = sg.n_windows * d.E;
   const uint64_t i0 = (b - sg.block_base) * kPackBlock;
   const uint32_t nb = (uint32_t)(L - i0 < kPackBlock ? L - i0 : kPackBlock);
   const uint8_t *lv = p.levels + sg.level_offset + i0;
-  const uint8_t *len = p.lens + d.code_off;
-  uint32_t rb = 0, rc = 0, closes = 0, r = 0;
-  auto fetch = [&](uint32_t at) -> uint32_t {  // levels at .. at + 127, four per lane
-    const uint32_t o = at + 4 * lane;
-    if (o + 4 <= nb && (reinterpret_cast<uintptr_t>(lv + o) & 3u) == 0) return *reinterpret_cast<const uint32_t *>(lv + o);
-    uint32_t t = 0;
-    for (uint32_t q = 0; q < 4 && o + q < nb; ++q) t |= (uint32_t)lv[o + q] << (8 * q);
-    return t;
-  };
-  uint32_t cur = fetch(0);
-  for (uint32_t at = 0; at < nb; at += 128) {
-    const uint32_t nxt = at + 128 < nb ? fetch(at + 128) : 0u;
-#pragma unroll 1
-    for (uint32_t k = 0; k < 4; ++k) {
-      const uint32_t c = at + 32 * k;
-      if (c >= nb) break;
-      const uint32_t valid = nb - c < 32 ? nb - c : 32;
-      const uint32_t vw = __shfl_sync(0xffffffffu, cur, 8 * k + (lane >> 2));
-      const uint32_t cl = lane < valid ? __ldg(len + ((vw >> (8 * (lane & 3))) & 0xffu)) : 0u;
-      const uint32_t S = lane_prefix(cl, lane);
-      const uint32_t rm = chunk_starts(S, lane, valid, rb, rc);
-      const uint32_t tm = chunk_starts(S, lane, valid, bits, count);
-      const uint32_t both = rm & tm;
-      if (both) {  // they meet at symbol c + t
-        const uint32_t before = (1u << (__ffs(both) - 1)) - 1u;
-        closes += __popc(tm & before);
-        r += __popc(rm & before);
-        return BlockTrans{(int32_t)(closes + 1u) - (int32_t)r, 0u, 0u, kTransMerged};
-      }
-      closes += __popc(tm);
-      r += __popc(rm);
+  const uint32_t *tab = p.code_tab + sg.domain * 256u;
+  uint32_t *row = p.masks + b * kMaskWords;
+  auto fetch = [&](uint32_t at) -> uint32_t { return at + lane < nb ? (uint32_t)__ldg(lv + at + lane) : 0u; };
+  uint32_t cur = fetch(0), v = 64u - u;
+  for (uint32_t at = 0; at < nb; at += 32) {
+    const uint32_t nxt = fetch(at + 32);
+    const uint32_t valid = nb - at < 32 ? nb - at : 32;
+    const uint32_t S = lane_prefix(lane < valid ? entry_len(__ldg(tab + cur)) : 0u, lane);
+    const uint32_t r = row[at >> 5];
+    __syncwarp();
+    const uint32_t t = chunk_starts(S, lane, valid, v);
+    const uint32_t both = t & r;
+    const uint32_t below = both ? (both & (0u - both)) - 1u : 0xffffffffu;
+    starts += __popc(t & below) - __popc(r & below);
+    if (lane == 0) row[at >> 5] = (t & below) | (r & ~below);
+    if (both) {
+      u = u_out;
+      return;
     }
     cur = nxt;
   }
-  return BlockTrans{(int32_t)closes, bits, count, 0u};
+  u = 64u - v;
 }
 
-// One warp per stream: the true packing state block after block from the
-// blocks' transfers, 32 blocks at a time (a warp scan of their word counts);
-// each block's entry state for k_enc_pack; the words two blocks share are
-// zeroed for the blocks' atomicOr; code and room checks; the stream's word
-// count.  A block entered in another state than its transfer assumed (its
-// predecessor never met its reference) is walked again from the true state.
+// One warp per stream: the words before each block from the blocks' records,
+// 32 blocks at a time (a warp scan), the next 32 records in flight; a block
+// entered in another state than assumed is walked again from the true one;
+// code and room checks; the stream's word count.
 __global__ void __launch_bounds__(128) k_enc_scan(EncParams p) {
   const uint64_t s = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint32_t lane = threadIdx.x & 31u;
   if (s >= p.n_segs) return;  // the whole warp
   const EncSeg sg = p.segs[s];
-  const EncDomain d = p.doms[sg.domain];
+  const EncDomain &d = p.doms[sg.domain];
   const uint64_t L = sg.n_windows * d.E;
   const uint64_t nblk = (L + kPackBlock - 1) / kPackBlock;
-  uint64_t w = 0;  // the open word (words closed so far)
-  uint32_t bits = 0, count = 0;
-  bool assumed = true;  // the next block is entered in the state its transfer assumed
+  uint64_t w = 0;  // words that start before the group
   bool bad = false;
-  uint64_t jb = 0;
-  while (jb < nblk) {
+  auto fetch = [&](uint64_t jb) -> PackRec {
+    return jb + lane < nblk ? p.recs[sg.block_base + jb + lane] : PackRec{0u, 0u, 0u, 0u};
+  };
+  uint32_t u_prev = 64u;  // the state the block before the group is left in
+  PackRec rec = fetch(0);
+  for (uint64_t jb = 0; jb < nblk; jb += 32) {
+    const PackRec nxt = fetch(jb + 32);
     const uint64_t b0 = sg.block_base + jb;
-    if (!assumed) {
-      if (lane == 0) {
-        p.blocks[b0] = PackState{w, bits, count};
-        if (bits > 0 && w < sg.room) p.words[sg.word_offset + w] = 0;  // shared with the previous block
-      }
-      const RefEnd re = p.ref_end[b0];
-      if (re.bad) {
-        bad = true;
-        break;
-      }
-      const BlockTrans t = walk_block(p, sg, d, b0, bits, count, lane);
-      const bool met = (t.flags & kTransMerged) != 0;
-      w += (uint64_t)((int64_t)t.adj + (met ? (int64_t)re.words : 0));
-      bits = met ? re.bits : t.bits;
-      count = met ? re.count : t.count;
-      assumed = met;
-      ++jb;
-      continue;
-    }
     const uint32_t n = nblk - jb < 32 ? (uint32_t)(nblk - jb) : 32u;
-    BlockTrans t{0, 0u, 0u, 0u};
-    RefEnd re{0u, 0u, 0u, 0u};
-    if (lane < n) {
-      t = p.trans[b0 + lane];
-      re = p.ref_end[b0 + lane];
+    bad = __any_sync(0xffffffffu, rec.bad != 0u);
+    if (bad) break;
+    while (true) {  // the first block entered in another state than assumed, until there is none
+      uint32_t u = __shfl_up_sync(0xffffffffu, rec.u_out, 1);
+      if (lane == 0) u = u_prev;
+      const uint32_t off = __ballot_sync(0xffffffffu, lane < n && u != rec.u_in);
+      if (!off) break;
+      const uint32_t at = (uint32_t)(__ffs(off) - 1);
+      uint32_t ua = __shfl_sync(0xffffffffu, u, at), st = __shfl_sync(0xffffffffu, rec.starts, at);
+      const uint32_t uo = __shfl_sync(0xffffffffu, rec.u_out, at);
+      if (lane == at) rec.u_in = ua;
+      walk_block(p, sg, d, b0 + at, ua, st, uo, lane);
+      if (lane == at) {
+        rec.starts = st;
+        rec.u_out = ua;
+      }
     }
-    const bool met = (t.flags & kTransMerged) != 0;
-    const uint32_t delta = (uint32_t)(t.adj + (met ? (int32_t)re.words : 0));
-    const uint32_t xb = met ? re.bits : t.bits, xc = met ? re.count : t.count;  // the state it leaves
-    const uint32_t badm = __ballot_sync(0xffffffffu, lane < n && re.bad);
-    const uint32_t open = __ballot_sync(0xffffffffu, lane < n && !met);
-    // the blocks entered as assumed: up to the first that did not meet its
-    // reference (it is itself one), before the first bad one
-    uint32_t m = n;
-    if (open) m = min(m, (uint32_t)__ffs(open));
-    const uint32_t first_bad = badm ? (uint32_t)(__ffs(badm) - 1) : 32u;
-    m = min(m, first_bad);
-    uint32_t eb = __shfl_up_sync(0xffffffffu, xb, 1), ec = __shfl_up_sync(0xffffffffu, xc, 1);
-    if (lane == 0) {
-      eb = bits;
-      ec = count;
-    }
-    const uint32_t dl = lane < m ? delta : 0u;
-    const uint32_t incl = lane_prefix(dl, lane);
-    const uint64_t we = w + (incl - dl);
-    if (lane < m) {
-      p.blocks[b0 + lane] = PackState{we, eb, ec};
-      if (eb > 0 && we < sg.room) p.words[sg.word_offset + we] = 0;  // shared with the previous block
-    }
-    if (m > 0) {
-      w += __shfl_sync(0xffffffffu, incl, m - 1);
-      bits = __shfl_sync(0xffffffffu, xb, m - 1);
-      count = __shfl_sync(0xffffffffu, xc, m - 1);
-      assumed = ((open >> (m - 1)) & 1u) == 0u;
-    }
-    jb += m;
-    if (badm && m == first_bad) {
-      bad = true;
-      break;
-    }
+    const uint32_t add = lane < n ? rec.starts : 0u;
+    const uint32_t incl = lane_prefix(add, lane);
+    if (lane < n) p.first_word[b0 + lane] = w + (incl - add);
+    w += __shfl_sync(0xffffffffu, incl, 31);
+    u_prev = __shfl_sync(0xffffffffu, rec.u_out, n - 1);
+    rec = nxt;
   }
   if (lane == 0) {
     if (bad) enc_flag(p.status, FPTC_ENC_FLAG_NO_CODE, s);
-    const uint64_t total = w + (count > 0 ? 1u : 0u);
-    if (!bad && total > sg.room) {
+    if (!bad && w > sg.room) {
       enc_flag(p.status, FPTC_ENC_FLAG_ROOM, s);
       bad = true;
     }
     p.seg_bad[s] = bad ? 1u : 0u;
-    p.n_words[s] = bad ? 0u : total;
+    p.n_words[s] = bad ? 0u : w;
   }
 }
 
@@ -1002,132 +1120,117 @@ __global__ void __launch_bounds__(256) k_enc_fallback(EncParams p) {
   }
 }
 
-// k_enc_pack: one thread per packing block, Alg. 1 from the block's entry
-// state, branch-free per codeword (one table load gives code and length).  A
-// word that closes is staged in shared memory; after every 64 codewords the
-// warp writes its lanes' staged words out together, two lanes' words per
-// round (16 lanes each), so that a store instruction writes one lane's
-// consecutive words instead of one word of each of 32 streams.  The first
-// word of a block entered with bits already used is shared with the previous
-// block and goes out with a 64-bit atomicOr (the two parts' bits are
-// disjoint; the scan zeroed it), as does the word a block leaves open for the
-// next.  Each word's symbol count is written by the block that closes it.
-constexpr uint32_t kStageWords = 16;  // words that can close in 64 codewords (>= 4 codewords each: lmax <= 16)
-constexpr uint32_t kStagePitch = 17;  // per lane, padded against bank conflicts
+// k_enc_pack: one warp per part of a block.  The part's levels (and the 64 after
+// it, which its last word may reach into) come into shared memory; the lanes turn
+// two words of the start bitmap each into a list of starts; then one lane per
+// word: its codewords shifted into 64 bits one after the other (a table entry
+// holds the code left-aligned above its length, so a funnel shift by the entry
+// appends it), five operations a codeword beside the loop.  A word belongs to
+// the part it starts in.
 constexpr uint32_t kPackWarps = 4;
+constexpr uint32_t kPackPart = 2048;                       // symbols of a part
+constexpr uint32_t kPartWords = kPackPart / 32;            // words of its bitmap (two a lane)
+constexpr uint32_t kPackSpan = kPackPart + 64;             // symbols a part's words may hold
+constexpr uint32_t kPackStage = (kPackSpan + 16 + 15) / 16 * 16;
+constexpr uint32_t kPackList = kPackPart / 4 + 2;          // starts of a part (a word holds at least four codewords) + end
 
-struct PackLane {
-  const uint8_t *lv = nullptr;    // the block's levels
-  const uint32_t *tab = nullptr;  // code | length << 16 per level
-  uint64_t g0 = 0;                // index in p.words of the block's first word
-  uint32_t n = 0;                 // codewords of the block (0: no work)
-  uint32_t bits = 0, count = 0;   // Alg. 1's state
-  uint32_t wf = 0, ns = 0;        // words of the block written out; staged
-  uint64_t buffer = 0;            // the open word's codewords, left-aligned
-  bool shared_first = false;      // the block's first word holds bits of the previous block
-};
-
-template <bool FULL>
-__device__ __forceinline__ void pack_step64(PackLane &t, const uint4 (&v)[4], uint32_t i, unsigned long long *sw,
-                                            uint8_t *sc) {
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const uint32_t vw[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      if (!FULL && i + 16 * q + j >= t.n) break;
-      const uint32_t e = __ldg(t.tab + ((vw[j >> 2] >> (8 * (j & 3))) & 0xffu));
-      const uint32_t cl = e >> 16;
-      const bool close = t.bits + cl > 64u;
-      if (close) {
-        sw[t.ns] = t.buffer;
-        sc[t.ns] = (uint8_t)t.count;
-      }
-      t.ns += close ? 1u : 0u;
-      t.bits = (close ? 0u : t.bits) + cl;
-      t.count = (close ? 0u : t.count) + 1u;
-      t.buffer = (close ? 0ull : t.buffer) | ((uint64_t)(e & 0xffffu) << (64u - t.bits));
-    }
-  }
-}
-
+template <bool TAB>
 __global__ void __launch_bounds__(kPackWarps * 32) k_enc_pack(EncParams p) {
-  __shared__ unsigned long long stage_w[kPackWarps][32 * kStagePitch];
-  __shared__ uint8_t stage_c[kPackWarps][32 * kStageWords];
-  __shared__ uint4 stage_i[kPackWarps][32];  // per lane: first staged word (index in p.words), count, shared flag
+  extern __shared__ uint32_t code_s[];  // TAB: [n_domains][256] table entries
+  __shared__ __align__(16) uint8_t stage_s[kPackWarps][kPackStage];
+  __shared__ uint16_t list_s[kPackWarps][kPackList];
+  if (TAB) {
+    for (uint32_t i = threadIdx.x; i < p.n_doms * 256u; i += kPackWarps * 32) code_s[i] = __ldg(p.code_tab + i);
+    __syncthreads();
+  }
   const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
-  unsigned long long *const sw = stage_w[wid] + lane * kStagePitch;
-  uint8_t *const sc = stage_c[wid] + lane * kStageWords;
-  const uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  PackLane t;
-  bool last = false;  // the block ends its stream
-  if (b < p.n_blocks) {
-    const uint32_t s = p.block_seg[b];
-    if (!p.seg_bad[s]) {
-      const EncSeg sg = p.segs[s];
-      const EncDomain d = p.doms[sg.domain];
-      const uint64_t L = sg.n_windows * d.E;
-      const uint64_t i0 = (b - sg.block_base) * kPackBlock;
-      t.n = (uint32_t)(L - i0 < kPackBlock ? L - i0 : kPackBlock);
-      t.lv = p.levels + sg.level_offset + i0;
-      t.tab = p.code_tab + d.code_off;
-      const PackState st = p.blocks[b];
-      t.g0 = sg.word_offset + st.word;
-      t.bits = st.bits;
-      t.count = st.count;
-      t.shared_first = st.bits > 0;
-      last = i0 + t.n == L;
-    }
-  }
-  const uint32_t nmax = __reduce_max_sync(0xffffffffu, t.n);
-  uint4 v[4], vn[4];
-  if (t.n) load_raw64(t.lv, 0, t.n, v);
-  for (uint32_t i = 0; i < nmax; i += 64) {
-    if (i < t.n) {
-      if (i + 64 < t.n) load_raw64(t.lv, i + 64, t.n, vn);
-      if (i + 64 <= t.n)
-        pack_step64<true>(t, v, i, sw, sc);
-      else
-        pack_step64<false>(t, v, i, sw, sc);
+  const uint64_t item = (uint64_t)blockIdx.x * kPackWarps + wid, b = item / (kPackBlock / kPackPart);
+  const uint32_t part = (uint32_t)(item % (kPackBlock / kPackPart));
+  if (b >= p.n_blocks) return;  // the whole warp
+  const uint32_t s = p.block_seg[b];
+  if (p.seg_bad[s]) return;
+  const EncSeg &sg = p.segs[s];
+  const uint64_t L = sg.n_windows * p.doms[sg.domain].E;
+  const uint64_t i0 = (b - sg.block_base) * kPackBlock + part * kPackPart;
+  if (i0 >= L) return;
+  const uint32_t nb = (uint32_t)(L - i0 < kPackPart ? L - i0 : kPackPart);
+  const uint32_t span = (uint32_t)(L - i0 < kPackSpan ? L - i0 : kPackSpan);
+  const uint8_t *const lv = p.levels + sg.level_offset;  // the stream's levels
+  uint8_t *const stage = stage_s[wid];
+  uint16_t *const list = list_s[wid];
+  // levels: 16-byte pieces from the aligned address at or before the block's first
+  const uintptr_t a0 = reinterpret_cast<uintptr_t>(lv + i0);
+  const uint32_t sh = (uint32_t)(a0 & 15u);
+  const uintptr_t lo = reinterpret_cast<uintptr_t>(lv), hi = lo + L;
+  for (uint32_t c = lane * 16u; c < sh + span; c += 512u) {
+    const uintptr_t a = a0 - sh + c;
+    uint4 q = make_uint4(0u, 0u, 0u, 0u);
+    if (a >= lo && a + 16 <= hi) {
+      q = __ldg(reinterpret_cast<const uint4 *>(a));
+    } else {  // the stream's ends: nothing outside it is read
+      uint32_t t[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-      for (int q = 0; q < 4; ++q) v[q] = vn[q];
+      for (int r = 0; r < 16; ++r)
+        if (a + r >= lo && a + r < hi) t[r >> 2] |= (uint32_t)__ldg(reinterpret_cast<const uint8_t *>(a + r)) << (8 * (r & 3));
+      q = make_uint4(t[0], t[1], t[2], t[3]);
     }
-    // the warp writes its staged words: round r, half h writes lane 2 r + h's
-    stage_i[wid][lane] = make_uint4((uint32_t)(t.g0 + t.wf), (uint32_t)((t.g0 + t.wf) >> 32), t.ns,
-                                    t.shared_first && t.wf == 0u ? 1u : 0u);
-    __syncwarp();
-    const uint32_t h = lane >> 4, j = lane & 15u;
-#pragma unroll 4
-    for (uint32_t r = 0; r < 16; ++r) {
-      const uint32_t src = 2u * r + h;
-      const uint4 si = stage_i[wid][src];
-      if (j < si.z) {
-        const uint64_t g = ((uint64_t)si.y << 32 | si.x) + j;
-        const unsigned long long wv = stage_w[wid][src * kStagePitch + j];
-        if (j == 0 && si.w)
-          atomicOr(reinterpret_cast<unsigned long long *>(p.words) + g, wv);
-        else
-          p.words[g] = wv;
-        p.symlen[g] = stage_c[wid][src * kStageWords + j];
-      }
-    }
-    __syncwarp();
-    t.wf += t.ns;
-    t.ns = 0;
+    *reinterpret_cast<uint4 *>(stage + c) = q;
   }
-  if (t.n) {
-    unsigned long long *const wp = reinterpret_cast<unsigned long long *>(p.words) + t.g0 + t.wf;
-    if (last) {  // the stream's last word
-      if (t.count > 0) {
-        if (t.wf == 0 && t.shared_first)
-          atomicOr(wp, (unsigned long long)t.buffer);
-        else
-          *wp = t.buffer;
-        p.symlen[t.g0 + t.wf] = (uint8_t)t.count;
-      }
-    } else {  // the open word continues in the next block (zeroed by the scan)
-      atomicOr(wp, (unsigned long long)t.buffer);
+  // starts
+  const uint32_t *const row = p.masks + b * kMaskWords + part * kPartWords;
+  const uint2 m = *(reinterpret_cast<const uint2 *>(row) + lane);
+  uint32_t before = 0;  // words that start in the block's parts before this one
+  for (uint32_t q = 1; q <= part; ++q) {
+    const uint2 x = *(reinterpret_cast<const uint2 *>(row - q * kPartWords) + lane);
+    before += __popc(x.x) + __popc(x.y);
+  }
+  before = __reduce_add_sync(0xffffffffu, before);
+  // a row's words past the stream's symbols are not written by k_enc_starts
+  uint32_t m0 = 64u * lane < nb ? m.x : 0u, m1 = 64u * lane + 32u < nb ? m.y : 0u;
+  const uint32_t cnt = __popc(m0) + __popc(m1);
+  const uint32_t incl = lane_prefix(cnt, lane);
+  const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+  uint32_t o = incl - cnt;
+  for (; m0; m0 &= m0 - 1u) list[o++] = (uint16_t)(64u * lane + (uint32_t)(__ffs(m0) - 1));
+  for (; m1; m1 &= m1 - 1u) list[o++] = (uint16_t)(64u * lane + 32u + (uint32_t)(__ffs(m1) - 1));
+  if (lane == 0) {
+    // the last word ends at the next part's first start (among its first 64
+    // symbols), or with the stream
+    uint32_t end = span;
+    if (i0 + nb < L) {
+      const uint32_t *nx = row + kPartWords;  // the next part's row, in this block or the next
+      const uint32_t rest = (uint32_t)(L - i0 - nb < 64 ? L - i0 - nb : 64);
+      const uint32_t n0 = nx[0], n1 = rest > 32u ? nx[1] : 0u;
+      if (n0)
+        end = nb + (uint32_t)(__ffs(n0) - 1);
+      else if (n1)
+        end = nb + 32u + (uint32_t)(__ffs(n1) - 1);
     }
+    list[total] = (uint16_t)end;
+  }
+  __syncwarp();
+  const uint64_t g0 = sg.word_offset + p.first_word[b] + before;
+  const uint32_t *const tab = TAB ? code_s + sg.domain * 256u : p.code_tab + sg.domain * 256u;
+  for (uint32_t j = lane; j < total; j += 32) {
+    const uint32_t from = list[j], n = list[j + 1] - from;
+    const uint8_t *src = stage + sh + from;
+    uint32_t h = 0, l = 0, used = 0;
+    auto add = [&](uint32_t level) {
+      const uint32_t e = TAB ? tab[level] : __ldg(tab + level);
+      h = __funnelshift_l(l, h, e);
+      l = __funnelshift_l(e, l, e);
+      used += e;  // the lengths add up in the low 16 bits (codes lie above them)
+    };
+    uint32_t i = 0;
+    for (; i + 4 <= n; i += 4) {
+      add(src[i]);
+      add(src[i + 1]);
+      add(src[i + 2]);
+      add(src[i + 3]);
+    }
+    for (; i < n; ++i) add(src[i]);
+    p.words[g0 + j] = ((uint64_t)h << 32 | l) << (64u - (used & 0xffffu));
+    p.symlen[g0 + j] = (uint8_t)n;
   }
 }
 
@@ -1161,9 +1264,9 @@ struct fptc_encoder {
   EncDomain *d_doms = nullptr;
   double *d_cos = nullptr;
   float *d_cosf = nullptr;
-  PackState *d_blocks = nullptr;
-  RefEnd *d_ref_end = nullptr;              // [n_blocks]
-  BlockTrans *d_trans = nullptr;            // [n_blocks]
+  PackRec *d_recs = nullptr;                // [n_blocks]
+  uint32_t *d_masks = nullptr;              // [n_blocks][kMaskWords]
+  uint64_t *d_first_word = nullptr;         // [n_blocks]
   uint32_t *d_block_seg = nullptr;          // [n_blocks]
   uint32_t *d_code_tab = nullptr;           // [n_domains][256]
   uint32_t *d_lv_seg = nullptr;             // [warps of k_enc_levels_w32]
@@ -1175,8 +1278,7 @@ struct fptc_encoder {
   uint32_t fb_cap = 0;
   uint64_t n_blocks = 0;
   int sm_count = 1;
-  uint32_t *d_codes = nullptr;
-  uint8_t *d_lens = nullptr;
+  uint32_t n_doms = 0;
   EncStatus *d_status = nullptr;
   uint8_t *d_lev_scratch = nullptr;
 };
@@ -1188,9 +1290,9 @@ void enc_free(fptc_encoder *e) {
   cudaFree(e->d_doms);
   cudaFree(e->d_cos);
   cudaFree(e->d_cosf);
-  cudaFree(e->d_blocks);
-  cudaFree(e->d_ref_end);
-  cudaFree(e->d_trans);
+  cudaFree(e->d_recs);
+  cudaFree(e->d_masks);
+  cudaFree(e->d_first_word);
   cudaFree(e->d_block_seg);
   cudaFree(e->d_code_tab);
   cudaFree(e->d_lv_seg);
@@ -1198,8 +1300,6 @@ void enc_free(fptc_encoder *e) {
   cudaFree(e->d_seg_bad);
   cudaFree(e->d_fb_list);
   cudaFree(e->d_fb_count);
-  cudaFree(e->d_codes);
-  cudaFree(e->d_lens);
   cudaFree(e->d_status);
   cudaFree(e->d_lev_scratch);
 }
@@ -1229,9 +1329,10 @@ EncParams enc_params(const fptc_encoder *e, uint64_t *d_words, uint8_t *d_symlen
   p.doms = e->d_doms;
   p.cosv = e->d_cos;
   p.cosf = e->d_cosf;
-  p.blocks = e->d_blocks;
-  p.ref_end = e->d_ref_end;
-  p.trans = e->d_trans;
+  p.recs = e->d_recs;
+  p.masks = e->d_masks;
+  p.first_word = e->d_first_word;
+  p.n_doms = e->n_doms;
   p.block_seg = e->d_block_seg;
   p.code_tab = e->d_code_tab;
   p.lv_seg = e->d_lv_seg;
@@ -1241,8 +1342,6 @@ EncParams enc_params(const fptc_encoder *e, uint64_t *d_words, uint8_t *d_symlen
   p.fb_count = e->d_fb_count;
   p.fb_cap = e->fb_cap;
   p.n_blocks = e->n_blocks;
-  p.codes = e->d_codes;
-  p.lens = e->d_lens;
   p.status = e->d_status;
   p.n_segs = e->n_segs;
   p.n_levels = e->n_levels;
@@ -1270,8 +1369,6 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
     }
     std::vector<EncDomain> doms(n_domains);
     std::vector<double> cosv;
-    std::vector<uint32_t> codes;
-    std::vector<uint8_t> lens;
     std::vector<uint32_t> code_tab;
     std::vector<double> bounds(2 * 255 * (size_t)n_domains);
     std::vector<long long> bound_keys(bounds.size());
@@ -1323,14 +1420,12 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
       x.cos_off = (uint32_t)cosv.size();
       for (uint32_t k = 0; k < dm.E; ++k)
         for (uint32_t n = 0; n < dm.N; ++n) cosv.push_back(std::cos(M_PI * (2.0 * n + 1.0) * k / (2.0 * dm.N)));
-      x.code_off = (uint32_t)codes.size();
       uint32_t c[256];
       st = fptc_canonical_codes(&dm, c);
       if (st != FPTC_OK) return st;
-      for (int s = 0; s < 256; ++s) {
-        codes.push_back(c[s]);
-        lens.push_back(dm.code_len[s]);
-        code_tab.push_back(c[s] | (uint32_t)dm.code_len[s] << 16);  // codes have <= lmax <= 16 bits
+      for (int s = 0; s < 256; ++s) {  // codes have <= lmax <= 16 bits
+        const uint32_t l = dm.code_len[s];
+        code_tab.push_back(l ? c[s] << (32u - l) | l : 0u);
       }
     }
     // the same cosines as FP32 high and low parts, transposed per domain:
@@ -1397,6 +1492,7 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
     e->device = device;
     e->n_segs = n_segments;
     e->n_windows = win;
+    e->n_doms = n_domains;
     e->n_levels = lv;
     e->n_blocks = blocks;
     e->level_off = level_off;
@@ -1404,9 +1500,12 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
     if (err == cudaSuccess) err = enc_upload(&e->d_doms, doms.data(), doms.size());
     if (err == cudaSuccess) err = enc_upload(&e->d_cos, cosv.data(), cosv.size());
     if (err == cudaSuccess) err = enc_upload(&e->d_cosf, cosf.data(), cosf.size());
-    if (err == cudaSuccess) err = cudaMalloc(&e->d_blocks, std::max<uint64_t>(blocks, 1) * sizeof(PackState));
-    if (err == cudaSuccess) err = cudaMalloc(&e->d_ref_end, std::max<uint64_t>(blocks, 1) * sizeof(RefEnd));
-    if (err == cudaSuccess) err = cudaMalloc(&e->d_trans, std::max<uint64_t>(blocks, 1) * sizeof(BlockTrans));
+    if (err == cudaSuccess)
+      err = cudaFuncSetAttribute(k_enc_starts<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (kStartWarps + 1) * kStartWarpBytes + kTabDomains * 1024u);
+    if (err == cudaSuccess) err = cudaMalloc(&e->d_recs, std::max<uint64_t>(blocks, 1) * sizeof(PackRec));
+    if (err == cudaSuccess) err = cudaMalloc(&e->d_masks, std::max<uint64_t>(blocks, 1) * kMaskWords * 4);
+    if (err == cudaSuccess) err = cudaMalloc(&e->d_first_word, std::max<uint64_t>(blocks, 1) * 8);
     if (err == cudaSuccess) err = enc_upload(&e->d_block_seg, block_seg.data(), block_seg.size());
     if (err == cudaSuccess) err = enc_upload(&e->d_code_tab, code_tab.data(), code_tab.size());
     for (size_t i = 0; i < bounds.size(); ++i) {  // order keys (see order_key); a NaN bound: no level reached
@@ -1437,8 +1536,6 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
     if (err == cudaSuccess) err = cudaMalloc(&e->d_fb_list, (size_t)e->fb_cap * sizeof(unsigned long long));
     if (err == cudaSuccess) err = cudaMalloc(&e->d_fb_count, sizeof(unsigned int));
     if (err == cudaSuccess) err = cudaDeviceGetAttribute(&e->sm_count, cudaDevAttrMultiProcessorCount, device);
-    if (err == cudaSuccess) err = enc_upload(&e->d_codes, codes.data(), codes.size());
-    if (err == cudaSuccess) err = enc_upload(&e->d_lens, lens.data(), lens.size());
     if (err == cudaSuccess) {
       const EncStatus s0{0u, 0u, ~0ull};
       err = enc_upload(&e->d_status, &s0, 1);
@@ -1522,8 +1619,14 @@ static fptc_status enc_run(fptc_encoder *enc, const float *d_x, bool levels_give
       e = cudaGetLastError();
     }
   }
+  const bool tab = enc->n_doms <= kTabDomains;
   if (e == cudaSuccess && enc->n_blocks) {
-    k_enc_ref<<<(unsigned)((enc->n_blocks + 127) / 128), 128, 0, s>>>(p);
+    const unsigned grid = (unsigned)((enc->n_blocks + kStartWarps - 1) / kStartWarps);
+    const size_t smem = (kStartWarps + 1) * kStartWarpBytes + (tab ? enc->n_doms * 1024u : 0u);
+    if (tab)
+      k_enc_starts<true><<<grid, (kStartWarps + 1) * 32, smem, s>>>(p);
+    else
+      k_enc_starts<false><<<grid, (kStartWarps + 1) * 32, smem, s>>>(p);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
@@ -1531,7 +1634,11 @@ static fptc_status enc_run(fptc_encoder *enc, const float *d_x, bool levels_give
     e = cudaGetLastError();
   }
   if (e == cudaSuccess && enc->n_blocks) {
-    k_enc_pack<<<(unsigned)((enc->n_blocks + kPackWarps * 32 - 1) / (kPackWarps * 32)), kPackWarps * 32, 0, s>>>(p);
+    const unsigned grid = (unsigned)((enc->n_blocks * (kPackBlock / kPackPart) + kPackWarps - 1) / kPackWarps);
+    if (tab)
+      k_enc_pack<true><<<grid, kPackWarps * 32, enc->n_doms * 1024u, s>>>(p);
+    else
+      k_enc_pack<false><<<grid, kPackWarps * 32, 0, s>>>(p);
     e = cudaGetLastError();
   }
   if (e != cudaSuccess) return enc_cuda_fail(e, "encode launch");

@@ -219,3 +219,42 @@ def test_encode_zone1_narrow_linear_part(alpha1):
     else:
         z1 = lh[:enc.n_levels].reshape(-1, d.E)[:, d.B1:d.B2]
         assert np.all(z1 == 128)
+
+
+@pytest.mark.parametrize("n_doms", [1, 20])
+@pytest.mark.parametrize("E", [16, 5, 1])
+def test_pack_block_edges(E, n_doms):
+    """Streams that end just before, on and just after a packing block's last
+    symbol (2048 symbols) and the 64 symbols a word may reach beyond it, at every
+    byte alignment of their levels (E = 5, 1), with few and with more domains than
+    the code tables in shared memory hold: words and counts equal Alg. 1's."""
+    from paper_2605_01086_gb300 import Encoder
+    rng = np.random.default_rng(100 * E + n_doms)
+    doms = []
+    for k in range(n_doms):
+        cl = np.full(256, 13, np.uint8)
+        cl[100:130] = 6
+        cl[130], cl[131] = 2 + k % 3, 3
+        doms.append(oracle.Domain(16, E, min(2, E), E, 50.0, 0.004, (1.0, 1.0, 0.0), 13, cl))
+    edges = [2048 * b + d for b in (1, 2, 64) for d in (-17, -1, 0, 1, 3, 31, 32, 33, 63, 64, 65)] + [1, 16, 17, 63]
+    lens, idx, levels = [], [], []
+    for i, n in enumerate(edges):
+        W = -(-n // E)
+        lens.append(W * 16)
+        idx.append(i % n_doms)
+        kind = i % 3  # mixed lengths, short codes only (long words), constant lengths (packings that never meet)
+        pool = np.arange(256) if kind == 0 else np.array([130, 130, 130, 110]) if kind == 1 else np.array([101, 120])
+        levels.append(rng.choice(pool, size=W * E).astype(np.uint8))
+    enc = Encoder([product_domain(d) for d in doms], lens, idx)
+    lv = np.zeros(max(1, enc.n_levels), np.uint8)
+    for i, L in enumerate(levels):
+        lv[int(enc.level_offsets[i]):int(enc.level_offsets[i]) + L.size] = L
+    words, symlen, n_words = enc.pack(torch.from_numpy(lv).to(enc.device))
+    assert enc.status()[0] == 0
+    wh, sh, nh = words.cpu().numpy().view(np.uint64), symlen.cpu().numpy(), n_words.cpu().numpy()
+    for i, L in enumerate(levels):
+        d = doms[idx[i]]
+        w_o, s_o = oracle.pack_symlen(L, oracle.canonical_codes(d.code_len, d.lmax), d.code_len)
+        w_g, s_g = _room_words(enc, wh, sh, nh, i)
+        np.testing.assert_array_equal(w_g, w_o, err_msg=f"words of stream {i} ({L.size} levels)")
+        np.testing.assert_array_equal(s_g, s_o, err_msg=f"symlen of stream {i} ({L.size} levels)")
