@@ -5,8 +5,9 @@
 //                 window's 16 bins of Eq. 1 by the even/odd butterfly in FP32
 //                 (dct32.cuh) with a bound on its error, and the zone
 //                 quantizer bracketed by that bound.
-//   k_enc_levels  (other shapes) one thread per (window, bin): the bin as a
-//                 compensated FP32 dot product with a bound on its error.
+//   k_enc_levels_any  (other shapes) a warp per tile of windows, folded once
+//                 by the mirror symmetry of the basis: four windows by four
+//                 bins per lane in FP32 with a bound on the sums' error.
 //                 In both, every zone map is monotone in the coefficient, so
 //                 when the levels at c - err and c + err agree the FP64
 //                 coefficient (which lies between) has that level too;
@@ -56,6 +57,8 @@ struct EncDomain {
   // most 126 2^-23 / 2^-12 = 0.06 of a level; otherwise FP64 decides every
   // zone-1 bin outside the deadzone
   uint32_t z1_f32;
+  uint32_t dot_off;      // first of its cosines in rows of any_pairs4(N) (k_enc_levels_any)
+  float two_over_n;
   uint32_t bnd_off;      // first of the domain's 2 x 255 boundaries of the host encoder's zone maps
 };
 
@@ -78,6 +81,7 @@ struct EncStatus {
 };
 
 struct PackRec;
+struct EncUnit;
 
 struct EncParams {
   const float *x;
@@ -94,6 +98,8 @@ struct EncParams {
   uint64_t *first_word;  // per packing block: the stream's words that start before it
   const uint32_t *block_seg;  // per packing block: its segment
   const uint32_t *code_tab;   // per domain, 256 entries: codeword << (32 - length) | length, 0: no codeword
+  const EncUnit *units;       // k_enc_levels_any: the windows of each warp
+  const float *dots;          // and its cosines
   const uint32_t *lv_seg;     // k_enc_levels_w32: the segment of each warp's first window
   const long long *bound_keys;  // per domain: zone 0's, then zone 1's 255 level boundaries (order keys)
   uint32_t n_doms;
@@ -263,64 +269,6 @@ __device__ __forceinline__ unsigned int fb_slot(const EncParams &p) {
   return slot < p.fb_cap ? slot : ~0u;
 }
 
-// One thread per (window, bin): thread g writes level g of the level buffer
-// (streams in caller order, windows, bins), so a warp covers a few windows, the
-// lanes of a window read its samples as broadcasts and the FP32 cosines (a
-// high and a low part) are stored transposed (cosf[2 (n E + k)]) for one
-// wavefront per sample.  The bin is accumulated as a compensated FP32 dot
-// product (exact products by FMA, exact sums by two-sum), whose error is
-// O((N u)^2 sum |x|) + u |c|; the quantizer is evaluated in FP32 at the ends
-// of a bracket that covers that error and the FP32 evaluation's own slack.
-// Bins whose bracket straddles a level boundary go to a list for
-// k_enc_fallback (or, when the list is full, are decided here in FP64).
-__global__ void __launch_bounds__(256) k_enc_levels(EncParams p) {
-  const uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= p.n_levels) return;
-  const uint64_t s = last_leq(p.n_segs, g, [&](uint64_t i) { return p.segs[i].level_offset; });
-  const EncSeg sg = p.segs[s];
-  const EncDomain d = p.doms[sg.domain];
-  const uint32_t N = d.N, E = d.E;
-  const uint64_t local = g - sg.level_offset;
-  const uint64_t w = local / E;
-  const uint32_t k = (uint32_t)(local - w * E);
-  uint32_t L = 128u;
-  if (k < d.B2) {
-    const uint64_t i0 = w * N;
-    const uint64_t avail = sg.n_samples - i0;  // >= 1
-    const uint32_t nn = avail < N ? (uint32_t)avail : N;  // samples past S are zero
-    const float *src = p.x + sg.in_offset + i0;
-    const float2 *ct = reinterpret_cast<const float2 *>(p.cosf) + d.cos_off + k;
-    float hi = 0.0f, lo = 0.0f, s1 = 0.0f;
-    for (uint32_t n = 0; n < nn; ++n) {
-      const float xv = src[n];
-      const float2 cs = ct[(size_t)n * E];
-      // explicit roundings (no contraction): the exact product error by FMA, an exact two-sum
-      const float pr = __fmul_rn(xv, cs.x);
-      const float pe = __fadd_rn(__fmaf_rn(xv, cs.x, -pr), __fmul_rn(xv, cs.y));
-      const float t = __fadd_rn(hi, pr);
-      const float bp = __fsub_rn(t, hi);
-      lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(t, bp)), __fsub_rn(pr, bp)), pe));
-      hi = t;
-      s1 += fabsf(xv);
-    }
-    // |c - c64| bound for c = hi + lo scaled in FP64: twice the compensated
-    // sum's (2^-34 (2/N) sum |x|, which also covers the cosines' representation
-    // and the FP64 evaluation's own rounding for N <= 128)
-    const float err = s1 * (2.0f / (float)N) * 0x1p-34f + 1e-30f;
-    const double cd = ((double)hi + (double)lo) * (2.0 / (double)N);
-    const bool decided = level_bracket64(p, k, cd, 2.0 * (double)err, level_estimate(k, (float)cd, d), d, L);
-    if (!decided) {
-      const unsigned int slot = fb_slot(p);
-      if (slot != ~0u) {
-        p.fb_list[slot] = fb_entry(g, s);
-        return;  // k_enc_fallback writes the level
-      }
-      L = level_fp64_seg(p, g, s);
-    }
-  }
-  p.levels[g] = (uint8_t)L;
-}
-
 // First tier of k_enc_levels_w32 for the 16 bins of a window: levels into lv,
 // the bins the bound cannot settle into the mask undecided (their level 0).
 // T1: the zones of Table 1 (B1 = 2, B2 = 16), fixed per bin at compile time.
@@ -482,7 +430,7 @@ __device__ __forceinline__ void lv_load_async(const EncParams &p, const LvWin &w
 // a bound on each bin's error from the butterfly's own intermediate sums
 // (dct32.cuh dct2_16_bounded; the exact scale 2/N, 4/N for bin 0), plus the
 // FP64 encoder's own rounding; the zone quantizer is bracketed by that bound
-// as in k_enc_levels.  Bins it cannot settle are computed again, spread over
+// as in k_enc_levels_any.  Bins it cannot settle are computed again, spread over
 // the warp's lanes, as compensated dot products; what those cannot settle goes
 // to the FP64 list.  A warp takes `groups` groups of 32 consecutive windows
 // (kLvGroups, fewer where a batch has too few windows to fill the chip with
@@ -551,7 +499,7 @@ __global__ void __launch_bounds__(kLvThreads, 5) k_enc_levels_w32(EncParams p, u
     if (!valid) undecided = 0u;
     // second tier, spread over the warp's lanes: each undecided bin again as a
     // compensated FP32 dot product (|error| <= 2^-34 (2/N) sum |x|, as in
-    // k_enc_levels); what that cannot settle goes to the FP64 list
+    // level_compensated); what that cannot settle goes to the FP64 list
     const uint32_t cnt = (uint32_t)__popc(undecided);
     const uint32_t incl = lane_prefix(cnt, lane);
     const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
@@ -1079,9 +1027,11 @@ __global__ void __launch_bounds__(128) k_enc_scan(EncParams p) {
   }
 }
 
-// Level of listed bin g of segment s from its compensated FP32 coefficient (as
-// in k_enc_levels: |error| <= 2^-34 (2/N) sum |x|); false when that bound
-// cannot settle it.
+// Level of bin g of segment s from its compensated FP32 coefficient (exact
+// products by FMA, exact sums by two-sum: error O((N u)^2 sum |x|) + u |c|; the
+// bound 2^-34 (2/N) sum |x| also covers the cosines' representation and the
+// FP64 evaluation's own rounding for N <= 128); false when that bound cannot
+// settle it.
 __device__ __forceinline__ bool level_compensated(const EncParams &p, uint64_t g, uint64_t s, uint32_t &L) {
   const EncSeg sg = p.segs[s];
   const EncDomain d = p.doms[sg.domain];
@@ -1125,6 +1075,285 @@ __device__ __forceinline__ bool level_compensated(const EncParams &p, uint64_t g
   const float err2 = s1 * (2.0f / (float)d.N) * 0x1p-34f + 1e-30f;
   const double cd = ((double)hi + (double)lo) * (2.0 / (double)d.N);
   return level_bracket64(p, k, cd, 2.0 * (double)err2, level_estimate(k, (float)cd, d), d, L);
+}
+
+// ---- level kernel for every other shape (N in [4, 128], any E) ------------------
+// A warp takes tiles of `tile` windows.  A window is folded once, u[n] = x[n] +
+// x[N-1-n] and v[n] = x[n] - x[N-1-n] for n < P = ceil(N / 2) (the middle sample
+// of an odd N alone in u), because bin k of Eq. 1 is sum_n u[n] cos(k, n) for
+// even k and the same of v for odd k.  A lane then has four windows and four
+// bins of one parity: 64 multiply-adds for four 16-byte reads of the folded
+// windows and four of the cosines, in FP32.  The next tile's samples are
+// copied into shared memory meanwhile.
+//
+// Error of such a sum against the exact one: each of the P fused multiply-adds
+// rounds a partial sum of magnitude at most S = sum |u| (or |v|), the folding
+// rounds each u to 2^-24 |u| and the cosines (at most 1) are off by at most
+// 2^-25, so (P + 1.5) 2^-24 S and terms of second order; (P + 4) 2^-24 S is
+// used, and 2^-40 (sum |u| + sum |v|) for the host encoder's own rounding in FP64
+// (N 2^-52 sum |x|, and sum |x| <= sum |u| + sum |v|).  The zone maps are bracketed
+// by that bound as in the window kernel; a bin it does not settle (about one
+// in 200) goes to the list of k_enc_fallback, or, where a tile has many, is
+// settled here by the compensated sum.
+// Bound by instruction issue (about 30 instructions a sample at N = 64, E = 32).
+// 16.8 M samples at N = 64, E = 32: 75 us (one thread per bin with the compensated
+// sum for every bin took 457 us).
+constexpr uint32_t kAnyWarps = 4;
+constexpr uint32_t kAnyTile0 = 4;  // zone-0 bins of a window mapped by all lanes together
+
+struct EncUnit {
+  uint64_t win;  // first window in its stream
+  uint32_t seg;
+  uint32_t n;    // windows
+};
+
+// Rows of n floats in 16-byte pieces, an odd number of them (rows of
+// different windows start in different banks).
+__host__ __device__ constexpr uint32_t any_pitch(uint32_t n) { return ((n + 3) / 4 | 1u) * 4; }
+__host__ __device__ constexpr uint32_t any_pairs4(uint32_t N) { return ((N + 1) / 2 + 3) / 4 * 4; }
+// Windows per tile: enough for one item of four windows and four bins per
+// lane, within 2048 samples.
+__host__ __device__ constexpr uint32_t any_groups(uint32_t E) { return ((E + 1) / 2 + 3) / 4 + (E / 2 + 3) / 4; }
+__host__ __device__ constexpr uint32_t any_tile(uint32_t N, uint32_t E) {
+  uint32_t t = 16;
+  while (t < 64 && any_groups(E) * t / 4 < 32 && 2 * t * N <= 2048) t *= 2;
+  return t;
+}
+// Bytes per warp: samples, folded rows, their sums of magnitudes, zone-0 bins,
+// the list of bins to settle, levels.
+__host__ __device__ constexpr uint32_t any_bytes(uint32_t N, uint32_t E) {
+  const uint32_t t = any_tile(N, E);
+  return t * any_pitch(N) * 4 + 2 * t * any_pitch(any_pairs4(N)) * 4 + 4 * t * 4 + t * kAnyTile0 * 4 + 512 * 2 +
+         (t * E + 15) / 16 * 16;
+}
+
+__global__ void __launch_bounds__(kAnyWarps * 32, 4) k_enc_levels_any(EncParams p, uint64_t n_units, uint32_t warp_bytes) {
+  extern __shared__ __align__(16) unsigned char any_smem[];
+  const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+  const uint64_t unit = (uint64_t)blockIdx.x * kAnyWarps + wid;
+  if (unit >= n_units) return;  // the whole warp
+  const EncUnit un = p.units[unit];
+  const EncSeg &sg = p.segs[un.seg];
+  const EncDomain &d = p.doms[sg.domain];
+  const uint32_t N = d.N, E = d.E, B1 = d.B1, B2 = d.B2;
+  const uint32_t P = (N + 1) / 2, P4 = any_pairs4(N), tile = any_tile(N, E);
+  const uint32_t xp = any_pitch(N), up = any_pitch(P4);
+  const uint32_t evens = (E + 1) / 2, ge = (evens + 3) / 4, go = (E / 2 + 3) / 4;
+  float *const xs = reinterpret_cast<float *>(any_smem + (size_t)wid * warp_bytes);
+  float *const us = xs + tile * xp;          // [tile][up], then v
+  float *const vs = us + tile * up;
+  float *const sums = vs + tile * up;        // [u half 0, u half 1, v half 0, v half 1][tile]
+  float *const z0 = sums + 4 * tile;         // [tile][kAnyTile0]
+  uint16_t *const work = reinterpret_cast<uint16_t *>(z0 + tile * kAnyTile0);
+  uint8_t *const lev = reinterpret_cast<uint8_t *>(work + 512);
+  const float *const src0 = p.x + sg.in_offset + un.win * N;
+  const uint64_t avail0 = sg.n_samples - un.win * N;  // samples of the stream from the unit's first
+  const bool vec = N % 4 == 0 && (reinterpret_cast<uintptr_t>(src0) & 15u) == 0;
+  const float *const dots = p.dots + d.dot_off;
+  // n < 2^16 divided by N or N / 4 by a multiplication
+  const uint32_t magic = (uint32_t)((0x100000000ull + N - 1) / N);
+  auto load = [&](uint32_t w0) {  // the tile's samples, zero past the stream's end
+    const uint32_t nw = un.n - w0 < tile ? un.n - w0 : tile, total = nw * N;
+    const float *src = src0 + (uint64_t)w0 * N;
+    const uint64_t left = avail0 - (uint64_t)w0 * N;
+    if (vec && left >= total) {
+      for (uint32_t i = 4 * lane; i < total; i += 128) {
+        const uint32_t w = __umulhi(i, magic);
+        cp_async_16(xs + w * xp + (i - w * N), src + i);
+      }
+    } else {
+      for (uint32_t i = lane; i < total; i += 32) {
+        const uint32_t w = __umulhi(i, magic);
+        cp_async_4z(xs + w * xp + (i - w * N), i < left ? src + i : p.x, i < left ? 4u : 0u);
+      }
+    }
+    cp_async_commit_group();
+  };
+  load(0);
+  for (uint32_t w0 = 0; w0 < un.n; w0 += tile) {
+    const uint32_t nw = un.n - w0 < tile ? un.n - w0 : tile;
+    cp_async_wait_group<0>();
+    __syncwarp();
+    // ---- fold: lane (or lanes' turn t) = window and every other piece of four pairs
+    for (uint32_t t = lane; t < 2 * tile; t += 32) {
+      const uint32_t w = t % tile, h = t / tile;
+      const float *x = xs + w * xp;
+      float su = 0.0f, sv = 0.0f;
+      for (uint32_t c = 4 * h; c < P4; c += 8) {
+        float a[4], b[4];
+        if (N % 4 == 0) {
+          const float4 q = *reinterpret_cast<const float4 *>(x + c);
+          const float4 r = *reinterpret_cast<const float4 *>(x + N - 4 - c);
+          a[0] = q.x, a[1] = q.y, a[2] = q.z, a[3] = q.w;
+          b[0] = r.w, b[1] = r.z, b[2] = r.y, b[3] = r.x;
+        } else {
+#pragma unroll
+          for (uint32_t i = 0; i < 4; ++i) {
+            a[i] = c + i < P ? x[c + i] : 0.0f;
+            b[i] = c + i < P ? x[N - 1 - c - i] : 0.0f;
+          }
+        }
+        float u[4], v[4];
+#pragma unroll
+        for (uint32_t i = 0; i < 4; ++i) {
+          const bool in = c + i < P, mid = 2 * (c + i) + 1 == N;
+          u[i] = in ? (mid ? a[i] : a[i] + b[i]) : 0.0f;
+          v[i] = in && !mid ? a[i] - b[i] : 0.0f;
+          su += fabsf(u[i]);
+          sv += fabsf(v[i]);
+        }
+        *reinterpret_cast<float4 *>(us + w * up + c) = make_float4(u[0], u[1], u[2], u[3]);
+        *reinterpret_cast<float4 *>(vs + w * up + c) = make_float4(v[0], v[1], v[2], v[3]);
+      }
+      sums[h * tile + w] = su;
+      sums[(2 + h) * tile + w] = sv;
+    }
+    __syncwarp();
+    if (w0 + tile < un.n) load(w0 + tile);
+    // ---- bins, four windows x four bins a lane and round
+    const uint64_t win = un.win + w0;
+    const uint32_t wgs = tile / 4, items = wgs * (ge + go);
+    for (uint32_t i0 = 0; i0 < items; i0 += 32) {
+      const uint32_t item = i0 + lane;
+      uint32_t undecided = 0, wg = 0, k0 = 0;
+      if (item < items) {
+        wg = item % wgs;
+        const uint32_t bg = item / wgs;
+        const bool odd = bg >= ge;
+        k0 = odd ? 8 * (bg - ge) + 1 : 8 * bg;  // bins k0, k0 + 2, + 4, + 6
+        const float *rows = (odd ? vs : us) + wg * up;
+        const float *cs[4];
+#pragma unroll
+        for (uint32_t j = 0; j < 4; ++j) cs[j] = dots + (k0 + 2 * j < E ? k0 + 2 * j : k0) * P4;
+        float acc[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
+#pragma unroll 2
+        for (uint32_t c = 0; c < P4; c += 4) {
+          float4 f[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) f[i] = *reinterpret_cast<const float4 *>(rows + i * wgs * up + c);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float4 g = __ldg(reinterpret_cast<const float4 *>(cs[j] + c));
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              acc[i][j] = fmaf(f[i].x, g.x, acc[i][j]);
+              acc[i][j] = fmaf(f[i].y, g.y, acc[i][j]);
+              acc[i][j] = fmaf(f[i].z, g.z, acc[i][j]);
+              acc[i][j] = fmaf(f[i].w, g.w, acc[i][j]);
+            }
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const uint32_t w = wg + i * wgs;
+          if (w >= nw) continue;
+          const float su = sums[w] + sums[tile + w], sv = sums[2 * tile + w] + sums[3 * tile + w];
+          const bool finite = su + sv <= 1.0e38f;
+          // bound on |a - a64|, a the unscaled sum (c = a 2 / N)
+          const float eb = (odd ? sv : su) * ((float)(P + 4) * 0x1p-24f) + (su + sv) * 0x1p-40f + 1e-28f;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint32_t k = k0 + 2 * j;
+            if (k >= E) continue;
+            if (k < B1 && k < kAnyTile0) {
+              z0[w * kAnyTile0 + k] = acc[i][j];
+              continue;
+            }
+            uint32_t L = 128u;
+            bool und = false;
+            if (k < B2) {
+              if (!finite) {
+                und = true;
+              } else if (k < B1) {
+                const float c = acc[i][j] * d.two_over_n;
+                const float m = eb * d.two_over_n + d.slack0 + fabsf(c) * 0x1p-21f;
+                L = zone0_level32(c - m, d);
+                und = L != zone0_level32(c + m, d);
+              } else if (d.z1_f32) {  // as in tier1_bins_fast
+                const float ak = fabsf(acc[i][j]);
+                const float m = eb + d.u1_slack + ak * 0x1p-21f;
+                const float lo = ak - m, hi = ak + m;
+                const bool dz = hi < d.u1_d1, edge = lo <= d.u1_d1, pos = acc[i][j] > 0.0f;
+                const float kk = pos ? d.u1_kp : d.u1_kn;
+                const int v0 = __float2int_rd(fmaf(fminf(lo, d.u1_A1) - d.u1_d1, kk, 0.5f));
+                const int v1 = __float2int_rd(fmaf(fminf(hi, d.u1_A1) - d.u1_d1, kk, 0.5f));
+                und = !dz && (edge || v0 != v1);
+                L = dz ? 128u : (uint32_t)(pos ? 129 + v0 : 127 - v0);
+              } else {
+                const float c = acc[i][j] * d.two_over_n;
+                und = !zone1_decide32(c, eb * d.two_over_n + d.slack1 + fabsf(c) * 0x1p-21f, d, L);
+              }
+            }
+            undecided |= und ? 1u << (4 * i + j) : 0u;
+            lev[w * E + k] = (uint8_t)(und ? 0u : L);
+          }
+        }
+      }
+      // ---- the bins that bound did not settle: a few to the list (their level, 0
+      // here, is written after the tile's), many from the compensated sum
+      const uint32_t cnt = (uint32_t)__popc(undecided);
+      const uint32_t incl = lane_prefix(cnt, lane);
+      const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+      if (total) {
+        uint32_t o = incl - cnt;
+        for (uint32_t u = undecided; u; u &= u - 1u) {
+          const uint32_t q = (uint32_t)(__ffs(u) - 1);
+          work[o++] = (uint16_t)((wg + (q >> 2) * wgs) * 128u + k0 + 2 * (q & 3u));
+        }
+        __syncwarp();
+        for (uint32_t i = lane; i < total; i += 32) {
+          const uint32_t w = work[i] >> 7, k = work[i] & 127u;
+          const uint64_t g = sg.level_offset + (win + w) * E + k;
+          uint32_t L = 0u;
+          if (total <= kTier2Inline || !level_compensated(p, g, un.seg, L)) {
+            const unsigned int slot = fb_slot(p);
+            L = 0u;
+            if (slot != ~0u)
+              p.fb_list[slot] = fb_entry(g, un.seg);
+            else
+              L = level_fp64_seg(p, g, un.seg);
+          }
+          lev[w * E + k] = (uint8_t)L;
+        }
+      }
+      __syncwarp();
+    }
+    // ---- zone 0, a bin a lane
+    const uint32_t nz = B1 < kAnyTile0 ? B1 : kAnyTile0;
+    for (uint32_t t = lane; t < nw * nz; t += 32) {
+      const uint32_t w = t / nz, k = t - w * nz;
+      const float su = sums[w] + sums[tile + w], sv = sums[2 * tile + w] + sums[3 * tile + w];
+      const float eb = ((k & 1u) ? sv : su) * ((float)(P + 4) * 0x1p-24f) + (su + sv) * 0x1p-40f + 1e-28f;
+      const float c = z0[w * kAnyTile0 + k] * d.two_over_n;
+      const float m = eb * d.two_over_n + d.slack0 + fabsf(c) * 0x1p-21f;
+      uint32_t L = zone0_level32(c - m, d);
+      if (!(su + sv <= 1.0e38f) || L != zone0_level32(c + m, d)) {
+        const uint64_t g = sg.level_offset + (win + w) * E + k;
+        const unsigned int slot = fb_slot(p);
+        L = 0u;
+        if (slot != ~0u)
+          p.fb_list[slot] = fb_entry(g, un.seg);
+        else
+          L = level_fp64_seg(p, g, un.seg);
+      }
+      lev[w * E + k] = (uint8_t)L;
+    }
+    __syncwarp();
+    // ---- the tile's levels, consecutive lanes to consecutive bytes
+    uint8_t *const dst = p.levels + sg.level_offset + win * E;
+    const uint32_t bytes = nw * E;
+    if ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0 && (bytes & 15u) == 0) {
+      for (uint32_t i = 16 * lane; i < bytes; i += 512)
+        *reinterpret_cast<uint4 *>(dst + i) = *reinterpret_cast<const uint4 *>(lev + i);
+    } else {
+      for (uint32_t i = lane; i < bytes; i += 32) dst[i] = lev[i];
+    }
+    __syncwarp();
+  }
 }
 
 // The listed bins, one per thread: from their compensated FP32 coefficient
@@ -1291,6 +1520,10 @@ struct fptc_encoder {
   uint32_t *d_code_tab = nullptr;           // [n_domains][256]
   uint32_t *d_lv_seg = nullptr;             // [warps of k_enc_levels_w32]
   long long *d_bound_keys = nullptr;        // [n_domains][2][255]
+  EncUnit *d_units = nullptr;               // [n_units] (k_enc_levels_any)
+  float *d_dots = nullptr;                  // its cosines
+  uint64_t n_units = 0;
+  uint32_t any_warp_bytes = 0;              // its shared memory per warp
   bool w32 = false;               // every domain N = 32, E = 16: the window-per-thread level kernel
   uint32_t *d_seg_bad = nullptr;
   unsigned long long *d_fb_list = nullptr;
@@ -1316,6 +1549,8 @@ void enc_free(fptc_encoder *e) {
   cudaFree(e->d_block_seg);
   cudaFree(e->d_code_tab);
   cudaFree(e->d_lv_seg);
+  cudaFree(e->d_units);
+  cudaFree(e->d_dots);
   cudaFree(e->d_bound_keys);
   cudaFree(e->d_seg_bad);
   cudaFree(e->d_fb_list);
@@ -1356,6 +1591,8 @@ EncParams enc_params(const fptc_encoder *e, uint64_t *d_words, uint8_t *d_symlen
   p.block_seg = e->d_block_seg;
   p.code_tab = e->d_code_tab;
   p.lv_seg = e->d_lv_seg;
+  p.units = e->d_units;
+  p.dots = e->d_dots;
   p.bound_keys = e->d_bound_keys;
   p.seg_bad = e->d_seg_bad;
   p.fb_list = e->d_fb_list;
@@ -1389,6 +1626,7 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
     }
     std::vector<EncDomain> doms(n_domains);
     std::vector<double> cosv;
+    uint32_t dots_size = 0;
     std::vector<uint32_t> code_tab;
     std::vector<double> bounds(2 * 255 * (size_t)n_domains);
     std::vector<long long> bound_keys(bounds.size());
@@ -1438,6 +1676,9 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
       host_zone_bounds(dm, 0, bounds.data() + x.bnd_off);
       host_zone_bounds(dm, 1, bounds.data() + x.bnd_off + 255);
       x.cos_off = (uint32_t)cosv.size();
+      x.dot_off = dots_size;
+      dots_size += any_pairs4(dm.N) * dm.E;
+      x.two_over_n = (float)(2.0 / dm.N);
       for (uint32_t k = 0; k < dm.E; ++k)
         for (uint32_t n = 0; n < dm.N; ++n) cosv.push_back(std::cos(M_PI * (2.0 * n + 1.0) * k / (2.0 * dm.N)));
       uint32_t c[256];
@@ -1516,7 +1757,8 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
     e->n_levels = lv;
     e->n_blocks = blocks;
     e->level_off = level_off;
-    cudaError_t err = enc_upload(&e->d_segs, segs.data(), segs.size());
+    cudaError_t err = cudaDeviceGetAttribute(&e->sm_count, cudaDevAttrMultiProcessorCount, device);
+    if (err == cudaSuccess) err = enc_upload(&e->d_segs, segs.data(), segs.size());
     if (err == cudaSuccess) err = enc_upload(&e->d_doms, doms.data(), doms.size());
     if (err == cudaSuccess) err = enc_upload(&e->d_cos, cosv.data(), cosv.size());
     if (err == cudaSuccess) err = enc_upload(&e->d_cosf, cosf.data(), cosf.size());
@@ -1548,6 +1790,33 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
       }
       err = enc_upload(&e->d_lv_seg, lvs.data(), lvs.size());
     }
+    if (err == cudaSuccess && !e->w32) {  // units of whole tiles, up to eight where that leaves the chip full
+      std::vector<float> dots;
+      for (uint32_t d = 0; d < n_domains; ++d) {
+        const uint32_t N = doms[d].N, pairs = (N + 1) / 2, p4 = any_pairs4(N);
+        e->any_warp_bytes = std::max(e->any_warp_bytes, (any_bytes(N, doms[d].E) + 15u) / 16u * 16u);
+        for (uint32_t k = 0; k < doms[d].E; ++k)
+          for (uint32_t n = 0; n < p4; ++n)
+            dots.push_back(n < pairs ? (float)cosv[doms[d].cos_off + (size_t)k * N + n] : 0.0f);
+      }
+      uint64_t tiles = 0;
+      for (const EncSeg &sg : segs) {
+        const uint32_t t = any_tile(doms[sg.domain].N, doms[sg.domain].E);
+        tiles += (sg.n_windows + t - 1) / t;
+      }
+      const uint64_t per = std::min<uint64_t>(8, std::max<uint64_t>(1, tiles / ((uint64_t)e->sm_count * 32u)));
+      std::vector<EncUnit> units;
+      for (uint64_t i = 0; i < n_segments; ++i) {
+        const uint64_t step = per * any_tile(doms[segs[i].domain].N, doms[segs[i].domain].E);
+        for (uint64_t w = 0; w < segs[i].n_windows; w += step)
+          units.push_back(EncUnit{w, (uint32_t)i, (uint32_t)std::min<uint64_t>(step, segs[i].n_windows - w)});
+      }
+      e->n_units = units.size();
+      err = enc_upload(&e->d_units, units.data(), units.size());
+      if (err == cudaSuccess) err = enc_upload(&e->d_dots, dots.data(), dots.size());
+      if (err == cudaSuccess)
+        err = set_dynamic_smem_limit(reinterpret_cast<const void *>(&k_enc_levels_any), kAnyWarps * e->any_warp_bytes);
+    }
     if (err == cudaSuccess) err = cudaMalloc(&e->d_seg_bad, std::max<uint64_t>(n_segments, 1) * sizeof(uint32_t));
     // room for the bins decided in FP64: 0.2 % of them on signals, a few percent when
     // decoded signals are encoded again (their levels 127 and 129 reconstruct on the
@@ -1555,7 +1824,6 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
     e->fb_cap = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(lv / 16, 4096), uint64_t(1) << 28);
     if (err == cudaSuccess) err = cudaMalloc(&e->d_fb_list, (size_t)e->fb_cap * sizeof(unsigned long long));
     if (err == cudaSuccess) err = cudaMalloc(&e->d_fb_count, sizeof(unsigned int));
-    if (err == cudaSuccess) err = cudaDeviceGetAttribute(&e->sm_count, cudaDevAttrMultiProcessorCount, device);
     if (err == cudaSuccess) {
       const EncStatus s0{0u, 0u, ~0ull};
       err = enc_upload(&e->d_status, &s0, 1);
@@ -1624,7 +1892,6 @@ static fptc_status enc_run(fptc_encoder *enc, const float *d_x, bool levels_give
   p.x = d_x;
   cudaError_t e = cudaSuccess;
   if (!levels_given && enc->n_levels) {
-    const uint64_t blocks = (enc->n_levels + 255) / 256;
     e = cudaMemsetAsync(enc->d_fb_count, 0, sizeof(unsigned int), s);
     if (e == cudaSuccess) {
       if (enc->w32) {
@@ -1633,8 +1900,10 @@ static fptc_status enc_run(fptc_encoder *enc, const float *d_x, bool levels_give
         const uint32_t groups = (uint32_t)std::min<uint64_t>(kLvGroups, (all + warps - 1) / warps);
         const uint64_t per = (uint64_t)kLvThreads * groups;
         k_enc_levels_w32<<<(unsigned)((enc->n_windows + per - 1) / per), kLvThreads, 0, s>>>(p, enc->n_windows, groups);
-      } else
-        k_enc_levels<<<(unsigned)blocks, 256, 0, s>>>(p);
+      } else {
+        k_enc_levels_any<<<(unsigned)((enc->n_units + kAnyWarps - 1) / kAnyWarps), kAnyWarps * 32,
+                           kAnyWarps * enc->any_warp_bytes, s>>>(p, enc->n_units, enc->any_warp_bytes);
+      }
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) {

@@ -258,3 +258,43 @@ def test_pack_block_edges(E, n_doms):
         w_g, s_g = _room_words(enc, wh, sh, nh, i)
         np.testing.assert_array_equal(w_g, w_o, err_msg=f"words of stream {i} ({L.size} levels)")
         np.testing.assert_array_equal(s_g, s_o, err_msg=f"symlen of stream {i} ({L.size} levels)")
+
+
+@pytest.mark.parametrize("N,E,B1", [(4, 4, 2), (5, 5, 0), (6, 3, 3), (8, 3, 2), (16, 8, 2), (24, 12, 2), (32, 32, 6),
+                                    (33, 17, 1), (48, 24, 2), (64, 32, 2), (100, 50, 2), (127, 127, 5), (128, 64, 2),
+                                    (128, 1, 1)])
+def test_encode_shapes_match_host(N, E, B1):
+    """Levels and words of other shapes equal the FP64 host encoder's in every bin:
+    tiles cut by stream ends, streams that start at any alignment, bins that the
+    single-precision bound cannot settle (decoded signals encoded again: their
+    levels sit on the deadzone edge), values near the largest float."""
+    from paper_2605_01086_gb300 import Encoder, codec
+    lens = [1, N - 1, N, N + 1, 15 * N, 16 * N + 3, 64 * N, 129 * N + 1, 40001]
+    idx = [0] * len(lens)
+    flat, offs = siggen.signals([i % 4 for i in range(len(lens))], [siggen.stream_seed(9, i) for i in range(len(lens))],
+                                lens)
+    dom = codec.train_domain(flat, offs, np.array(lens, np.uint64), N, E, B1, max(B1, E - 1), 50.0, 0.004, 12, 99.9)
+    flat = flat.copy()
+    big = int(offs[7])
+    flat[big:big + 2 * N] *= np.float32(1e30)
+    flat[big + 5 * N:big + 5 * N + 2] = np.float32(3e38)
+    again = np.zeros_like(flat)
+    for r in range(2):  # the signals, then what they decode to
+        x = flat if r == 0 else again
+        enc = Encoder([dom], lens, idx)
+        lv = torch.empty(max(1, enc.n_levels), dtype=torch.uint8, device=enc.device)
+        words, symlen, n_words = enc.encode(torch.from_numpy(x).to(enc.device), levels=lv)
+        assert enc.status()[0] == 0
+        wh, sh, nh, lh = (words.cpu().numpy().view(np.uint64), symlen.cpu().numpy(), n_words.cpu().numpy(),
+                          lv.cpu().numpy())
+        od = oracle.Domain(dom.N, dom.E, dom.B1, dom.B2, dom.mu, dom.alpha1, tuple(dom.scale), dom.lmax, dom.code_len)
+        for i, S in enumerate(lens):
+            o = int(offs[i])
+            w_h, s_h, l_h = codec.encode_stream(dom, x[o:o + S])
+            l_g = lh[int(enc.level_offsets[i]):int(enc.level_offsets[i]) + l_h.size]
+            np.testing.assert_array_equal(l_g, l_h, err_msg=f"levels of stream {i}")
+            w_g, s_g = _room_words(enc, wh, sh, nh, i)
+            np.testing.assert_array_equal(w_g, w_h, err_msg=f"words of stream {i}")
+            np.testing.assert_array_equal(s_g, s_h, err_msg=f"symlen of stream {i}")
+            if r == 0:
+                again[o:o + S] = oracle.decode_stream(w_h, s_h, S, od)[0].astype(np.float32)
