@@ -217,17 +217,24 @@ cudaError_t launch_tcs(const DecodeParams &p, const WarpParams &wp, const TcPara
 
 // warp-tile kernel for other shapes: N in [4, 128] for every domain (several N
 // in one plan), any E <= N (decode_shape.cu); tiles of shape_windows_per_tile(N,
-// E) windows; `any`: some domain's N is not a power of two (shape_pow2_only
-// false), served by the kernel instance that holds that transform
+// E) windows; forms: the OR of what its domains' transforms are at this thread
+// count (kz = min(E, B2)), which picks the kernel instance
+constexpr uint32_t kShapeCompiled = 1, kShapeAny = 2;
 bool shape_supported(uint32_t N);
-bool shape_pow2_only(uint32_t N);
+uint32_t shape_forms(uint32_t N, uint32_t kz, uint32_t threads);
 uint32_t shape_windows_per_tile(uint32_t N, uint32_t E);
 size_t shape_smem_layout(uint32_t threads, const uint32_t *lmax, const uint32_t *N, const uint32_t *E,
-                         uint32_t n_domains, WarpParams *wp);
-cudaError_t shape_smem_config(uint32_t threads, bool any, size_t smem);
-cudaError_t shape_occupancy(uint32_t threads, bool any, size_t smem, int *ctas_per_sm);
-cudaError_t launch_shape(const DecodeParams &p, const WarpParams &wp, const CUtensorMap &out_map, uint32_t threads,
-                         bool any, uint32_t grid, size_t smem, cudaStream_t stream);
+                         const uint32_t *kz, uint32_t n_domains, WarpParams *wp);
+cudaError_t shape_smem_config(uint32_t threads, uint32_t forms, size_t smem);
+cudaError_t shape_occupancy(uint32_t threads, uint32_t forms, size_t smem, int *ctas_per_sm);
+// The output's tensor maps: rows of 32 floats (WarpParams out_tma bit 0), and
+// windows x chunks x 32 floats for N = 64 (bit 1) and N = 128 (bit 2).
+struct ShapeMaps {
+  CUtensorMap rows, n64, n128;
+};
+bool encode_window_map(CUtensorMap *map, float *out, uint64_t extent, uint32_t N);
+cudaError_t launch_shape(const DecodeParams &p, const WarpParams &wp, const ShapeMaps &maps, uint32_t threads,
+                         uint32_t forms, uint32_t grid, size_t smem, cudaStream_t stream);
 
 // adjoint for N = 32, E = 16 plans on the warp-tile machinery (backward_warp.cu)
 size_t backward_warp_smem_layout(uint32_t threads, const uint32_t *lmax, uint32_t n_domains, WarpParams *wp);

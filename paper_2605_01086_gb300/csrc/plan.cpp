@@ -51,7 +51,7 @@ struct fptc_plan {
   bool shape = false;     // every domain has N in [4, 128] and the warp-tile kernel of
                           // decode_shape.cu serves the plan (N = 32, E = 16 plans use decode_warp.cu)
   uint32_t tcs_N = 0, tcs_E = 0;  // the tensor-core kernel of decode_tcs.cu serves this shape (0: decode_tc.cu)
-  bool shape_any = false; // a domain's N is not a power of two (the shape kernel instance with that transform)
+  uint32_t shape_forms = 0; // transforms its domains use (kShapeCompiled, kShapeAny): the kernel instance
   WarpParams wp{};
   TcParams tp{};
   uint32_t threads = 256, grid = 0, ctas_per_sm = 0;
@@ -212,11 +212,12 @@ fptc_status smem_fits(const char *kernel, uint32_t threads, size_t smem) {
 fptc_status configure_launch(fptc_plan *p) {
   uint32_t threads = p->opts.threads ? p->opts.threads : (p->kind == FPTC_KERNEL_TENSOR ? 512u : 256u);
   const bool shape = p->kind == FPTC_KERNEL_WARP_TILE && p->shape;
-  std::vector<uint32_t> lm, ns, es;
+  std::vector<uint32_t> lm, ns, es, kz;
   for (const auto &d : p->domains) {
     lm.push_back(d.lmax);
     ns.push_back(d.N);
     es.push_back(d.E);
+    kz.push_back(std::min(d.E, d.B2));
   }
   if (p->kind == FPTC_KERNEL_WARP_TILE && p->opts.threads == 0) {
     // as many warps per SM as one CTA's shared memory allows (32 at most; 16
@@ -228,7 +229,7 @@ fptc_status configure_launch(fptc_plan *p) {
     threads = 128;
     if (shape) {
       for (uint32_t t : {512u, 256u})
-        if (shape_smem_layout(t, lm.data(), ns.data(), es.data(), (uint32_t)lm.size(), &probe) <= (size_t)optin) {
+        if (shape_smem_layout(t, lm.data(), ns.data(), es.data(), kz.data(), (uint32_t)lm.size(), &probe) <= (size_t)optin) {
           threads = t;
           break;
         }
@@ -313,11 +314,13 @@ fptc_status configure_launch(fptc_plan *p) {
     }
     if (e == cudaSuccess) occ = std::min<int>(occ, 1);
   } else if (shape) {
-    p->smem = shape_smem_layout(threads, lm.data(), ns.data(), es.data(), (uint32_t)lm.size(), &p->wp);
+    p->shape_forms = 0;
+    for (size_t d = 0; d < lm.size(); ++d) p->shape_forms |= shape_forms(ns[d], kz[d], threads);
+    p->smem = shape_smem_layout(threads, lm.data(), ns.data(), es.data(), kz.data(), (uint32_t)lm.size(), &p->wp);
     if (const fptc_status fs = smem_fits("warp-tile", threads, p->smem); fs != FPTC_OK) return fs;
-    e = shape_smem_config(threads, p->shape_any, p->smem);
+    e = shape_smem_config(threads, p->shape_forms, p->smem);
     if (e != cudaSuccess) return cuda_fail(e, "decode shared-memory size");
-    e = shape_occupancy(threads, p->shape_any, p->smem, &occ);
+    e = shape_occupancy(threads, p->shape_forms, p->smem, &occ);
   } else if (p->kind == FPTC_KERNEL_WARP_TILE) {
     p->smem = warp_smem_layout(threads, lm.data(), (uint32_t)lm.size(), &p->wp);
     if (const fptc_status fs = smem_fits("warp-tile", threads, p->smem); fs != FPTC_OK) return fs;
@@ -480,10 +483,22 @@ cudaError_t run_range(const fptc_plan *p, const IndexParams &ip0, const DecodePa
   if (p->kind == FPTC_KERNEL_BLOCK_TILE) return launch_fixed(dp, p->threads, grid, p->smem, st);
   if (p->kind == FPTC_KERNEL_WARP_TILE) {
     WarpParams wp = p->wp;
+    if (p->shape) {
+      ShapeMaps maps;
+      std::memset(&maps, 0, sizeof(maps));
+      wp.out_tma = encode_out_map(&maps.rows, dp.out, p->out_extent) ? 1u : 0u;
+      bool n64 = false, n128 = false;
+      for (const auto &d : p->domains) {
+        n64 = n64 || d.N == 64;
+        n128 = n128 || d.N == 128;
+      }
+      if (n64 && encode_window_map(&maps.n64, dp.out, p->out_extent, 64)) wp.out_tma |= 2u;
+      if (n128 && encode_window_map(&maps.n128, dp.out, p->out_extent, 128)) wp.out_tma |= 4u;
+      return launch_shape(dp, wp, maps, p->threads, p->shape_forms, grid, p->smem, st);
+    }
     CUtensorMap map;
     std::memset(&map, 0, sizeof(map));
     wp.out_tma = encode_out_map(&map, dp.out, p->out_extent) ? 1u : 0u;
-    if (p->shape) return launch_shape(dp, wp, map, p->threads, p->shape_any, grid, p->smem, st);
     return launch_warp(dp, wp, map, p->threads, grid, p->smem, st);
   }
   if (p->kind == FPTC_KERNEL_TENSOR && p->tcs_N) {
@@ -628,12 +643,13 @@ fptc_status fptc_plan_create(fptc_plan **out, int device, const fptc_domain *dom
         if (fixed_ok) {
           fits = warp_smem_layout(128, lm.data(), n_domains, &probe) <= (size_t)optin;
         } else {
-          std::vector<uint32_t> ns(n_domains), es(n_domains);
+          std::vector<uint32_t> ns(n_domains), es(n_domains), kz(n_domains);
           for (uint32_t d = 0; d < n_domains; ++d) {
             ns[d] = domains[d].N;
             es[d] = domains[d].E;
+            kz[d] = std::min(domains[d].E, domains[d].B2);
           }
-          fits = shape_smem_layout(256, lm.data(), ns.data(), es.data(), n_domains, &probe) <= (size_t)optin;
+          fits = shape_smem_layout(256, lm.data(), ns.data(), es.data(), kz.data(), n_domains, &probe) <= (size_t)optin;
         }
       }
       o.kernel = fits ? FPTC_KERNEL_WARP_TILE : (all_fixed ? FPTC_KERNEL_BLOCK_TILE : FPTC_KERNEL_GENERIC);
@@ -725,8 +741,6 @@ fptc_status fptc_plan_create(fptc_plan **out, int device, const fptc_domain *dom
     p->lut_cap = 1u << max_lmax;
     p->kind = (int)o.kernel;
     p->shape = shape_ok;
-    p->shape_any = false;
-    for (uint32_t d = 0; d < n_domains; ++d) p->shape_any = p->shape_any || !shape_pow2_only(domains[d].N);
     p->tcs_N = tcs_ok ? domains[0].N : 0u;
     p->tcs_E = tcs_ok ? domains[0].E : 0u;
 

@@ -197,3 +197,33 @@ def test_tensor_core_shape_trained_signals():
     _, _, out32, _ = gpu_decode(ref, b, out_fill=0.0)
     rel = float(torch.linalg.vector_norm((out - out32).double()) / torch.linalg.vector_norm(out32.double()))
     assert rel < 1e-6
+
+
+@pytest.mark.parametrize("N,E,B1", [(16, 4, 0), (16, 5, 5), (32, 9, 3), (32, 32, 2), (64, 16, 2), (64, 17, 1),
+                                    (64, 33, 4), (64, 64, 2), (128, 32, 0), (128, 33, 2), (128, 64, 3),
+                                    (128, 65, 2)])
+@pytest.mark.parametrize("align", [32, 4])
+def test_shape_transform_forms(N, E, B1, align):
+    """Bin counts on both sides of where the compiled transforms change, first
+    zones other than Table 1's, streams that end inside an output step and whose
+    outputs start at any chunk of a window row of the output."""
+    cl = np.full(256, 8, np.uint8)
+    doms = [oracle.Domain(N, E, B1, E, 40.0, 0.01, (2.0, 1.5, 0.0), 8, cl),
+            oracle.Domain(32, 16, 2, 16, 50.0, 0.004, (1.0, 1.0, 0.0), 8, cl)]
+    rng = np.random.default_rng(N * 1000 + E)
+    lens, idx, levels = [], [], []
+    for S in [1, N, 32 * N, 32 * N + 33, 64 * N, 65 * N - 1, 100 * N + 7, 20000]:
+        for d in (0, 1):
+            lens.append(S)
+            idx.append(d)
+            levels.append(rng.integers(0, 256, size=doms[d].windows(S) * doms[d].E).astype(np.uint8))
+    b = crafted_batch(doms, levels, lens, idx)
+    plan = make_plan(b, out_align=align, kernel="warp_tile")
+    _, _, out, lv = gpu_decode(plan, b, out_fill=float("nan"))
+    compare_with_oracle(plan, b, out, lv)
+    h = out.cpu().numpy()
+    mask = np.ones(h.size, bool)
+    for sg in plan.segments:
+        mask[int(sg["out_offset"]):int(sg["out_offset"]) + int(sg["n_samples"])] = False
+    assert np.all(np.isnan(h[mask]))
+    assert plan.device_status()[0] == 0
