@@ -11,7 +11,8 @@
 // sum_n v[n] B[2j+1][n] and the even bins the same construction on u (twice
 // more), 232 FP32 operations per window with compile-time cosines.
 //
-// Per tile of 128 windows (a warp's contiguous tile range): levels come from
+// Per group of tiles of one segment, up to 128 windows (a warp's contiguous tile
+// range): levels come from
 // the saved level buffer (16 bytes per window) or are decoded again; the
 // gradient rows of each 32-window step arrive by a TMA tensor load into the
 // warp's shared tile (rows of 32 floats, 128-byte swizzle; the next step's
@@ -80,11 +81,11 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_backward_warp(const BackwardP
   unit_tiles(p, (uint64_t)blockIdx.x * WARPS + warp, (uint64_t)gridDim.x * WARPS, tw0, tw1);
   if (tw0 >= tw1) return;
 
-  uint32_t s = find_segment(p.segs, p.seg_begin, p.seg_end, tw0);
+  uint32_t s = warp_find_segment(p.segs, p.seg_begin, p.seg_end, tw0, lane);
   uint32_t pn = 0;
   Ctx nxt{0, 0, 0, s, 0};
   if (redecode) {  // where tile tw0 starts, then its first words
-    nxt = first_ctx(p, s, tw0, lane);
+    nxt = first_ctx(p, s, tw0, lane, (uint64_t)p.domains[p.segs[s].domain].tile_windows * kE);
     pn = fetch_pass0(p, nxt, lane, wbuf);
   }
 
@@ -107,8 +108,12 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_backward_warp(const BackwardP
     acc0 = acc1 = 0.0;
   };
 
-  for (uint64_t g = tw0; g < tw1 && !timeout; ++g) {
+  uint64_t g1 = tw0;  // tiles [g, g1) are taken together
+  for (uint64_t g = tw0; g < tw1 && !timeout; g = g1) {
     while (g >= p.segs[s].tile_base + p.segs[s].n_tiles) ++s;
+    const uint32_t T = p.domains[p.segs[s].domain].tile_windows;
+    g1 = g + (T < (uint32_t)kT ? kT / T : 1u);
+    g1 = min(min(g1, tw1), p.segs[s].tile_base + p.segs[s].n_tiles);
     Ctx cur{0, 0, 0, s, 1};
     uint64_t w[kWPL] = {0, 0};
     uint32_t n[kWPL] = {0, 0};
@@ -122,8 +127,8 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_backward_warp(const BackwardP
         n[u] = (pn >> (8 * u)) & 0xffu;
       }
       __syncwarp();
-      if (!cur.ok && g + 1 < tw1) {  // skipped tile: the next one is located without it
-        nxt = next_ctx(p, g, s, cur, TileEnd{0u, 0u, 0u});
+      if (!cur.ok && g1 < tw1) {  // skipped tiles: the next one is located without them
+        nxt = next_ctx(p, g1 - 1, s, cur, TileEnd{0u, 0u, 0u});
         pn = fetch_pass0(p, nxt, lane, wbuf);
       }
     }
@@ -134,9 +139,9 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_backward_warp(const BackwardP
       flush();
       acc_dom = sg.domain;
     }
-    const uint64_t win0 = (g - sg.tile_base) * kT;
-    const uint64_t left = sg.n_windows - win0;
-    const uint32_t nwin = left < (uint64_t)kT ? (uint32_t)left : (uint32_t)kT;
+    const uint64_t win0 = (g - sg.tile_base) * T;
+    const uint64_t left = sg.n_windows - win0, tiles_win = (g1 - g) * T;
+    const uint32_t nwin = (uint32_t)(left < tiles_win ? left : tiles_win);
     const float *deq = reinterpret_cast<const float *>(smem_raw + dd.deq_off);
     const float a0 = p.scale ? p.scale[sg.domain * 3 + 0] : p.domains[sg.domain].scale[0];
     const float a1 = p.scale ? p.scale[sg.domain * 3 + 1] : p.domains[sg.domain].scale[1];
@@ -167,8 +172,8 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_backward_warp(const BackwardP
     if (redecode) {
       const TileEnd te = decode_tile(p, cur, nwin * kE, dd, smem_raw, stage, lane, w, n);
       if (te.bad && lane == 0) flag_bad(p.status, te.bad, sg.caller_index);
-      if (g + 1 < tw1) {  // tile g + 1 starts where tile g ended
-        nxt = next_ctx(p, g, s, cur, te);
+      if (g1 < tw1) {  // tile g1 starts where tile g1 - 1 ended
+        nxt = next_ctx(p, g1 - 1, s, cur, te);
         pn = fetch_pass0(p, nxt, lane, wbuf);
       }
       __syncwarp();

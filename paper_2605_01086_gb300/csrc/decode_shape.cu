@@ -112,13 +112,7 @@ __device__ __forceinline__ uint32_t load_shape_tables(const DecodeParams &p, uin
       x.pad = 0;
       ds[d] = x;
     }
-    uint16_t *lut = reinterpret_cast<uint16_t *>(smem + lut_off);
-    const uint16_t *g_lut = p.luts + dm.lut_offset;
-    const uint32_t entries = 1u << dm.lmax;
-    for (uint32_t i = threadIdx.x; i < entries; i += THREADS) {
-      const uint32_t v = __ldg(g_lut + i);
-      lut[i] = (uint16_t)((v >> 8) | ((v & 0xffu) << 8));
-    }
+    load_warp_lut<THREADS>(p.luts + dm.lut_offset, dm.lmax, smem + lut_off);
     float a0 = p.scale ? p.scale[d * 3 + 0] : dm.scale[0];
     float a1 = p.scale ? p.scale[d * 3 + 1] : dm.scale[1];
     a0 = a0 > 1e-30f ? a0 : 0.0f;
@@ -537,7 +531,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_decode_shape(const DecodePara
 
   Ctx nxt;
   {
-    const uint32_t s = find_segment(p.segs, p.seg_begin, p.seg_end, tw0);
+    const uint32_t s = warp_find_segment(p.segs, p.seg_begin, p.seg_end, tw0, lane);
     const DomS &d0 = ds[p.segs[s].domain];
     nxt = first_ctx(p, s, tw0, lane, (uint64_t)d0.T * d0.E);
   }

@@ -1,22 +1,24 @@
-// Fused decode for the Table 1 shape (N = 32, E = 16) with one warp per tile.
+// Fused decode for the Table 1 shape (N = 32, E = 16) with no block-wide barrier.
 //
-// Each warp owns a contiguous range of tiles of 128 windows (2048 symbols, 4096
-// samples) and runs Sec. 4.2 on each with no block-wide barrier:
+// Each warp owns a contiguous range of tiles of 32 windows (512 symbols, 1024
+// samples: what its lanes transform in one step) and runs Sec. 4.2 on it as one
+// stream (stream_tiles in warp_tile.cuh):
 //  1. SymLen decode.  A pass gives every lane two consecutive words; a warp
 //     scan of their symbol counts places each word's codewords (compaction,
 //     Sec. 4.2.1).  A lane decodes a word with one decode-table lookup per
-//     codeword and stores the codeword's level as one byte at its tile
-//     position (two per 16-bit store).  Nothing else happens per
-//     codeword: the dequantization waits for step 2, where the bin of every
-//     value is known at compile time.  The 64-bit word is shifted through
-//     hi:lo with a marker bit under it, so a word whose codewords need more
-//     than 64 bits shows as an empty buffer at the end (no per-codeword count).
-//  2. Dequantization and inverse DCT, one window per lane.  The lane reads its
-//     window's 16 levels, turns each into A_z * unit_z(level) (one table read;
-//     the bin, hence the zone row, is fixed per register), and evaluates the
-//     inverse of Eq. 1 by the even/odd split of the DCT-III:
-//     x[n] = E[n] + O[n], x[31-n] = E[n] - O[n] with O the odd bins and E the
-//     even bins, itself split the same way twice (E[15-n] = EE[n] - EO[n],
+//     codeword and stores the codeword's level as one byte at its place behind
+//     the symbols not yet transformed (two per 16-bit store).  Nothing else
+//     happens per codeword: the dequantization waits for step 2, where the bin
+//     of every value is known at compile time.  The 64-bit word is shifted
+//     through hi:lo with a marker bit under it, so a word whose codewords need
+//     more than 64 bits shows as an empty buffer at the end (no per-codeword
+//     count).
+//  2. Dequantization and inverse DCT, one window per lane, whenever 512 symbols
+//     are there.  The lane reads its window's 16 levels, turns each into A_z *
+//     unit_z(level) (one table read; the bin, hence the zone row, is fixed per
+//     register), and evaluates the inverse of Eq. 1 by the even/odd split of the
+//     DCT-III: x[n] = E[n] + O[n], x[31-n] = E[n] - O[n] with O the odd bins and
+//     E the even bins, itself split the same way twice (E[15-n] = EE[n] - EO[n],
 //     EE[7-n] = EEE[n] - EEO[n]); 229 FP32 operations per window with the
 //     cosines as compile-time constants, so neither a basis nor coefficients
 //     pass through shared memory.
@@ -27,12 +29,17 @@
 //     with a TMA tensor store (the output viewed as rows of 32 floats), so the
 //     output never passes through the L1 load/store pipe.  Other windows use
 //     32-byte (or 16-byte, or scalar) streaming stores.
-//  The warp locates the first tile of its range from the index's chunk
-//  offsets; tile g+1 starts at the word where tile g's decode ended, and its
-//  first words are loaded then (hidden by tile g's transform); the words of a
-//  tile's next decode pass load while the current pass decodes.
+//  The warp locates the first word of its range from the index's chunk offsets;
+//  the words of a pass load while the pass before it decodes and its steps run.
 // The decode tables, dequantization rows and basis of every domain stay in
 // shared memory for the whole kernel.
+//
+// Bound by instruction issue (decode table lookups and the transform) on large
+// batches.  Tiles of 128 windows decoded one by one left 11 % of the warps'
+// time idle on 124 M samples (7.1 tiles a warp: some had 8), decoded the words
+// at a tile's end in a pass of their own and started every tile afresh: 3,750
+// warp instructions per 4096 samples, 144 us for 124 M samples (four domains,
+// ragged lengths); as one stream 119 us.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -122,6 +129,18 @@ __device__ __forceinline__ void idct32(const float (&c)[16], Put put) {
   }
 }
 
+// Symbols a warp's stage holds: a step's and a pass's (usually 600), and up to
+// the bytes a warp has beside its output tile in the other warp-tile kernels.
+constexpr int kCap = kMiscBytes - 2 * kStreamGuard;
+constexpr uint32_t kTileWin = 32;  // windows per tile: one step
+
+struct GeoW {
+  __device__ uint32_t tile_windows(const DomW &) const { return kTileWin; }
+  __device__ uint32_t tile_symbols(const DomW &) const { return kTileWin * kE; }
+  __device__ uint32_t step_windows(const DomW &) const { return kStepWin; }
+  __device__ uint32_t bins(const DomW &) const { return kE; }
+};
+
 template <int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, WARPS > 16 ? 1 : 32 / WARPS) k_decode_warp(
     const DecodeParams p, const WarpParams wp, const __grid_constant__ CUtensorMap out_map) {
@@ -132,106 +151,53 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS > 16 ? 1 : 32 / WARPS) k_dec
   load_domain_tables<WARPS * 32>(p, wp.n_domains, smem_raw);
   __syncthreads();
 
-  unsigned char *const wbase = smem_raw + wp.warp_off + warp * kMiscBytes;
-  uint64_t *const wbuf = reinterpret_cast<uint64_t *>(wbase);                       // first-pass words
-  uint8_t *const stage = wbase + kStageOff;                           // tile position 0
+  uint8_t *const stage = smem_raw + wp.warp_off + warp * stream_bytes(kCap) + kStreamGuard;
   // output staging tile: 1024-byte aligned (the period of the 128-byte swizzle)
-  const uintptr_t tiles0 = (reinterpret_cast<uintptr_t>(smem_raw + wp.warp_off + WARPS * kMiscBytes) + 1023) &
-                           ~uintptr_t(1023);
+  const uintptr_t tiles0 =
+      (reinterpret_cast<uintptr_t>(smem_raw + wp.warp_off + WARPS * stream_bytes(kCap)) + 1023) & ~uintptr_t(1023);
   unsigned char *const otile = reinterpret_cast<unsigned char *>(tiles0) + warp * kOutTile;
+  // row `lane` of the staging tile, 16-byte chunk c at c ^ (lane & 7)
+  unsigned char *const row = otile + lane * (kN * 4);
+  const uint32_t sx = lane & 7u;
   const bool want_lev = p.levels != nullptr;
-  bool tma_pending = false;
+  const bool out32 = (reinterpret_cast<uintptr_t>(p.out) & 31u) == 0;
 
   // ---- this warp's tiles: an even split of the launch's tile range over all warps
   uint64_t tw0, tw1;
   unit_tiles(p, (uint64_t)blockIdx.x * WARPS + warp, (uint64_t)gridDim.x * WARPS, tw0, tw1);
   if (tw0 >= tw1) return;
 
-  // prologue: where tile tw0 starts, then its first words
-  Ctx nxt = first_ctx(p, find_segment(p.segs, p.seg_begin, p.seg_end, tw0), tw0, lane);
-  uint32_t pn = fetch_pass0(p, nxt, lane, wbuf);
-
-  for (uint64_t g = tw0; g < tw1; ++g) {
-    // ---- tile g: its first words have been requested
-    cp_async_wait_all();
-    __syncwarp();
-    const Ctx cur = nxt;
-    uint64_t w[kWPL];
-    uint32_t n[kWPL];
-#pragma unroll
-    for (int u = 0; u < kWPL; ++u) {
-      w[u] = wbuf[kWPL * lane + u];
-      n[u] = (pn >> (8 * u)) & 0xffu;
-    }
-    __syncwarp();
-    const uint64_t g1 = g + 1;
-
-    const SegDev &sg = p.segs[cur.seg];
-    const DomW dd = dw[sg.domain];
-    const uint64_t win0 = (g - sg.tile_base) * kT;
-    const uint64_t left = sg.n_windows - win0;
-    const uint32_t nwin = left < (uint64_t)kT ? (uint32_t)left : (uint32_t)kT;
-
-    // ---- 1. SymLen decode into the level bytes
-    TileEnd te{0u, 0u, 0u};
-    if (cur.ok) {
-      te = decode_tile(p, cur, nwin * kE, dd, smem_raw, stage, lane, w, n);
-      if (te.bad && lane == 0) flag_bad(p.status, te.bad, sg.caller_index);
-    }
-
-    // ---- first words of tile g + 1 (in flight during the transform)
-    if (g1 < tw1) {
-      nxt = next_ctx(p, g, cur.seg, cur, te);
-      pn = fetch_pass0(p, nxt, lane, wbuf);
-    }
-    __syncwarp();
-
-    // ---- 2./3. dequantization + inverse transform + reassembly, one window per lane
-    if (cur.ok) {
-      const float *deq = reinterpret_cast<const float *>(smem_raw + dd.deq_off);
-      float *const out = p.out + sg.out_offset;
-      const uint64_t S = sg.n_samples;
-      const uint32_t aligned = sg.out_aligned;
-      const bool vec32 = (aligned & 2u) && (reinterpret_cast<uintptr_t>(p.out) & 31u) == 0;
-      const bool tma_seg = wp.out_tma && (aligned & 4u);
-      uint8_t *const lev = want_lev ? p.levels + sg.level_offset + win0 * kE : nullptr;
-#pragma unroll 1
-      for (uint32_t w0 = 0; w0 < nwin; w0 += kStepWin) {
-        const uint32_t wi = w0 + lane;
-        // all 32 windows of the step whole and inside the segment: one TMA store
-        const bool tma_step = tma_seg && w0 + kStepWin <= nwin && (win0 + w0 + kStepWin) * kN <= S;
-        if (tma_pending) {
-          if (lane == 0) tma_wait_read();  // the previous step has left the staging tile
-          __syncwarp();
-          tma_pending = false;
-        }
-        // row `lane` of the staging tile, 16-byte chunk c at c ^ (lane & 7)
-        unsigned char *const row = otile + lane * (kN * 4);
-        const uint32_t sx = lane & 7u;
-        if (wi < nwin) {
-          const uint4 sv = *reinterpret_cast<const uint4 *>(stage + wi * kE);
+  stream_tiles<kCap>(
+      p, tw0, tw1, dw, smem_raw, stage, lane, GeoW{},
+      // dequantization + inverse transform + reassembly, one window per lane
+      [&](const SegDev &sg, const DomW &dd, const uint8_t *levels, uint64_t win, uint32_t n) {
+        const float *deq = reinterpret_cast<const float *>(smem_raw + dd.deq_off);
+        const uint32_t aligned = sg.out_aligned;
+        const uint64_t s0 = win * kN, S = sg.n_samples;  // the step's first sample
+        if (lane == 0) tma_wait_read();  // the previous step has left the staging tile
+        __syncwarp();
+        if (lane < n) {
+          const uint4 sv = *reinterpret_cast<const uint4 *>(levels + lane * kE);
           float c[16];
           window_coefs(sv, deq, dd.zmask, c);
-          if (want_lev) put_levels(lev + wi * kE, sv);
+          if (want_lev) put_levels(p.levels + sg.level_offset + (win + lane) * kE, sv);
           idct32(c, [&](int b, const float(&v)[8]) {
             *reinterpret_cast<float4 *>(row + (((2 * b) ^ sx) << 4)) = make_float4(v[0], v[1], v[2], v[3]);
             *reinterpret_cast<float4 *>(row + (((2 * b + 1) ^ sx) << 4)) = make_float4(v[4], v[5], v[6], v[7]);
           });
         }
-        if (tma_step) {
+        // all 32 windows of the step whole and inside the segment: one TMA store
+        if (wp.out_tma && (aligned & 4u) && n == kStepWin && s0 + kStepWin * kN <= S) {
           fence_async_shared();
           __syncwarp();
-          if (lane == 0) tma_store_rows(&out_map, otile, (int32_t)((sg.out_offset >> 5) + win0 + w0));
-          tma_pending = true;
-        } else if (wi < nwin) {  // each lane stores its own row
-          const uint64_t s0 = (win0 + wi) * kN;
-          store_row(row, sx, out + s0, s0 + kN <= S ? kN : (uint32_t)(S - s0), vec32, aligned & 1u);
+          if (lane == 0) tma_store_rows(&out_map, otile, (int32_t)((sg.out_offset + s0) >> 5));
+        } else if (lane < n) {  // each lane stores its own row
+          const uint64_t r0 = s0 + lane * kN;
+          store_row(row, sx, p.out + sg.out_offset + r0, r0 + kN <= S ? kN : (uint32_t)(S - r0), out32 && (aligned & 2u),
+                    aligned & 1u);
         }
-      }
-    }
-    __syncwarp();  // the level bytes are rewritten by the next tile
-  }
-  if (tma_pending && lane == 0) tma_wait_all();
+      });
+  if (lane == 0) tma_wait_all();
 }
 
 template <int WARPS>
@@ -253,7 +219,7 @@ void *wpick(uint32_t threads) {
 
 }  // namespace
 
-uint32_t warp_tile_windows() { return kT; }
+uint32_t warp_tile_windows() { return kTileWin; }
 
 // Shared-memory layout of the warp-tile kernel; returns total bytes, fills wp.
 size_t warp_smem_layout(uint32_t threads, const uint32_t *lmax, uint32_t n_domains, WarpParams *wp) {
@@ -267,10 +233,10 @@ size_t warp_smem_layout(uint32_t threads, const uint32_t *lmax, uint32_t n_domai
   }
   o = align16(o);
   wp->warp_off = (uint32_t)o;
-  wp->warp_bytes = (uint32_t)kMiscBytes;
+  wp->warp_bytes = (uint32_t)stream_bytes(kCap);
   wp->out_tma = 0;
   const size_t warps = threads / 32;
-  return o + warps * kMiscBytes + 1023 + warps * kOutTile;  // + alignment of the staging tiles
+  return o + warps * stream_bytes(kCap) + 1023 + warps * kOutTile;  // + alignment of the staging tiles
 }
 
 bool encode_out_map(CUtensorMap *map, float *out, uint64_t extent) {

@@ -52,6 +52,28 @@ __device__ __forceinline__ uint32_t find_segment(const SegDev *segs, uint32_t lo
   return lo;
 }
 
+// Index of the last of n > 0 ascending entries with entry(i) <= g (entry(0) <=
+// g holds), by the whole warp: 32 probes a round, so three dependent loads for
+// 16,384 entries where a binary search takes fourteen.
+template <class F>
+__device__ __forceinline__ uint64_t warp_last_leq(uint64_t n, uint64_t g, uint32_t lane, F entry) {
+  uint64_t lo = 0;
+  while (n > 1) {
+    const uint64_t step = (n + 31) / 32, i = lane * step;
+    const uint32_t m = __ballot_sync(0xffffffffu, i < n && entry(lo + i) <= g);
+    const uint64_t k = (uint64_t)(__popc(m) - 1) * step;
+    lo += k;
+    n = n - k < step ? n - k : step;
+  }
+  return lo;
+}
+
+// find_segment by the whole warp.
+__device__ __forceinline__ uint32_t warp_find_segment(const SegDev *segs, uint32_t lo, uint32_t hi, uint64_t g,
+                                                      uint32_t lane) {
+  return lo + (uint32_t)warp_last_leq(hi - lo, g, lane, [&](uint64_t i) { return segs[lo + i].tile_base; });
+}
+
 // Huffman decode of one SymLen word (Sec. 4.2.1): peek lmax bits MSB first,
 // look the prefix up in the decode table (entry = level | length << 8), emit,
 // shift the word by the code length; exactly n codewords.  The symbol at tile

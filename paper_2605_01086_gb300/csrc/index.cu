@@ -23,11 +23,6 @@
 namespace fptc {
 namespace {
 
-__device__ __forceinline__ void flag_bad(DevStatus *st, unsigned int flag, uint32_t caller_index) {
-  atomicOr(&st->flags, flag);
-  atomicMin(&st->first_bad, (unsigned long long)caller_index);
-}
-
 // Segment (queue index) owning chunk c: the last segment whose chunk_base <= c.
 __device__ __forceinline__ uint32_t chunk_segment(const SegDev *segs, uint32_t lo, uint32_t hi, uint64_t c) {
   while (hi - lo > 1) {

@@ -12,7 +12,7 @@
 // segment is read.
 #pragma once
 
-#include "fptc_internal.h"
+#include "device_util.cuh"
 
 namespace fptc {
 
@@ -63,19 +63,13 @@ __device__ __forceinline__ bool block_over64(const uint4 &v) {
 // The word of segment sg that holds symbol `target` (< the segment's symbol
 // count) and how many of its symbols come before it, from the chunk offsets of
 // the index (chunk_off[c] = symbol offset in the segment of chunk c's first
-// word): the last chunk whose offset is <= target, by binary search, then a
+// word): the last chunk whose offset is <= target, by a search, then a
 // warp scan over that chunk's blocks.  Warp-collective; every lane gets the
 // result.
 __device__ __forceinline__ TileRec symbol_word(const uint8_t *symlen, const uint64_t *chunk_off, const SegDev &sg,
                                                uint64_t target, uint32_t lane) {
-  uint64_t lo = sg.chunk_base, hi = sg.chunk_base + sg.n_chunks;
-  while (hi - lo > 1) {
-    const uint64_t mid = lo + (hi - lo) / 2;
-    if (chunk_off[mid] <= target)
-      lo = mid;
-    else
-      hi = mid;
-  }
+  const uint64_t base = sg.chunk_base;
+  const uint64_t lo = base + warp_last_leq(sg.n_chunks, target, lane, [&](uint64_t i) { return chunk_off[base + i]; });
   const LaneBlock b = load_block(symlen, sg, lo - sg.chunk_base, lane);
   const uint32_t tsum = block_sum(b.v);
   uint32_t x = tsum;

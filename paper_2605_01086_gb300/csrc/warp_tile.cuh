@@ -249,6 +249,25 @@ __device__ __forceinline__ uint32_t fetch_pass0(const DecodeParams &p, const Ctx
   return packed;
 }
 
+// A domain's decode table into shared memory with its entries' bytes swapped
+// (len | level << 8), eight entries a load (the tables start on 16-byte boundaries).
+template <int THREADS>
+__device__ __forceinline__ void load_warp_lut(const uint16_t *g_lut, uint32_t lmax, unsigned char *dst) {
+  const uint32_t entries = 1u << lmax;
+  if (entries >= 8) {
+    for (uint32_t i = threadIdx.x; i < entries / 8; i += THREADS) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4 *>(g_lut) + i);
+      reinterpret_cast<uint4 *>(dst)[i] = make_uint4(__byte_perm(v.x, 0u, 0x2301), __byte_perm(v.y, 0u, 0x2301),
+                                                     __byte_perm(v.z, 0u, 0x2301), __byte_perm(v.w, 0u, 0x2301));
+    }
+  } else {
+    for (uint32_t i = threadIdx.x; i < entries; i += THREADS) {
+      const uint32_t v = __ldg(g_lut + i);
+      reinterpret_cast<uint16_t *>(dst)[i] = (uint16_t)((v >> 8) | ((v & 0xffu) << 8));
+    }
+  }
+}
+
 // Every domain's tables into shared memory from byte 0 (the layout of
 // warp_smem_layout; offsets computed here, not indexed from a parameter
 // block): the DomW array, then per domain the decode table (entries rewritten
@@ -275,13 +294,7 @@ __device__ __forceinline__ uint32_t load_domain_tables(const DecodeParams &p, ui
       x.pad[0] = x.pad[1] = x.pad[2] = 0;
       dw[d] = x;
     }
-    uint16_t *lut = reinterpret_cast<uint16_t *>(smem + lut_off);
-    const uint16_t *g_lut = p.luts + dm.lut_offset;
-    const uint32_t entries = 1u << dm.lmax;
-    for (uint32_t i = threadIdx.x; i < entries; i += THREADS) {
-      const uint32_t v = __ldg(g_lut + i);
-      lut[i] = (uint16_t)((v >> 8) | ((v & 0xffu) << 8));
-    }
+    load_warp_lut<THREADS>(p.luts + dm.lut_offset, dm.lmax, smem + lut_off);
     float a0 = p.scale ? p.scale[d * 3 + 0] : dm.scale[0];
     float a1 = p.scale ? p.scale[d * 3 + 1] : dm.scale[1];
     a0 = a0 > 1e-30f ? a0 : 0.0f;
@@ -441,6 +454,202 @@ __device__ __forceinline__ void store_row(const unsigned char *row, uint32_t sx,
   } else {
     for (uint32_t n = 0; n < m; ++n)
       dst[n] = *reinterpret_cast<const float *>(row + ((((n >> 2) ^ sx) << 4) | ((n & 3u) << 2)));
+  }
+}
+
+// ---- streaming decode -----------------------------------------------------------
+// A warp's range of tiles, segment by segment, decoded as one stream of passes:
+// a pass gives every lane two consecutive words, a scan of their symbol counts
+// their places behind the symbols already in the warp's stage; whenever a step's
+// symbols are there the caller's transform takes them, and what is left moves to
+// the front.  Nothing is decoded twice or left idle where a tile ends, so the
+// tile (the unit in which ranges are split) can be as small as a step.  The words
+// of a pass are loaded while the pass before it decodes and its steps run.
+
+constexpr int kStreamGuard = kGuard;  // bytes before (symbols of a unit's first word that are not its) and after the stage
+__host__ __device__ constexpr int stream_bytes(int cap) { return 2 * kStreamGuard + cap; }
+
+// Words of a pass: two consecutive words per lane, their counts n0 | n1 << 8.
+struct PassWords {
+  ulonglong2 w;
+  uint32_t n;
+};
+
+// Words base + 2 lane, + 1 of [lo, hi) (zero outside).  base: a 16-byte boundary.
+__device__ __forceinline__ PassWords load_pass_words(const DecodeParams &p, int64_t base, int64_t lo, int64_t hi,
+                                                     uint32_t lane) {
+  PassWords r{{0ull, 0ull}, 0u};
+  const int64_t i = base + 2 * (int64_t)lane;
+  if (base >= lo && base + kPassWords <= hi && (reinterpret_cast<uintptr_t>(p.symlen + base) & 1u) == 0) {
+    r.w = __ldg(reinterpret_cast<const ulonglong2 *>(p.words + i));
+    r.n = __ldg(reinterpret_cast<const uint16_t *>(p.symlen + i));
+  } else {
+    if (i >= lo && i < hi) {
+      r.w.x = __ldg(p.words + i);
+      r.n = __ldg(p.symlen + i);
+    }
+    if (i + 1 >= lo && i + 1 < hi) {
+      r.w.y = __ldg(p.words + i + 1);
+      r.n |= (uint32_t)__ldg(p.symlen + i + 1) << 8;
+    }
+  }
+  return r;
+}
+
+// One pass's words of a lane into the level bytes at dst (their order).
+template <class D>
+__device__ __forceinline__ uint32_t decode_pair(const PassWords &c, uint32_t n0, uint32_t n1, uint32_t gap,
+                                                uint8_t *dst, const uint16_t *lut, const D &dd) {
+  uint32_t bad;
+  if (dd.complete && dd.shift == 20u) {  // L_max = 12, the trained tables' limit
+    bad = decode_word<false, 20u>(c.w.x, n0, dst, lut, 20u);
+    bad |= decode_word<false, 20u>(c.w.y, n1, dst + gap, lut, 20u);
+  } else if (dd.complete) {
+    bad = decode_word<false>(c.w.x, n0, dst, lut, dd.shift);
+    bad |= decode_word<false>(c.w.y, n1, dst + gap, lut, dd.shift);
+  } else {
+    bad = decode_word<true>(c.w.x, n0, dst, lut, dd.shift);
+    bad |= decode_word<true>(c.w.y, n1, dst + gap, lut, dd.shift);
+  }
+  return bad;
+}
+
+// The tiles [t0, t1) (of T windows each, T = tile_windows(dd)) of a launch.
+// stage: kStreamGuard bytes before it and CAP + kStreamGuard from it on are the warp's;
+// step(sg, dd, levels, win, n): n windows of segment sg from window win, levels
+// at `levels` (16-byte aligned); step_windows(dd): windows of a whole step, whose
+// symbols are a multiple of 16 and, with a word's 64, at most CAP.
+// Shared memory per warp: kStreamGuard + CAP + kStreamGuard bytes.
+// Barriers: step is entered with the levels visible to the warp; they are
+// rewritten only after a warp barrier.
+template <int CAP, class Dom, class Geo, class Step>
+__device__ __forceinline__ void stream_tiles(const DecodeParams &p, uint64_t t0, uint64_t t1, const Dom *doms,
+                                             const unsigned char *smem, uint8_t *stage, uint32_t lane, const Geo &geo,
+                                             const Step &step) {
+  const uint32_t odd = (uint32_t)(reinterpret_cast<uintptr_t>(p.words) >> 3) & 1u;  // word 0 is off a 16-byte boundary
+  auto floor2 = [&](int64_t w) -> int64_t { return w - (int64_t)(((uint32_t)w + odd) & 1u); };
+  uint32_t s = warp_find_segment(p.segs, p.seg_begin, p.seg_end, t0, lane);
+  int64_t base;         // the pass's first word
+  int32_t fill = 0;     // symbols in the stage (negative: those of the unit's first word before it)
+  bool ok = p.seg_bad[s] == 0;
+  PassWords nx;
+  {
+    const SegDev &sg = p.segs[s];
+    int64_t lo = (int64_t)sg.word_offset;
+    if (ok && t0 != sg.tile_base) {
+      const TileRec r = symbol_word(p.symlen, p.chunk_off, sg, (t0 - sg.tile_base) * geo.tile_symbols(doms[sg.domain]), lane);
+      ok = r.pad == 0;
+      lo = (int64_t)r.first_word;
+      fill = -(int32_t)r.skip;
+    }
+    base = floor2(lo);
+    nx = load_pass_words(p, base, lo, ok ? (int64_t)(sg.word_offset + sg.n_words) : lo, lane);
+  }
+  uint64_t t = t0;
+  while (true) {
+    // ---- a unit: the range's tiles of segment s, from tile t
+    const SegDev &sg = p.segs[s];
+    const Dom &dd = doms[sg.domain];
+    const uint32_t E = geo.bins(dd), sw = geo.step_windows(dd);
+    uint64_t win = (t - sg.tile_base) * geo.tile_windows(dd);
+    // windows of the unit left (a warp's share of what device memory holds fits 32 bits)
+    uint32_t left;
+    {
+      const uint64_t seg_end = sg.tile_base + sg.n_tiles;
+      left = (uint32_t)((t1 < seg_end ? (t1 - sg.tile_base) * geo.tile_windows(dd) : sg.n_windows) - win);
+      t = t1 < seg_end ? t1 : seg_end;  // the next unit's first tile
+    }
+    uint32_t bad = 0;
+    uint32_t s1 = s;   // the next unit's segment, its words and whether it is decoded
+    int64_t lo1 = 0;
+    bool ok1 = false;
+    bool more = ok;
+    auto next_segment = [&](int64_t &hi1) {
+      do ++s1; while (t >= p.segs[s1].tile_base + p.segs[s1].n_tiles);  // segments without tiles
+      lo1 = (int64_t)p.segs[s1].word_offset;
+      hi1 = lo1 + (int64_t)p.segs[s1].n_words;
+      ok1 = p.seg_bad[s1] == 0;
+      if (!ok1) hi1 = lo1;
+    };
+    if (!ok && t < t1) {  // a segment the index rejected: only the next unit's first words
+      int64_t hi1;
+      next_segment(hi1);
+      nx = load_pass_words(p, floor2(lo1), lo1, hi1, lane);
+    }
+    while (more) {
+      const PassWords cw = nx;
+      uint32_t n0 = cw.n & 0xffu, n1 = cw.n >> 8;
+      const uint32_t gap = n0, tot = n0 + n1;
+      uint32_t x = tot;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= (uint32_t)o) x += y;
+      }
+      const int32_t after = fill + (int32_t)__shfl_sync(0xffffffffu, x, 31);
+      const int32_t p0 = fill + (int32_t)(x - tot);  // place of the lane's first symbol
+      // symbols from the stage's front to the unit's end (clipped: a pass adds 4096 at most)
+      const int32_t rem = (int32_t)((left < 65536u ? left : 65536u) * E);
+      const int64_t hi = (int64_t)(sg.word_offset + sg.n_words);
+      base += kPassWords;
+      const int32_t upto = after < rem ? after : rem;  // symbols this pass completes, less where the stage is too small
+      const bool last = (after >= rem || base >= hi) && upto <= CAP;
+      int64_t hi1 = 0;
+      if (last) {
+        // words that start at or after the unit's end are not decoded
+        if (p0 >= rem) n0 = 0u;
+        if (p0 + (int32_t)gap >= rem) n1 = 0u;
+        if (t < t1) next_segment(hi1);
+        fill = upto;  // (an inconsistent stream can run out of words before its end)
+      } else if (after > CAP) {
+        // the words that fit; the next pass starts behind them
+        const bool a0 = p0 + (int32_t)gap <= CAP, a1 = p0 + (int32_t)tot <= CAP;
+        const uint32_t m0 = __ballot_sync(0xffffffffu, a0), m1 = __ballot_sync(0xffffffffu, a1);
+        const uint32_t words = (uint32_t)(__popc(m0) + __popc(m1));
+        fill = (int32_t)__shfl_sync(0xffffffffu, (uint32_t)(p0 + (int32_t)(words & 1u ? gap : tot)), (words - 1) >> 1);
+        if (!a0) n0 = 0u;
+        if (!a1) n1 = 0u;
+        const int64_t lo = base - kPassWords + words;
+        base = floor2(lo);
+        nx = load_pass_words(p, base, lo, hi, lane);
+      } else {
+        fill = after;
+        nx = load_pass_words(p, base, base, hi, lane);
+      }
+      bad |= decode_pair(cw, n0, n1, gap, stage + p0, reinterpret_cast<const uint16_t *>(smem + dd.lut_off), dd);
+      if (last && t < t1) nx = load_pass_words(p, floor2(lo1), lo1, hi1, lane);
+      __syncwarp();
+      // ---- the steps that are complete
+      int32_t off = 0;
+      const int32_t need = (int32_t)(sw * E);
+      while (fill - off >= need || (last && off < fill)) {
+        const uint32_t n = left < sw ? left : sw;
+        step(sg, dd, stage + off, win, n);
+        win += n;
+        left -= n;
+        off += need;
+      }
+      more = !last;
+      if (more && off) {  // the symbols left, to the front
+        const int32_t r = fill - off;
+        for (int32_t i = 0; i < r; i += 512) {
+          uint4 v;
+          const int32_t at = i + 16 * (int32_t)lane;
+          if (at < r) v = *reinterpret_cast<const uint4 *>(stage + off + at);
+          __syncwarp();
+          if (at < r) *reinterpret_cast<uint4 *>(stage + at) = v;
+        }
+        fill = r;
+      }
+      __syncwarp();
+    }
+    bad = __reduce_or_sync(0xffffffffu, bad);
+    if (bad && lane == 0) flag_bad(p.status, bad, sg.caller_index);
+    if (t >= t1) break;
+    s = s1;
+    ok = ok1;
+    base = floor2(lo1);
+    fill = 0;
   }
 }
 
