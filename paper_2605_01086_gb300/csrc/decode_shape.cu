@@ -525,6 +525,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_decode_shape(const DecodePara
   unsigned char *const otile = reinterpret_cast<unsigned char *>(tiles0) + warp * TILES * kOutTile;
   const bool want_lev = p.levels != nullptr;
 
+  dependency_wait();  // the index: from here on its outputs are read
   uint64_t tw0, tw1;
   unit_tiles(p, (uint64_t)blockIdx.x * WARPS + warp, (uint64_t)gridDim.x * WARPS, tw0, tw1);
   if (tw0 >= tw1) return;
@@ -669,7 +670,7 @@ cudaError_t launch_shape(const DecodeParams &p, const WarpParams &wp, const Shap
   WarpParams ww = wp;
   ShapeMaps mm = maps;
   void *args[] = {&pp, &ww, &mm};
-  return cudaLaunchKernel(k, dim3(grid), dim3(threads), args, smem, stream);
+  return launch_after(k, grid, threads, args, smem, stream, p.after_index != 0);
 }
 
 }  // namespace fptc

@@ -101,7 +101,8 @@ __global__ void __launch_bounds__(NWG * 128, 1) k_decode_tc(const DecodeParams p
     rounds = b - a > rounds ? b - a : rounds;
   }
 
-  uint32_t s = find_segment(p.segs, p.seg_begin, p.seg_end, t0 < t1 ? t0 : p.tile_begin);
+  dependency_wait();  // the index: from here on its outputs are read
+  uint32_t s = warp_find_segment(p.segs, p.seg_begin, p.seg_end, t0 < t1 ? t0 : p.tile_begin, lane);
   uint32_t pn = 0;
   Ctx nxt{0, 0, 0, s, 0};
   if (t0 < t1) {  // where tile t0 starts, then its first words
@@ -371,7 +372,7 @@ cudaError_t launch_tc(const DecodeParams &p, const WarpParams &wp, const TcParam
   TcParams tt = tp;
   CUtensorMap mm = out_map;
   void *args[] = {&pp, &ww, &tt, &mm};
-  return cudaLaunchKernel(k, dim3(grid), dim3(threads), args, smem, stream);
+  return launch_after(k, grid, threads, args, smem, stream, p.after_index != 0);
 }
 
 }  // namespace fptc

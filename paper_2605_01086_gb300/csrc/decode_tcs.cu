@@ -227,7 +227,8 @@ __global__ void __launch_bounds__(tcs_nwg<MODE, N, E>() * 128, 1)
     rounds = b - a > rounds ? b - a : rounds;
   }
 
-  uint32_t s = find_segment(p.segs, p.seg_begin, p.seg_end, t0 < t1 ? t0 : p.tile_begin);
+  dependency_wait();  // the index: from here on its outputs are read
+  uint32_t s = warp_find_segment(p.segs, p.seg_begin, p.seg_end, t0 < t1 ? t0 : p.tile_begin, lane);
   uint32_t pn = 0;
   Ctx nxt{0, 0, 0, s, 0};
   if (t0 < t1) {
@@ -560,7 +561,7 @@ cudaError_t launch_tcs(const DecodeParams &p, const WarpParams &wp, const TcPara
   TcParams tt = tp;
   CUtensorMap mm = out_map;
   void *args[] = {&pp, &ww, &tt, &mm};
-  return cudaLaunchKernel(k, dim3(grid), dim3(tcs_threads(mode, N, E)), args, smem, stream);
+  return launch_after(k, grid, tcs_threads(mode, N, E), args, smem, stream, p.after_index != 0);
 }
 
 }  // namespace fptc

@@ -163,6 +163,7 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS > 16 ? 1 : 32 / WARPS) k_dec
   const bool out32 = (reinterpret_cast<uintptr_t>(p.out) & 31u) == 0;
 
   // ---- this warp's tiles: an even split of the launch's tile range over all warps
+  dependency_wait();  // the index: from here on its outputs are read
   uint64_t tw0, tw1;
   unit_tiles(p, (uint64_t)blockIdx.x * WARPS + warp, (uint64_t)gridDim.x * WARPS, tw0, tw1);
   if (tw0 >= tw1) return;
@@ -283,7 +284,7 @@ cudaError_t launch_warp(const DecodeParams &p, const WarpParams &wp, const CUten
   WarpParams ww = wp;
   CUtensorMap mm = out_map;
   void *args[] = {&pp, &ww, &mm};
-  return cudaLaunchKernel(k, dim3(grid), dim3(threads), args, smem, stream);
+  return launch_after(k, grid, threads, args, smem, stream, p.after_index != 0);
 }
 
 }  // namespace fptc

@@ -137,6 +137,32 @@ __device__ __forceinline__ void load_deq(float *s_deq, const DomainDev &dm, cons
   }
 }
 
+// Waits until the kernel this one was allowed to overlap has ended and its
+// writes are visible (returns at once for an ordinary launch).
+__device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the kernel behind this one start its CTAs as SMs become free.
+__device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// cudaLaunchKernel, or, with overlap, a launch that may begin before the kernel
+// in front of it in the stream has ended: that must be a kernel of this library
+// which itself began after everything before it, and the launched kernel calls
+// dependency_wait before it touches anything but the plan's own tables.
+inline cudaError_t launch_after(const void *kernel, uint32_t grid, uint32_t threads, void **args, size_t smem,
+                                cudaStream_t stream, bool overlap) {
+  if (!overlap) return cudaLaunchKernel(kernel, dim3(grid), dim3(threads), args, smem, stream);
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, kernel, args);
+}
+
 __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
 // The dynamic shared-memory limit is a per-kernel attribute shared by every plan

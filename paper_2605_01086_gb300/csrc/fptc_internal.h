@@ -20,6 +20,10 @@ namespace fptc {
 constexpr uint32_t kChunkWords = 496;
 // Chunks of a segment of n words for any placement of its first byte.
 __host__ __device__ constexpr uint64_t chunks_of(uint64_t n) { return n ? ((n + 15) / 16 + 1 + 30) / 31 : 0; }
+// Chunks a warp of the index kernel takes at once (a group; groups do not cross
+// segments).
+constexpr uint32_t kGroupChunks = 8;
+__host__ __device__ constexpr uint64_t groups_of(uint64_t chunks) { return (chunks + kGroupChunks - 1) / kGroupChunks; }
 constexpr uint32_t kMaxLmax = 16;
 constexpr uint32_t kChunkBad = 0xFFFFFFFFu;  // chunk sum sentinel: a symlen > 64 was seen
 
@@ -73,6 +77,7 @@ struct SegDev {
   uint64_t tile_base;    // global index of the segment's first tile
   uint64_t n_tiles;
   uint64_t chunk_base;   // global index of the segment's first index chunk
+  uint64_t group_base;   // and of its first group of chunks
   uint32_t n_chunks;
   uint32_t domain;
   uint32_t caller_index; // position in the caller's segment array
@@ -93,6 +98,12 @@ struct DevStatus {
   unsigned long long first_bad;  // smallest caller index of a bad segment
 };
 
+// A group of index chunks: its segment (queue index) and first chunk in it.
+struct IndexGroup {
+  uint32_t seg;
+  uint32_t chunk;
+};
+
 struct IndexParams {
   const uint8_t *symlen;
   const SegDev *segs;
@@ -102,6 +113,9 @@ struct IndexParams {
   uint32_t *seg_bad;
   TileRec *tiles;
   DevStatus *status;
+  const IndexGroup *groups;         // the groups, or null: found by a search over group_base
+  uint32_t *done;                   // per segment: its groups that are counted (0 between calls)
+  uint64_t group_begin, group_end;  // group range of this launch
   uint64_t chunk_begin, chunk_end;  // chunk range of this launch
   uint32_t seg_begin, seg_end;      // segment range of this launch
   uint32_t grid;                    // CTAs of the chunk kernels (0: a default)
@@ -126,6 +140,7 @@ struct DecodeParams {
   uint32_t seg_begin, seg_end;    // segment range covering it
   uint32_t lut_cap;               // decode-table entries that fit the shared buffer
   uint32_t coef_cap;              // tile_windows * E capacity of the shared tile buffers
+  uint32_t after_index;           // launched right behind the index kernel: may start before it ends (launch_after)
 };
 
 // Shared-memory layout of the warp-tile kernel (decode_warp.cu).

@@ -1,23 +1,27 @@
 // SymLen segment indexing (Sec. 4.2.1: an exclusive prefix sum over the symlen
 // array gives every compressed word the output position of its first symbol).
 //
-// Three kernels, none of which waits on another CTA:
-//   1. chunk_count: per chunk of kChunkWords words, the sum of symlen (and a
-//      check that no symlen exceeds 64);
-//   2. segment_scan: one warp per segment scans its chunk sums into chunk
-//      offsets and checks the segment total against W*E;
-//   3. tile_index: per chunk, a warp scan gives every word's symbol offset;
+//   1. k_index: a warp per group of 8 chunks of a segment sums each chunk's
+//      symlen (and checks that none exceeds 64); the warp that counts a
+//      segment's last group scans the segment's chunk sums into chunk offsets
+//      and checks the total against W*E.  No CTA waits on another: the last
+//      group is whichever comes last (a counter per segment, which wraps to 0).
+//   2. k_tile_index: per chunk, a warp scan gives every word's symbol offset;
 //      every word that holds the first symbol of a tile (tile = tile_windows
 //      windows = tile_windows * E symbols) writes (word, symbols to skip).
 // The decode kernels then start each tile without decoding earlier words.
 //
-// Kernels 1 and 3 run one warp per chunk over a contiguous chunk range per
-// warp (the segment cursor advances with the chunk index, so no per-chunk
-// table is read), with the next chunks' blocks loaded while the current ones
-// are reduced; the chunk geometry is that of symlen_chunks.cuh.  Kernel 3 runs
-// only for the kernels that read a record per tile: the warp-tile kernels
-// locate the first tile of their range from the chunk offsets
-// (symbol_word) and every later one from the tile decoded before it.
+// A few MB are read, so k_index is bound by the dependent loads of a warp:
+// group, segment, symlen (eight chunks at once).  Two kernels, one finding its
+// segment by a binary search, took 16 us for the 13 M words of a mixed batch and
+// 23 us for 16,384 streams of 370 words; this one 8 and 15 us, and the decode
+// kernel behind it loads its tables meanwhile (launch_after).
+// k_tile_index runs one warp per chunk over a contiguous chunk range per warp
+// (the segment cursor advances with the chunk index), with the next chunks'
+// blocks loaded while the current ones are reduced, and only for the kernels
+// that read a record per tile: the warp-tile kernels locate the first word of
+// their range from the chunk offsets (symbol_word).  The chunk geometry is that
+// of symlen_chunks.cuh.
 #include "symlen_chunks.cuh"
 
 namespace fptc {
@@ -44,10 +48,6 @@ __device__ __forceinline__ void warp_chunks(const IndexParams &p, uint64_t &c0, 
   c1 = p.chunk_begin + n * (gw + 1) / nw;
 }
 
-// Chunks in flight per warp: the loads of the next group of chunks are issued
-// before the current group is reduced (four for the chunk sums, two for the
-// tile index, whose group holds more state).
-
 // Symlen blocks of chunks c .. c + P - 1 (clipped to c1) with their segments;
 // the segment cursor s advances monotonically.
 template <int P>
@@ -70,61 +70,106 @@ __device__ __forceinline__ void load_group(const IndexParams &p, uint64_t c, uin
   }
 }
 
-__global__ void __launch_bounds__(256, 4) k_chunk_count(IndexParams p) {
-  const uint32_t lane = threadIdx.x & 31;
-  uint64_t c0, c1;
-  warp_chunks(p, c0, c1);
-  if (c0 >= c1) return;
-  uint32_t s = chunk_segment(p.segs, p.seg_begin, p.seg_end, c0);
-  constexpr int kPipe = 4;
-  ChunkGroup<kPipe> cur;
-  load_group(p, c0, c1, lane, s, cur);
-  for (uint64_t c = c0; c < c1; c += kPipe) {
-    ChunkGroup<kPipe> nxt;
-    load_group(p, c + kPipe, c1, lane, s, nxt);
-#pragma unroll
-    for (int i = 0; i < kPipe; ++i) {
-      if (c + i >= c1) break;
-      const uint32_t sum = __reduce_add_sync(0xffffffffu, block_sum(cur.v[i]));
-      const uint32_t bad = __reduce_or_sync(0xffffffffu, block_over64(cur.v[i]) ? 1u : 0u);
-      if (lane == 0) p.chunk_sum[c + i] = bad ? kChunkBad : sum;
-    }
-    cur = nxt;
-  }
-}
-
-// one warp per segment
-__global__ void __launch_bounds__(256) k_segment_scan(IndexParams p) {
-  const uint32_t lane = threadIdx.x & 31;
-  const uint64_t s = (uint64_t)p.seg_begin + (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) / 32;
-  if (s >= p.seg_end) return;
-  const SegDev sg = p.segs[s];
-  uint64_t run = 0;
-  bool range_bad = false;
-  for (uint32_t j0 = 0; j0 < sg.n_chunks; j0 += 32) {
-    const uint32_t j = j0 + lane;
-    uint32_t v = j < sg.n_chunks ? p.chunk_sum[sg.chunk_base + j] : 0u;
-    if (v == kChunkBad) {
-      range_bad = true;
-      v = 0;
-    }
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= (uint32_t)o) x += y;
-    }
-    if (j < sg.n_chunks) p.chunk_off[sg.chunk_base + j] = run + x - v;
-    run += __shfl_sync(0xffffffffu, x, 31);
-  }
-  range_bad = __any_sync(0xffffffffu, range_bad);
-  const uint64_t expect = sg.n_windows * (uint64_t)p.domains[sg.domain].E;
-  const bool count_bad = run != expect;
+// The segment's symbol total against what its windows need, and whether a word
+// claims more than 64 symbols: its flag and the plan's status.
+__device__ __forceinline__ void close_segment(const IndexParams &p, uint32_t s, const SegDev &sg, uint64_t total,
+                                              bool range_bad, uint32_t lane) {
+  const bool count_bad = total != sg.n_windows * (uint64_t)p.domains[sg.domain].E;
   if (lane == 0) {
     p.seg_bad[s] = (range_bad || count_bad) ? 1u : 0u;
     if (range_bad) flag_bad(p.status, kFlagSymlenRange, sg.caller_index);
     if (count_bad) flag_bad(p.status, kFlagSymbolCount, sg.caller_index);
   }
+}
+
+// Inclusive warp scan.
+__device__ __forceinline__ uint32_t scan32(uint32_t x, uint32_t lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= (uint32_t)o) x += y;
+  }
+  return x;
+}
+
+__global__ void __launch_bounds__(256) k_index(IndexParams p) {
+  dependents_may_start();
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t g = p.group_begin + (uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (g >= p.group_end) return;  // the whole warp
+  uint32_t s, c0;
+  if (p.groups) {
+    const IndexGroup r = p.groups[g];
+    s = r.seg;
+    c0 = r.chunk;
+  } else {
+    const uint32_t b = p.seg_begin;
+    s = b + (uint32_t)warp_last_leq(p.seg_end - b, g, lane, [&](uint64_t i) { return p.segs[b + i].group_base; });
+    c0 = (uint32_t)(g - p.segs[s].group_base) * kGroupChunks;
+  }
+  const SegDev &sg = p.segs[s];
+  const uint32_t n_chunks = sg.n_chunks, n = n_chunks - c0 < kGroupChunks ? n_chunks - c0 : kGroupChunks;
+  uint4 v[kGroupChunks];
+#pragma unroll
+  for (uint32_t i = 0; i < kGroupChunks; ++i)
+    v[i] = i < n ? load_block(p.symlen, sg, c0 + i, lane).v : make_uint4(0u, 0u, 0u, 0u);
+  uint32_t sum = 0u, over = 0u;  // lane i: chunk i's sum and whether a word of it claims more than 64
+#pragma unroll
+  for (uint32_t i = 0; i < kGroupChunks; ++i) {
+    const uint32_t x = __reduce_add_sync(0xffffffffu, block_sum(v[i]));
+    const bool o = __any_sync(0xffffffffu, block_over64(v[i]));
+    if (lane == i) {
+      sum = x;
+      over = o ? 1u : 0u;
+    }
+  }
+  if (n_chunks <= kGroupChunks) {  // the whole segment
+    const uint32_t incl = scan32(sum, lane);
+    if (lane < n) p.chunk_off[sg.chunk_base + lane] = incl - sum;
+    close_segment(p, s, sg, __shfl_sync(0xffffffffu, incl, 31), __any_sync(0xffffffffu, over != 0u), lane);
+    return;
+  }
+  if (lane < n) __stcg(p.chunk_sum + sg.chunk_base + c0 + lane, over ? kChunkBad : sum);
+  __threadfence();
+  __syncwarp();
+  const uint32_t groups = (uint32_t)groups_of(n_chunks);
+  uint32_t before = 0u;
+  if (lane == 0) before = atomicInc(p.done + s, groups - 1u);
+  if (__shfl_sync(0xffffffffu, before, 0) != groups - 1u) return;
+  __threadfence();
+  // ---- the segment's last group: every chunk sum is there.  Four a lane and
+  // round, the next round's in flight
+  uint64_t run = 0;
+  bool range_bad = false;
+  uint32_t nx[4];
+  auto fetch = [&](uint32_t j0) {
+#pragma unroll
+    for (uint32_t q = 0; q < 4; ++q) {
+      const uint32_t j = j0 + 4 * lane + q;
+      nx[q] = j < n_chunks ? __ldcg(p.chunk_sum + sg.chunk_base + j) : 0u;
+    }
+  };
+  fetch(0);
+  for (uint32_t j0 = 0; j0 < n_chunks; j0 += 128) {
+    uint32_t c[4];
+#pragma unroll
+    for (uint32_t q = 0; q < 4; ++q) {
+      range_bad = range_bad || nx[q] == kChunkBad;
+      c[q] = nx[q] == kChunkBad ? 0u : nx[q];
+    }
+    if (n_chunks - j0 > 128) fetch(j0 + 128);
+    const uint32_t tot = c[0] + c[1] + c[2] + c[3];
+    const uint32_t incl = scan32(tot, lane);
+    uint64_t off = run + (incl - tot);
+#pragma unroll
+    for (uint32_t q = 0; q < 4; ++q) {
+      const uint32_t j = j0 + 4 * lane + q;
+      if (j < n_chunks) p.chunk_off[sg.chunk_base + j] = off;
+      off += c[q];
+    }
+    run += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  close_segment(p, s, sg, run, __any_sync(0xffffffffu, range_bad), lane);
 }
 
 __global__ void __launch_bounds__(256, 3) k_tile_index(IndexParams p) {
@@ -231,16 +276,13 @@ __global__ void __launch_bounds__(256) k_word_offsets(IndexParams p, uint32_t *w
 }  // namespace
 
 cudaError_t launch_index(const IndexParams &p, cudaStream_t stream) {
-  const uint64_t n_chunks = p.chunk_end - p.chunk_begin;
-  const uint32_t n_segs = p.seg_end - p.seg_begin;
-  if (n_segs == 0) return cudaSuccess;
+  const uint64_t n_chunks = p.chunk_end - p.chunk_begin, n_groups = p.group_end - p.group_begin;
+  if (p.seg_end <= p.seg_begin || n_groups == 0) return cudaSuccess;
+  k_index<<<(unsigned)((n_groups + 7) / 8), 256, 0, stream>>>(p);
   // persistent warps over the chunks: at most one chunk per warp, at most p.grid CTAs of 8 warps
   const uint64_t want = (n_chunks + 7) / 8;
   const uint32_t grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(p.grid ? p.grid : 1024u, want));
-  if (n_chunks > 0) k_chunk_count<<<grid, 256, 0, stream>>>(p);
-  const uint64_t warps_threads = (uint64_t)n_segs * 32;
-  k_segment_scan<<<(unsigned)((warps_threads + 255) / 256), 256, 0, stream>>>(p);
-  if (n_chunks > 0 && p.records) k_tile_index<<<grid, 256, 0, stream>>>(p);
+  if (p.records) k_tile_index<<<grid, 256, 0, stream>>>(p);
   return cudaGetLastError();
 }
 

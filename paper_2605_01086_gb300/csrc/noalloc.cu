@@ -32,7 +32,8 @@ constexpr uint32_t kNaMaxLmax = 12;                              // decode table
 constexpr size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 constexpr size_t kOffStatus = 0;
 constexpr size_t kOffSegBad = a256(kOffStatus + sizeof(DevStatus));
-constexpr size_t kOffSeg = a256(kOffSegBad + sizeof(uint32_t));
+constexpr size_t kOffDone = a256(kOffSegBad + sizeof(uint32_t));
+constexpr size_t kOffSeg = a256(kOffDone + sizeof(uint32_t));
 constexpr size_t kOffDom = a256(kOffSeg + sizeof(SegDev));
 constexpr size_t kOffLut = a256(kOffDom + sizeof(DomainDev));
 constexpr size_t kOffBasis = a256(kOffLut + (size_t(2) << kNaMaxLmax));
@@ -65,6 +66,7 @@ __global__ void k_na_setup(const __grid_constant__ NaSetup a) {
   if (threadIdx.x == 0) {
     *reinterpret_cast<DevStatus *>(scr + kOffStatus) = a.status;
     *reinterpret_cast<uint32_t *>(scr + kOffSegBad) = 0u;
+    *reinterpret_cast<uint32_t *>(scr + kOffDone) = 0u;
     *reinterpret_cast<SegDev *>(scr + kOffSeg) = a.seg;
     *reinterpret_cast<DomainDev *>(scr + kOffDom) = a.dom;
   }
@@ -155,6 +157,7 @@ extern "C" fptc_status fptc_decode_stream_noalloc(const fptc_domain *domain, con
   sg.tile_base = 0;
   sg.n_tiles = (W + dd.tile_windows - 1) / dd.tile_windows;
   sg.chunk_base = 0;
+  sg.group_base = 0;
   sg.n_chunks = (uint32_t)chunks_of(n_words);
   sg.domain = 0;
   sg.caller_index = 0;
@@ -184,6 +187,9 @@ extern "C" fptc_status fptc_decode_stream_noalloc(const fptc_domain *domain, con
   ip.seg_bad = reinterpret_cast<uint32_t *>(scr + kOffSegBad);
   ip.tiles = reinterpret_cast<TileRec *>(scr + kOffTiles);
   ip.status = reinterpret_cast<DevStatus *>(scr + kOffStatus);
+  ip.done = reinterpret_cast<uint32_t *>(scr + kOffDone);
+  ip.group_begin = 0;
+  ip.group_end = groups_of(sg.n_chunks);
   ip.chunk_begin = 0;
   ip.chunk_end = sg.n_chunks;
   ip.seg_begin = 0;

@@ -30,7 +30,7 @@ struct fptc_plan {
   std::vector<SegDev> segs;              // queue order
   std::vector<DomainDev> dom_dev;
   std::vector<uint64_t> level_off;       // caller order
-  uint64_t n_tiles = 0, n_chunks = 0, n_levels = 0;
+  uint64_t n_tiles = 0, n_chunks = 0, n_groups = 0, n_levels = 0;
   uint64_t words_extent = 0, out_extent = 0, n_samples = 0, n_words = 0;
   // device memory owned by the plan
   DomainDev *d_domains = nullptr;
@@ -40,6 +40,8 @@ struct fptc_plan {
   uint32_t *d_chunk_sum = nullptr;
   uint64_t *d_chunk_off = nullptr;
   uint32_t *d_seg_bad = nullptr;
+  IndexGroup *d_groups = nullptr;   // [n_groups]
+  uint32_t *d_done = nullptr;       // per segment: the index kernel's count of its groups (0 between calls)
   uint32_t *d_word_off = nullptr;   // three-kernel schedule: symbol offset of every word
   uint8_t *d_lev_scratch = nullptr; // three-kernel schedule: the level array
   TileRec *d_tiles = nullptr;
@@ -115,6 +117,8 @@ void free_device(fptc_plan *p) {
   cudaFree(p->d_chunk_sum);
   cudaFree(p->d_chunk_off);
   cudaFree(p->d_seg_bad);
+  cudaFree(p->d_groups);
+  cudaFree(p->d_done);
   cudaFree(p->d_word_off);
   cudaFree(p->d_lev_scratch);
   cudaFree(p->d_tiles);
@@ -132,7 +136,7 @@ void free_device(fptc_plan *p) {
 void PlanDeleter::operator()(fptc_plan *p) const {
   if (!p) return;
   if (p->d_domains || p->d_segs || p->d_luts || p->d_basis || p->d_chunk_sum || p->d_chunk_off || p->d_seg_bad ||
-      p->d_word_off || p->d_lev_scratch || p->d_tiles || p->d_status || p->up || p->ev_start || p->aux[0] ||
+      p->d_groups || p->d_done || p->d_word_off || p->d_lev_scratch || p->d_tiles || p->d_status || p->up || p->ev_start || p->aux[0] ||
       p->ev[0] || p->evh[0]) {
     DeviceGuard g(p->device);
     free_device(p);
@@ -415,6 +419,10 @@ IndexParams index_params(const fptc_plan *p, const uint8_t *d_symlen, bool recor
   ip.seg_bad = p->d_seg_bad;
   ip.tiles = p->d_tiles;
   ip.status = p->d_status;
+  ip.groups = p->d_groups;
+  ip.done = p->d_done;
+  ip.group_begin = 0;
+  ip.group_end = p->n_groups;
   ip.chunk_begin = 0;
   ip.chunk_end = p->n_chunks;
   ip.seg_begin = 0;
@@ -463,6 +471,8 @@ cudaError_t run_range(const fptc_plan *p, const IndexParams &ip0, const DecodePa
     IndexParams ip = ip0;
     ip.seg_begin = s0;
     ip.seg_end = s1;
+    ip.group_begin = a.group_base;
+    ip.group_end = b.group_base + groups_of(b.n_chunks);
     ip.chunk_begin = a.chunk_base;
     ip.chunk_end = b.chunk_base + b.n_chunks;
     cudaError_t e = launch_index(ip, st);
@@ -471,6 +481,8 @@ cudaError_t run_range(const fptc_plan *p, const IndexParams &ip0, const DecodePa
   }
   if (!decode) return cudaSuccess;
   DecodeParams dp = dp0;
+  // right behind the index kernel (which began after everything before it): may start beside it
+  dp.after_index = index && !ip0.records && b.group_base + groups_of(b.n_chunks) > a.group_base;
   dp.seg_begin = s0;
   dp.seg_end = s1;
   dp.tile_begin = a.tile_base;
@@ -760,6 +772,7 @@ fptc_status fptc_plan_create(fptc_plan **out, int device, const fptc_domain *dom
     p->n_levels = lv;
     p->segs.resize(n_segments);
     uint64_t chunk = 0;
+    std::vector<IndexGroup> groups;
     for (uint64_t qi = 0; qi < n_segments; ++qi) {
       const uint32_t ci = p->queue[qi];
       const fptc_segment &s = segments[ci];
@@ -779,8 +792,11 @@ fptc_status fptc_plan_create(fptc_plan **out, int device, const fptc_domain *dom
       sd.chunk_base = chunk;
       sd.n_chunks = (uint32_t)chunks_of(s.n_words);
       chunk += sd.n_chunks;
+      sd.group_base = groups.size();
+      for (uint32_t c = 0; c < sd.n_chunks; c += kGroupChunks) groups.push_back(IndexGroup{(uint32_t)qi, c});
     }
     p->n_chunks = chunk;
+    p->n_groups = groups.size();
     layout_tiles(p, o.tile_samples);
 
     // ---- device
@@ -799,7 +815,8 @@ fptc_status fptc_plan_create(fptc_plan **out, int device, const fptc_domain *dom
       size_t b = 0;
       if ((e = upload(&p->d_domains, p->dom_dev, &b)) != cudaSuccess ||
           (e = upload(&p->d_segs, p->segs, &b)) != cudaSuccess ||
-          (e = upload(&p->d_luts, luts, &b)) != cudaSuccess || (e = upload(&p->d_basis, basis, &b)) != cudaSuccess) {
+          (e = upload(&p->d_luts, luts, &b)) != cudaSuccess || (e = upload(&p->d_basis, basis, &b)) != cudaSuccess ||
+          (e = upload(&p->d_groups, groups, &b)) != cudaSuccess) {
         st = cuda_fail(e, "plan upload");
       }
       if (st == FPTC_OK) {
@@ -807,13 +824,15 @@ fptc_status fptc_plan_create(fptc_plan **out, int device, const fptc_domain *dom
         if ((e = cudaMalloc(&p->d_chunk_sum, nc * 4)) != cudaSuccess ||
             (e = cudaMalloc(&p->d_chunk_off, nc * 8)) != cudaSuccess ||
             (e = cudaMalloc(&p->d_seg_bad, ns * 4)) != cudaSuccess ||
+            (e = cudaMalloc(&p->d_done, ns * 4)) != cudaSuccess ||
             (e = cudaMalloc(&p->d_status, sizeof(DevStatus))) != cudaSuccess) {
           st = cuda_fail(e, "plan scratch");
         } else {
-          b += nc * 12 + ns * 4 + sizeof(DevStatus);
+          b += nc * 12 + ns * 8 + sizeof(DevStatus);
           DevStatus s0{0u, 0u, ~0ull};
           e = cudaMemcpy(p->d_status, &s0, sizeof(s0), cudaMemcpyHostToDevice);
           if (e == cudaSuccess) e = cudaMemset(p->d_seg_bad, 0, ns * 4);
+          if (e == cudaSuccess) e = cudaMemset(p->d_done, 0, ns * 4);
           if (e == cudaSuccess && o.schedule == FPTC_SCHEDULE_THREE_KERNEL) {
             e = cudaMalloc(&p->d_word_off, std::max<uint64_t>(p->words_extent, 1) * 4);
             if (e == cudaSuccess) e = cudaMalloc(&p->d_lev_scratch, std::max<uint64_t>(p->n_levels, 1));
@@ -893,10 +912,12 @@ fptc_status fptc_plan_level_offsets(const fptc_plan *p, uint64_t *offsets) {
 uint32_t fptc_plan_launches_per_decode(const fptc_plan *p) {
   if (!p) return 0;
   if (p->segs.empty()) return 0;
-  if (p->opts.schedule == FPTC_SCHEDULE_PERSISTENT) return (p->n_chunks ? 3u : 1u) + 1u;
-  if (p->opts.schedule == FPTC_SCHEDULE_THREE_KERNEL) return (p->n_chunks ? 4u : 1u) + (p->n_chunks ? 2u : 1u);
+  const uint32_t index = needs_records(p) ? 2u : 1u;  // index kernels of a range that has words
+  const uint32_t all = p->n_groups ? index : 0u;
+  if (p->opts.schedule == FPTC_SCHEDULE_PERSISTENT) return all + (p->n_tiles ? 1u : 0u);
+  if (p->opts.schedule == FPTC_SCHEDULE_THREE_KERNEL) return p->n_chunks ? all + 3u : 0u;
   uint32_t n = 0;
-  for (const auto &s : p->segs) n += (s.n_chunks ? 3u : 1u) + 1u;
+  for (const auto &s : p->segs) n += (s.n_chunks ? index : 0u) + (s.n_tiles ? 1u : 0u);
   return n;
 }
 
