@@ -4,7 +4,8 @@
 //   dL/dA_z  = sum over bins k of zone z of g_C[w][k] * unit_z(level[w][k])
 // because the reconstruction of zone z is A_z * unit_z(level) (both the mu-law
 // expander and the deadzone lattice scale linearly with A_z).
-// Per tile: levels come from the saved level buffer or are decoded again
+// Per group of tiles of a segment (one tile of the generic kernel's plans; several
+// of the small tiles of the shape kernel's): levels come from the saved level buffer or are decoded again
 // (same SymLen decode as the forward kernel), g_x is staged in shared memory,
 // one thread per (window, bin) does the N-term FP32 dot product against the
 // transposed basis, products g_C * unit go to an FP32 partial per thread and
@@ -82,11 +83,13 @@ __global__ void __launch_bounds__(THREADS) k_backward(const BackwardParams bp) {
   double acc0 = 0.0, acc1 = 0.0;
   unsigned int err = 0;
 
-  for (uint64_t g = t0; g < t1; ++g) {
+  uint64_t g1 = t0;  // tiles [g, g1) of a segment are taken together
+  for (uint64_t g = t0; g < t1; g = g1) {
     while (g >= p.segs[s].tile_base + p.segs[s].n_tiles) ++s;
-    if (p.seg_bad[s] && bp.levels_in == nullptr) continue;
     const SegDev sg = p.segs[s];
     const DomainDev &dm = p.domains[sg.domain];
+    g1 = min(min(g + dm.group, t1), sg.tile_base + sg.n_tiles);
+    if (p.seg_bad[s] && bp.levels_in == nullptr) continue;
     const uint32_t N = dm.N, E = dm.E, B1 = dm.B1, B2 = dm.B2, lmax = dm.lmax;
     if (sg.domain != cur_dom) {
       if (cur_dom != 0xFFFFFFFFu) {
@@ -116,7 +119,8 @@ __global__ void __launch_bounds__(THREADS) k_backward(const BackwardParams bp) {
     const uint64_t tin = g - sg.tile_base;
     const uint64_t win0 = tin * dm.tile_windows;
     const uint64_t left = sg.n_windows - win0;
-    const uint32_t nwin = left < dm.tile_windows ? (uint32_t)left : dm.tile_windows;
+    const uint32_t most = (uint32_t)(g1 - g) * dm.tile_windows;
+    const uint32_t nwin = left < most ? (uint32_t)left : most;
     const uint32_t tsyms = nwin * E;
 
     // levels of the tile
@@ -126,8 +130,8 @@ __global__ void __launch_bounds__(THREADS) k_backward(const BackwardParams bp) {
     } else {
       const TileRec tr = p.tiles[g];
       uint64_t lw;
-      if (tin + 1 < sg.n_tiles) {
-        const TileRec nx = p.tiles[g + 1];
+      if (g1 < sg.tile_base + sg.n_tiles) {
+        const TileRec nx = p.tiles[g1];
         lw = nx.first_word - (nx.skip == 0 ? 1u : 0u);
       } else {
         lw = sg.word_offset + sg.n_words - 1;

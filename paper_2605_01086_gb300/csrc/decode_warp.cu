@@ -131,7 +131,7 @@ __device__ __forceinline__ void idct32(const float (&c)[16], Put put) {
 
 // Symbols a warp's stage holds: a step's and a pass's (usually 600), and up to
 // the bytes a warp has beside its output tile in the other warp-tile kernels.
-constexpr int kCap = kMiscBytes - 2 * kStreamGuard;
+constexpr int kCap = kMiscBytes - stream_bytes(0);
 constexpr uint32_t kTileWin = 32;  // windows per tile: one step
 
 struct GeoW {
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS > 16 ? 1 : 32 / WARPS) k_dec
   load_domain_tables<WARPS * 32>(p, wp.n_domains, smem_raw);
   __syncthreads();
 
-  uint8_t *const stage = smem_raw + wp.warp_off + warp * stream_bytes(kCap) + kStreamGuard;
+  uint8_t *const stage = smem_raw + wp.warp_off + warp * stream_bytes(kCap) + kStreamStage;
   // output staging tile: 1024-byte aligned (the period of the 128-byte swizzle)
   const uintptr_t tiles0 =
       (reinterpret_cast<uintptr_t>(smem_raw + wp.warp_off + WARPS * stream_bytes(kCap)) + 1023) & ~uintptr_t(1023);
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS > 16 ? 1 : 32 / WARPS) k_dec
   stream_tiles<kCap>(
       p, tw0, tw1, dw, smem_raw, stage, lane, GeoW{},
       // dequantization + inverse transform + reassembly, one window per lane
-      [&](const SegDev &sg, const DomW &dd, const uint8_t *levels, uint64_t win, uint32_t n) {
+      [&](const UnitSeg &sg, const DomW &dd, const uint8_t *levels, uint64_t win, uint32_t n) {
         const float *deq = reinterpret_cast<const float *>(smem_raw + dd.deq_off);
         const uint32_t aligned = sg.out_aligned;
         const uint64_t s0 = win * kN, S = sg.n_samples;  // the step's first sample

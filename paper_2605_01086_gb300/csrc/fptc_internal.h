@@ -39,6 +39,7 @@ struct DomainDev {
   uint32_t N, E, B1, B2;
   uint32_t lmax;
   uint32_t tile_windows;   // windows per tile
+  uint32_t group;          // tiles the block adjoint takes together
   uint32_t lut_offset;     // first entry of this domain's decode table
   uint32_t basis_offset;   // first float of this domain's E x N inverse-transform basis
   float scale[3];          // the plan's A_0, A_1, A_2 rounded to float
@@ -231,17 +232,22 @@ cudaError_t launch_tcs(const DecodeParams &p, const WarpParams &wp, const TcPara
                        uint32_t mode, uint32_t N, uint32_t E, uint32_t grid, size_t smem, cudaStream_t stream);
 
 // warp-tile kernel for other shapes: N in [4, 128] for every domain (several N
-// in one plan), any E <= N (decode_shape.cu); tiles of shape_windows_per_tile(N,
-// E) windows; forms: the OR of what its domains' transforms are at this thread
-// count (kz = min(E, B2)), which picks the kernel instance
+// in one plan), any E <= N (decode_shape.cu); tiles of whole steps of
+// shape_step_windows windows.  tiles: output tiles per warp (two, or one where two do not fit the
+// shared memory or with 24 warps); forms: the OR of what its domains' transforms
+// then are (kz = min(E, B2)), which picks the kernel instance
 constexpr uint32_t kShapeCompiled = 1, kShapeAny = 2;
 bool shape_supported(uint32_t N);
-uint32_t shape_forms(uint32_t N, uint32_t kz, uint32_t threads);
-uint32_t shape_windows_per_tile(uint32_t N, uint32_t E);
-size_t shape_smem_layout(uint32_t threads, const uint32_t *lmax, const uint32_t *N, const uint32_t *E,
-                         const uint32_t *kz, uint32_t n_domains, WarpParams *wp);
-cudaError_t shape_smem_config(uint32_t threads, uint32_t forms, size_t smem);
-cudaError_t shape_occupancy(uint32_t threads, uint32_t forms, size_t smem, int *ctas_per_sm);
+uint32_t shape_forms(uint32_t N, uint32_t kz, uint32_t tiles);
+// The compiled transform of a domain (0: none); where all domains have the same
+// one, forms carries it above bit 8.
+uint32_t shape_one_form(uint32_t N, uint32_t kz, uint32_t tiles);
+void *shape_kernel_one(uint32_t form);  // decode_shape_one.cu
+uint32_t shape_step_windows(uint32_t N, uint32_t E, uint32_t kz, uint32_t tiles);
+size_t shape_smem_layout(uint32_t threads, uint32_t tiles, const uint32_t *lmax, const uint32_t *N, const uint32_t *kz,
+                         uint32_t n_domains, WarpParams *wp);
+cudaError_t shape_smem_config(uint32_t threads, uint32_t tiles, uint32_t forms, size_t smem);
+cudaError_t shape_occupancy(uint32_t threads, uint32_t tiles, uint32_t forms, size_t smem, int *ctas_per_sm);
 // The output's tensor maps: rows of 32 floats (WarpParams out_tma bit 0), and
 // windows x chunks x 32 floats for N = 64 (bit 1) and N = 128 (bit 2).
 struct ShapeMaps {
@@ -249,7 +255,7 @@ struct ShapeMaps {
 };
 bool encode_window_map(CUtensorMap *map, float *out, uint64_t extent, uint32_t N);
 cudaError_t launch_shape(const DecodeParams &p, const WarpParams &wp, const ShapeMaps &maps, uint32_t threads,
-                         uint32_t forms, uint32_t grid, size_t smem, cudaStream_t stream);
+                         uint32_t tiles, uint32_t forms, uint32_t grid, size_t smem, cudaStream_t stream);
 
 // adjoint for N = 32, E = 16 plans on the warp-tile machinery (backward_warp.cu)
 size_t backward_warp_smem_layout(uint32_t threads, const uint32_t *lmax, uint32_t n_domains, WarpParams *wp);

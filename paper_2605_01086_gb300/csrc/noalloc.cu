@@ -143,6 +143,7 @@ extern "C" fptc_status fptc_decode_stream_noalloc(const fptc_domain *domain, con
   DomainDev &dd = a.dom;
   fill_domain_dev(dm, &dd);  // the plan's own per-domain record
   dd.tile_windows = std::max<uint32_t>(1u, kNaTileSamples / dm.N);
+  dd.group = 1;
   dd.lut_offset = 0;
   dd.basis_offset = 0;
   a.lut_entries = 1u << dm.lmax;

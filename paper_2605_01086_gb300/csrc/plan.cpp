@@ -53,6 +53,7 @@ struct fptc_plan {
   bool shape = false;     // every domain has N in [4, 128] and the warp-tile kernel of
                           // decode_shape.cu serves the plan (N = 32, E = 16 plans use decode_warp.cu)
   uint32_t tcs_N = 0, tcs_E = 0;  // the tensor-core kernel of decode_tcs.cu serves this shape (0: decode_tc.cu)
+  uint32_t shape_threads = 0, shape_tiles = 0;  // and its threads and output tiles per warp
   uint32_t shape_forms = 0; // transforms its domains use (kShapeCompiled, kShapeAny): the kernel instance
   WarpParams wp{};
   TcParams tp{};
@@ -180,15 +181,75 @@ void fptc::fill_domain_dev(const fptc_domain &dm, DomainDev *dd) {
 
 namespace {
 
+// Threads and output tiles per warp of the shape kernel: the requested threads
+// with two tiles if they fit, else one; by default 16 warps with two tiles (64
+// and 128-sample windows are only compiled for two) where the domains have one
+// transform, 12 where they have several or N = 128, then what fits.
+void choose_shape(fptc_plan *p) {
+  std::vector<uint32_t> lm, ns, kz;
+  bool wide = false;  // a domain whose compiled transform wants two tiles
+  bool mixed = false; // domains of different transforms
+  for (const auto &d : p->domains) {
+    lm.push_back(d.lmax);
+    ns.push_back(d.N);
+    kz.push_back(std::min(d.E, d.B2));
+    wide = wide || shape_forms(d.N, kz.back(), 2) != shape_forms(d.N, kz.back(), 1);
+    mixed = mixed || shape_one_form(d.N, kz.back(), 2) != shape_one_form(ns[0], kz[0], 2);
+  }
+  int optin = 0;
+  if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device) != cudaSuccess) optin = 0;
+  auto fits = [&](uint32_t threads, uint32_t tiles) {
+    WarpParams probe{};
+    return shape_smem_layout(threads, tiles, lm.data(), ns.data(), kz.data(), (uint32_t)lm.size(), &probe) <= (size_t)optin;
+  };
+  if (p->opts.threads) {
+    p->shape_threads = p->opts.threads;
+    p->shape_tiles = (p->opts.threads == 256 || p->opts.threads == 512) && fits(p->opts.threads, 2) ? 2u : 1u;
+    return;
+  }
+  p->shape_threads = 128;  // nothing fits: refused by configure_launch
+  p->shape_tiles = 1;
+  if (shape_one_form(ns[0], kz[0], 2) >> 8 == 128) mixed = true;  // as large a transform as any
+  const uint32_t order[5][2] = {{mixed ? 384u : 512u, 2}, {512, 1}, {256, 2}, {512, 1}, {256, 1}};
+  for (int i = 0; i < 5; ++i) {
+    if (i == 1 && wide) continue;
+    if (!fits(order[i][0], order[i][1])) continue;
+    p->shape_threads = order[i][0];
+    p->shape_tiles = order[i][1];
+    return;
+  }
+}
+
 // Layout of the tile queue for a tile size (target samples per tile).
 void layout_tiles(fptc_plan *p, uint32_t tile_samples) {
   p->coef_cap = 0;
   p->gx_cap = 0;
   const bool shape = p->kind == FPTC_KERNEL_WARP_TILE && p->shape;
+  // the shape kernel splits its work by tiles, so a domain's tile is as many of its
+  // steps as cost about what the dearest step of the plan does (instructions: 14 a
+  // symbol, 10 a sample)
+  auto step_of = [&](const DomainDev &dd) {
+    return shape_step_windows(dd.N, dd.E, std::min(dd.E, dd.B2), p->shape_tiles);
+  };
+  auto step_cost = [&](const DomainDev &dd) { return step_of(dd) * (25u * dd.E + (dd.N == 128 ? 20u : 10u) * dd.N); };
+  uint32_t dearest = 0;
+  if (shape) {
+    choose_shape(p);
+    for (const auto &dd : p->dom_dev) dearest = std::max(dearest, step_cost(dd));
+  }
   for (auto &dd : p->dom_dev) {
-    dd.tile_windows = shape ? shape_windows_per_tile(dd.N, dd.E) : std::max<uint32_t>(1u, tile_samples / dd.N);
-    p->coef_cap = std::max(p->coef_cap, dd.tile_windows * dd.E);
-    p->gx_cap = std::max(p->gx_cap, dd.tile_windows * dd.N);
+    dd.tile_windows = shape ? step_of(dd) * std::max<uint32_t>(1u, std::min<uint32_t>(
+                                                dearest / step_cost(dd),
+                                                std::min(8192u / (step_of(dd) * dd.N), 2048u / (step_of(dd) * dd.E))))
+                            : std::max<uint32_t>(1u, tile_samples / dd.N);
+    // the block adjoint takes up to 8192 samples and 2048 symbols of a segment's tiles together
+    dd.group = 1;
+    if (shape) {
+      const uint32_t T = dd.tile_windows;
+      dd.group = std::max<uint32_t>(1u, std::min<uint32_t>(8192u / (T * dd.N), 2048u / (T * dd.E)));
+    }
+    p->coef_cap = std::max(p->coef_cap, dd.tile_windows * dd.group * dd.E);
+    p->gx_cap = std::max(p->gx_cap, dd.tile_windows * dd.group * dd.N);
   }
   uint64_t t = 0;
   for (auto &s : p->segs) {
@@ -216,39 +277,32 @@ fptc_status smem_fits(const char *kernel, uint32_t threads, size_t smem) {
 fptc_status configure_launch(fptc_plan *p) {
   uint32_t threads = p->opts.threads ? p->opts.threads : (p->kind == FPTC_KERNEL_TENSOR ? 512u : 256u);
   const bool shape = p->kind == FPTC_KERNEL_WARP_TILE && p->shape;
-  std::vector<uint32_t> lm, ns, es, kz;
+  std::vector<uint32_t> lm, ns, kz;
   for (const auto &d : p->domains) {
     lm.push_back(d.lmax);
     ns.push_back(d.N);
-    es.push_back(d.E);
     kz.push_back(std::min(d.E, d.B2));
   }
   if (p->kind == FPTC_KERNEL_WARP_TILE && p->opts.threads == 0) {
-    // as many warps per SM as one CTA's shared memory allows (32 at most; 16
-    // for other shapes, whose transform wants more registers per thread)
+    // as many warps per SM as one CTA's shared memory allows (32 at most)
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     WarpParams probe{};
     threads = 128;
-    if (shape) {
-      for (uint32_t t : {512u, 256u})
-        if (shape_smem_layout(t, lm.data(), ns.data(), es.data(), kz.data(), (uint32_t)lm.size(), &probe) <= (size_t)optin) {
-          threads = t;
-          break;
-        }
-    } else {
+    if (!shape)
       // 896 before 1024: 28 warps run without spills (72 registers), 32 would spill at 64
       for (uint32_t t : {896u, 1024u, 768u, 512u, 256u})
         if (warp_smem_layout(t, lm.data(), (uint32_t)lm.size(), &probe) <= (size_t)optin) {
           threads = t;
           break;
         }
-    }
   }
+  if (shape) threads = p->shape_threads;
   if (p->kind == FPTC_KERNEL_TENSOR && p->tcs_N) threads = tcs_threads(p->opts.idct, p->tcs_N, p->tcs_E);
   const bool t_ok = (p->kind == FPTC_KERNEL_TENSOR && p->tcs_N) ? threads > 0
-                    : shape ? (threads == 256 || threads == 512 || threads == 768)
+                    : shape ? (threads == 256 || threads == 512 || threads == 768 ||
+                               (threads == 384 && p->opts.threads == 0))
                           : (threads == 128 || threads == 256 || threads == 512 ||
                              ((threads == 768 || threads == 896 || threads == 1024) &&
                               p->kind == FPTC_KERNEL_WARP_TILE) ||
@@ -319,12 +373,17 @@ fptc_status configure_launch(fptc_plan *p) {
     if (e == cudaSuccess) occ = std::min<int>(occ, 1);
   } else if (shape) {
     p->shape_forms = 0;
-    for (size_t d = 0; d < lm.size(); ++d) p->shape_forms |= shape_forms(ns[d], kz[d], threads);
-    p->smem = shape_smem_layout(threads, lm.data(), ns.data(), es.data(), kz.data(), (uint32_t)lm.size(), &p->wp);
+    uint32_t one = shape_one_form(ns[0], kz[0], p->shape_tiles);
+    for (size_t d = 0; d < lm.size(); ++d) {
+      p->shape_forms |= shape_forms(ns[d], kz[d], p->shape_tiles);
+      if (shape_one_form(ns[d], kz[d], p->shape_tiles) != one) one = 0;
+    }
+    p->shape_forms |= one << 8;
+    p->smem = shape_smem_layout(threads, p->shape_tiles, lm.data(), ns.data(), kz.data(), (uint32_t)lm.size(), &p->wp);
     if (const fptc_status fs = smem_fits("warp-tile", threads, p->smem); fs != FPTC_OK) return fs;
-    e = shape_smem_config(threads, p->shape_forms, p->smem);
+    e = shape_smem_config(threads, p->shape_tiles, p->shape_forms, p->smem);
     if (e != cudaSuccess) return cuda_fail(e, "decode shared-memory size");
-    e = shape_occupancy(threads, p->shape_forms, p->smem, &occ);
+    e = shape_occupancy(threads, p->shape_tiles, p->shape_forms, p->smem, &occ);
   } else if (p->kind == FPTC_KERNEL_WARP_TILE) {
     p->smem = warp_smem_layout(threads, lm.data(), (uint32_t)lm.size(), &p->wp);
     if (const fptc_status fs = smem_fits("warp-tile", threads, p->smem); fs != FPTC_OK) return fs;
@@ -506,7 +565,7 @@ cudaError_t run_range(const fptc_plan *p, const IndexParams &ip0, const DecodePa
       }
       if (n64 && encode_window_map(&maps.n64, dp.out, p->out_extent, 64)) wp.out_tma |= 2u;
       if (n128 && encode_window_map(&maps.n128, dp.out, p->out_extent, 128)) wp.out_tma |= 4u;
-      return launch_shape(dp, wp, maps, p->threads, p->shape_forms, grid, p->smem, st);
+      return launch_shape(dp, wp, maps, p->threads, p->shape_tiles, p->shape_forms, grid, p->smem, st);
     }
     CUtensorMap map;
     std::memset(&map, 0, sizeof(map));
@@ -655,13 +714,12 @@ fptc_status fptc_plan_create(fptc_plan **out, int device, const fptc_domain *dom
         if (fixed_ok) {
           fits = warp_smem_layout(128, lm.data(), n_domains, &probe) <= (size_t)optin;
         } else {
-          std::vector<uint32_t> ns(n_domains), es(n_domains), kz(n_domains);
+          std::vector<uint32_t> ns(n_domains), kz(n_domains);
           for (uint32_t d = 0; d < n_domains; ++d) {
             ns[d] = domains[d].N;
-            es[d] = domains[d].E;
             kz[d] = std::min(domains[d].E, domains[d].B2);
           }
-          fits = shape_smem_layout(256, lm.data(), ns.data(), es.data(), kz.data(), n_domains, &probe) <= (size_t)optin;
+          fits = shape_smem_layout(256, 1, lm.data(), ns.data(), kz.data(), n_domains, &probe) <= (size_t)optin;
         }
       }
       o.kernel = fits ? FPTC_KERNEL_WARP_TILE : (all_fixed ? FPTC_KERNEL_BLOCK_TILE : FPTC_KERNEL_GENERIC);

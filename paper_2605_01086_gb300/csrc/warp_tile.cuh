@@ -467,7 +467,21 @@ __device__ __forceinline__ void store_row(const unsigned char *row, uint32_t sx,
 // of a pass are loaded while the pass before it decodes and its steps run.
 
 constexpr int kStreamGuard = kGuard;  // bytes before (symbols of a unit's first word that are not its) and after the stage
-__host__ __device__ constexpr int stream_bytes(int cap) { return 2 * kStreamGuard + cap; }
+
+// What a unit's passes and steps read of its segment.  In shared memory: beside
+// 200 KB of tables and stages L1 keeps little, and a pass that read the segment
+// record again waited for L2.
+struct UnitSeg {
+  int64_t word_end;
+  uint64_t n_samples, out_offset, level_offset;
+  uint32_t out_aligned;
+  uint32_t caller_index;
+  uint32_t pad[6];
+};
+static_assert(sizeof(UnitSeg) == 64, "a warp's streaming area keeps its 16-byte alignment");
+__host__ __device__ constexpr int stream_bytes(int cap) { return (int)sizeof(UnitSeg) + 2 * kStreamGuard + cap; }
+// A warp's streaming area: the unit's segment, guard, stage, guard.
+constexpr int kStreamStage = (int)sizeof(UnitSeg) + kStreamGuard;
 
 // Words of a pass: two consecutive words per lane, their counts n0 | n1 << 8.
 struct PassWords {
@@ -515,11 +529,11 @@ __device__ __forceinline__ uint32_t decode_pair(const PassWords &c, uint32_t n0,
 }
 
 // The tiles [t0, t1) (of T windows each, T = tile_windows(dd)) of a launch.
-// stage: kStreamGuard bytes before it and CAP + kStreamGuard from it on are the warp's;
-// step(sg, dd, levels, win, n): n windows of segment sg from window win, levels
-// at `levels` (16-byte aligned); step_windows(dd): windows of a whole step, whose
-// symbols are a multiple of 16 and, with a word's 64, at most CAP.
-// Shared memory per warp: kStreamGuard + CAP + kStreamGuard bytes.
+// stage: kStreamStage bytes into the warp's stream_bytes(CAP);
+// step(sg, dd, levels, win, n): n windows of the unit's segment from window win, levels
+// at `levels` (16-byte aligned where every step is a multiple of 16 symbols);
+// step_windows(dd): windows of a whole step, whose symbols and a word's 64 are at
+// most CAP.
 // Barriers: step is entered with the levels visible to the warp; they are
 // rewritten only after a warp barrier.
 template <int CAP, class Dom, class Geo, class Step>
@@ -548,15 +562,25 @@ __device__ __forceinline__ void stream_tiles(const DecodeParams &p, uint64_t t0,
   uint64_t t = t0;
   while (true) {
     // ---- a unit: the range's tiles of segment s, from tile t
-    const SegDev &sg = p.segs[s];
-    const Dom &dd = doms[sg.domain];
+    const SegDev &seg = p.segs[s];
+    const Dom &dd = doms[seg.domain];
+    UnitSeg &sg = *reinterpret_cast<UnitSeg *>(stage - kStreamStage);
+    if (lane == 0) {
+      sg.word_end = (int64_t)(seg.word_offset + seg.n_words);
+      sg.n_samples = seg.n_samples;
+      sg.out_offset = seg.out_offset;
+      sg.level_offset = seg.level_offset;
+      sg.out_aligned = seg.out_aligned;
+      sg.caller_index = seg.caller_index;
+    }
+    __syncwarp();
     const uint32_t E = geo.bins(dd), sw = geo.step_windows(dd);
-    uint64_t win = (t - sg.tile_base) * geo.tile_windows(dd);
+    uint64_t win = (t - seg.tile_base) * geo.tile_windows(dd);
     // windows of the unit left (a warp's share of what device memory holds fits 32 bits)
     uint32_t left;
     {
-      const uint64_t seg_end = sg.tile_base + sg.n_tiles;
-      left = (uint32_t)((t1 < seg_end ? (t1 - sg.tile_base) * geo.tile_windows(dd) : sg.n_windows) - win);
+      const uint64_t seg_end = seg.tile_base + seg.n_tiles;
+      left = (uint32_t)((t1 < seg_end ? (t1 - seg.tile_base) * geo.tile_windows(dd) : seg.n_windows) - win);
       t = t1 < seg_end ? t1 : seg_end;  // the next unit's first tile
     }
     uint32_t bad = 0;
@@ -590,7 +614,7 @@ __device__ __forceinline__ void stream_tiles(const DecodeParams &p, uint64_t t0,
       const int32_t p0 = fill + (int32_t)(x - tot);  // place of the lane's first symbol
       // symbols from the stage's front to the unit's end (clipped: a pass adds 4096 at most)
       const int32_t rem = (int32_t)((left < 65536u ? left : 65536u) * E);
-      const int64_t hi = (int64_t)(sg.word_offset + sg.n_words);
+      const int64_t hi = sg.word_end;
       base += kPassWords;
       const int32_t upto = after < rem ? after : rem;  // symbols this pass completes, less where the stage is too small
       const bool last = (after >= rem || base >= hi) && upto <= CAP;
@@ -631,13 +655,12 @@ __device__ __forceinline__ void stream_tiles(const DecodeParams &p, uint64_t t0,
       }
       more = !last;
       if (more && off) {  // the symbols left, to the front
-        const int32_t r = fill - off;
-        for (int32_t i = 0; i < r; i += 512) {
-          uint4 v;
-          const int32_t at = i + 16 * (int32_t)lane;
-          if (at < r) v = *reinterpret_cast<const uint4 *>(stage + off + at);
-          __syncwarp();
-          if (at < r) *reinterpret_cast<uint4 *>(stage + at) = v;
+        const int32_t r = fill - off;  // fewer than a step's, so the two places do not overlap
+        if ((off & 15) == 0) {
+          for (int32_t at = 16 * (int32_t)lane; at < r; at += 512)
+            *reinterpret_cast<uint4 *>(stage + at) = *reinterpret_cast<const uint4 *>(stage + off + at);
+        } else {  // a step that is not a multiple of 16 symbols
+          for (int32_t at = (int32_t)lane; at < r; at += 32) stage[at] = stage[off + at];
         }
         fill = r;
       }
@@ -646,6 +669,7 @@ __device__ __forceinline__ void stream_tiles(const DecodeParams &p, uint64_t t0,
     bad = __reduce_or_sync(0xffffffffu, bad);
     if (bad && lane == 0) flag_bad(p.status, bad, sg.caller_index);
     if (t >= t1) break;
+    __syncwarp();  // the unit's segment has been read
     s = s1;
     ok = ok1;
     base = floor2(lo1);

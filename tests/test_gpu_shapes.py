@@ -242,3 +242,36 @@ def test_shape_transform_forms(N, E, B1, align):
         mask[int(sg["out_offset"]):int(sg["out_offset"]) + int(sg["n_samples"])] = False
     assert np.all(np.isnan(h[mask]))
     assert plan.device_status()[0] == 0
+
+
+@pytest.mark.parametrize("N,E", [(32, 16), (16, 8), (64, 32), (128, 128), (100, 50), (127, 127), (5, 5)])
+def test_long_and_short_words(N, E):
+    """Words of 64 one-bit codewords (a pass of 64 words holds 4096 symbols, more
+    than a warp's stage: the words that fit are decoded, the rest in the next
+    pass) beside words of a few long codewords, changing within a stream and from
+    stream to stream, in ranges that start and end anywhere in a word.  Levels
+    equal the oracle's bit for bit, samples within the FP32 bound."""
+    cl = np.zeros(256, np.uint8)
+    cl[128] = 1
+    cl[np.r_[0:32, 200:232]] = 7
+    d = oracle.Domain(N, E, min(2, E), E, 50.0, 0.004, (3.0, 2.0, 0.0), 8, cl)
+    long_codes = np.r_[0:32, 200:232]
+    rng = np.random.default_rng(N + E)
+    lens, levels = [], []
+    for i, W in enumerate([1, 3, 64, 1000, 4097, 300, 20000 // E]):
+        x = np.full(W * E, 128, np.uint8)
+        at = 0
+        while at < x.size:  # runs of either kind
+            n = int(rng.integers(1, 9000))
+            if i % 3 != 1 and rng.random() < 0.5:
+                x[at:at + n] = rng.choice(long_codes, size=x[at:at + n].size)
+            at += n
+        x[:E] = rng.choice(long_codes, size=E)  # no stream of zeros alone
+        lens.append(W * N)
+        levels.append(x)
+    b = crafted_batch([d], levels, lens, [0] * len(lens))
+    for ctas in (0, 1):
+        plan = make_plan(b, out_align=32, kernel="warp_tile", ctas_per_sm=ctas)
+        _, _, out, lv = gpu_decode(plan, b, out_fill=float("nan"))
+        assert plan.device_status()[0] == 0
+        compare_with_oracle(plan, b, out, lv)
