@@ -263,6 +263,12 @@ cudaError_t backward_warp_smem_config(uint32_t threads, size_t smem);
 cudaError_t launch_backward_warp(const BackwardParams &p, const WarpParams &wp, const CUtensorMap &gx_map,
                                  uint32_t threads, uint32_t grid, size_t smem, cudaStream_t stream);
 
+// adjoint from saved levels for any shape (backward_any.cu)
+size_t backward_any_smem(const uint32_t *N, const uint32_t *E, uint32_t n_domains, uint32_t *warp_bytes);
+cudaError_t backward_any_config(size_t smem, int *ctas_per_sm);
+cudaError_t launch_backward_any(const BackwardParams &p, uint32_t n_domains, uint32_t warp_bytes, uint32_t grid,
+                                size_t smem, cudaStream_t stream);
+
 cudaError_t launch_backward(const BackwardParams &p, uint32_t threads, uint32_t grid, size_t smem,
                             cudaStream_t stream);
 size_t backward_smem_bytes(uint32_t threads, uint32_t lut_cap, uint32_t coef_cap, uint32_t gx_cap,

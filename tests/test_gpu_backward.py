@@ -209,3 +209,53 @@ def test_backward_after_autotune():
     (g1, c1), (g2, c2) = outs
     np.testing.assert_allclose(g1, g2, rtol=1e-6, atol=1e-9)
     assert np.linalg.norm(c1 - c2) <= 1e-6 * np.linalg.norm(c2)
+
+
+@pytest.mark.parametrize("N,E,B1,B2", [(4, 3, 1, 2), (5, 5, 2, 5), (16, 16, 2, 16), (24, 12, 0, 12), (33, 17, 2, 16),
+                                       (64, 32, 2, 32), (64, 64, 5, 60), (100, 50, 2, 50), (127, 127, 2, 127),
+                                       (128, 64, 2, 64)])
+def test_backward_from_levels_any_shape(N, E, B1, B2):
+    """The adjoint from saved levels for other shapes: streams that end anywhere in
+    a group of windows, outputs and levels at any alignment, a domain with its
+    first zone off, against the FP64 oracle.
+
+    Bounds: dL/dC[k] of a window is a sum over n of g[n] B[k][n] by folding (one
+    rounding), at most ceil(N / 2) / 2 + 2 multiply-adds in a row and one addition,
+    with cosines off by 2^-25: within (N / 2 + 5) 2^-24 of S = sum |g[n]|.  dL/dA_z
+    adds those times unit_z (at most 1) over the bins, unit_z rounded to 2^-24, the
+    sum itself compensated: within sum (N / 2 + 5) 2^-24 S over the zone's bins, and
+    2^-24 of sum |terms|."""
+    from gpu_util import crafted_batch
+    cl = np.full(256, 8, np.uint8)
+    doms = [oracle.Domain(N, E, B1, B2, 30.0, 0.02, (0.0 if k else 3.0, 1.5, 0.0), 8, cl) for k in range(2)]
+    rng = np.random.default_rng(N * 10 + E)
+    lens = [1, N, 7 * N + 1, 16 * N, 33 * N + N // 2, 5000, 64 * N]
+    idx = [i % 2 for i in range(len(lens))]
+    levels = [rng.integers(0, 256, size=doms[j].windows(S) * E).astype(np.uint8) for S, j in zip(lens, idx)]
+    b = crafted_batch(doms, levels, lens, idx)
+    for align in (32, 1):
+        plan = make_plan(b, out_align=align, out_base=0 if align == 32 else 3)
+        _, _, out, lv = gpu_decode(plan, b)
+        gx = torch.randn(plan.info["out_extent"], generator=torch.Generator().manual_seed(3)).to(plan.device)
+        gco = torch.empty(plan.info["n_levels_total"], device=plan.device)
+        gsc, _ = plan.backward(gx, levels=lv, grad_coeffs=gco)
+        torch.cuda.synchronize()
+        gh = gx.double().cpu().numpy()
+        gA, absA, gC = _oracle_grads(plan, b, lv.cpu().numpy(), gh)
+        got = gco.double().cpu().numpy()
+        slack = 2.0 ** -24 * absA
+        for i, S in enumerate(lens):
+            a, o = int(plan.level_offsets[i]), int(plan.segments[i]["out_offset"])
+            W = doms[idx[i]].windows(S)
+            g = np.zeros(W * N)
+            g[:S] = np.abs(gh[o:o + S])
+            bound = (N / 2 + 5) * 2.0 ** -24 * g.reshape(W, N).sum(1)
+            c = gC[i].reshape(W, E)
+            assert np.all(np.abs(got[a:a + W * E].reshape(W, E) - c) <= bound[:, None]), i
+            slack[idx[i], 0] += bound.sum() * B1
+            slack[idx[i], 1] += bound.sum() * (B2 - B1)
+        g = gsc.cpu().numpy()
+        for d in range(2):
+            for z in range(2):
+                want = 0.0 if (z == 0 and d == 1) else gA[d, z]
+                assert abs(g[d, z] - want) <= slack[d, z], (d, z, g[d, z], want)
