@@ -16,16 +16,23 @@ from ._lib import CPlanInfo, CPlanOptions, check, lib
 from .codec import SEGMENT_DTYPE, Domain, c_domains
 
 
+# A call here is a few microseconds of Python around two or three kernel
+# launches, and a differentiable step runs some of it in autograd's own thread:
+# pointers and streams are passed as the integers they are, and a tensor that is
+# as required is found so by one expression.
+
 def _dptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream, device):
-    s = stream if stream is not None else torch.cuda.current_stream(device)
-    return ctypes.c_void_p(s.cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(device.index) if stream is None else stream.cuda_stream
 
 
 def _require(t, dtype, device, name, numel=None):
+    if isinstance(t, torch.Tensor) and t.dtype == dtype and t.device == device and t.is_contiguous() and \
+            (numel is None or t.numel() >= numel):
+        return
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if t.dtype != dtype:
@@ -34,8 +41,12 @@ def _require(t, dtype, device, name, numel=None):
         raise ValueError(f"{name} must be on {device}, got {t.device}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if numel is not None and t.numel() < numel:
-        raise ValueError(f"{name} needs at least {numel} elements, has {t.numel()}")
+    raise ValueError(f"{name} needs at least {numel} elements, has {t.numel()}")
+
+
+def _as_float32(t):
+    """t as a contiguous float32 tensor (t itself if it is one)."""
+    return t if t.dtype == torch.float32 and t.is_contiguous() else t.to(torch.float32).contiguous()
 
 
 class Plan:
@@ -200,9 +211,15 @@ class FPTCDecode(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, scale, coeff_probe, plan: Plan, words, symlen):
-        sc = scale.detach().to(torch.float32).contiguous()
-        levels = torch.empty(max(1, plan.info["n_levels_total"]), dtype=torch.uint8, device=plan.device)
-        out = plan.decode(words, symlen, levels=levels, scale=sc)
+        # Plan.decode with the buffers made here (which need no check)
+        dev, info = plan.device, plan.info
+        sc = _as_float32(scale.detach())
+        plan._check_inputs(words, symlen)
+        _require(sc, torch.float32, dev, "scale", 3 * len(plan.domains))
+        levels = torch.empty(max(1, info["n_levels_total"]), dtype=torch.uint8, device=dev)
+        out = torch.empty(max(1, info["out_extent"]), dtype=torch.float32, device=dev)
+        check(lib().fptc_decode_batch(plan._h, words.data_ptr(), symlen.data_ptr(), out.data_ptr(), levels.data_ptr(),
+                                      sc.data_ptr(), _stream(None, dev)))
         ctx.plan = plan
         ctx.scale_dtype = scale.dtype
         ctx.save_for_backward(sc, levels)
@@ -210,14 +227,20 @@ class FPTCDecode(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, grad_out):
+        # Plan.backward from the saved levels
         sc, levels = ctx.saved_tensors
         plan = ctx.plan
-        want_c = ctx.needs_input_grad[1]
-        gco = torch.empty(max(1, plan.info["n_levels_total"]), dtype=torch.float32,
-                          device=plan.device) if want_c else None
-        gsc, _ = plan.backward(grad_out.contiguous().to(torch.float32), levels=levels, scale=sc, grad_coeffs=gco)
-        g_scale = gsc.to(ctx.scale_dtype).reshape(sc.shape) if ctx.needs_input_grad[0] else None
-        return g_scale, gco, None, None, None
+        dev, n_levels = plan.device, plan.info["n_levels_total"]
+        want_scale, want_c = ctx.needs_input_grad[:2]
+        g = _as_float32(grad_out)
+        _require(g, torch.float32, dev, "grad_out", plan.info["out_extent"])
+        _require(levels, torch.uint8, dev, "levels", n_levels)
+        _require(sc, torch.float32, dev, "scale", 3 * len(plan.domains))
+        gco = torch.empty(max(1, n_levels), dtype=torch.float32, device=dev) if want_c else None
+        gsc = torch.empty(len(plan.domains), 3, dtype=torch.float64, device=dev)
+        check(lib().fptc_decode_backward(plan._h, None, None, levels.data_ptr(), sc.data_ptr(), g.data_ptr(),
+                                         _dptr(gco), gsc.data_ptr(), _stream(None, dev)))
+        return (gsc.to(ctx.scale_dtype).reshape(sc.shape) if want_scale else None), gco, None, None, None
 
 
 def decode_differentiable(plan: Plan, words, symlen, scale, coeff_probe=None):
