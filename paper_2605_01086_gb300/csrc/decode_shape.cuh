@@ -70,8 +70,12 @@ __host__ __device__ constexpr uint32_t shape_form(uint32_t N, uint32_t kz, uint3
   return N << 8 | bins;
 }
 
+// Windows per lane of shape_pairs: four, two with one output tile per warp (up to
+// 24 warps: 80 registers a thread, half of them accumulators at two).
+__host__ __device__ constexpr uint32_t shape_pair_windows(uint32_t tiles) { return tiles > 1 ? 4 : 2; }
+
 // Windows per output step.  Compiled forms: 32 lanes, 32 / N windows each for N
-// < 32.  shape_pairs: as many groups of four windows as lanes for their groups
+// < 32.  shape_pairs: as many groups of its windows as lanes for their groups
 // of eight pairs, less where the coefficients (twice) or the samples would not
 // fit the warp's output tiles.  Either way at most 2048 symbols.
 __host__ __device__ constexpr uint32_t shape_step(uint32_t N, uint32_t E, uint32_t kz, uint32_t tiles) {
@@ -80,7 +84,8 @@ __host__ __device__ constexpr uint32_t shape_step(uint32_t N, uint32_t E, uint32
     w = N >= 32 ? 32 : 1024 / N;
   } else {
     const uint32_t bytes = tiles * (uint32_t)kOutTile;
-    w = 32 / (shape_pairs8(N) / 8) * 4;
+    const uint32_t m = shape_pair_windows(tiles);
+    w = 32 / (shape_pairs8(N) / 8) * m;
     const uint32_t fit_c = bytes / (8 * (kz ? kz : 1)) / 4 * 4, fit_x = bytes / (4 * N) / 4 * 4;
     w = w < fit_c ? w : fit_c;
     w = w < fit_x ? w : fit_x;
@@ -463,14 +468,14 @@ __device__ __forceinline__ void bulk_store(float *dst, const void *src, uint32_t
   asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
-// The pair form, any N: a step of n windows (at most dd.step, a multiple of
-// four).  The warp's output tiles hold the step's coefficients ([bin][window],
+// The pair form, any N: a step of n windows (at most dd.step), MW a lane.  The warp's output tiles hold the step's coefficients ([bin][window],
 // each twice) and then its samples (as they lie in the output).
+template <int MW>
 __device__ __forceinline__ void shape_pairs(const DecodeParams &p, const UnitSeg &sg, const DomS &dd,
                                             const unsigned char *smem, const uint8_t *lv0, uint64_t win, uint32_t n,
                                             const ShapeOut &o) {
   const uint32_t lane = o.lane, N = dd.N, P = shape_pair_count(N), p8 = shape_pairs8(N), kz = dd.kz;
-  const uint32_t Ws = (dd.step + 3) / 4 * 4;  // rows of coefficients: whole groups of four windows
+  const uint32_t Ws = (dd.step + 3) / 4 * 4;  // rows of coefficients
   const float *deq = reinterpret_cast<const float *>(smem + dd.deq_off);
   const float *bas = reinterpret_cast<const float *>(smem + dd.basis_off);
   if (lane == 0) tma_wait_read_but<0>();  // earlier steps have left the tiles
@@ -492,28 +497,33 @@ __device__ __forceinline__ void shape_pairs(const DecodeParams &p, const UnitSeg
     }
   }
   __syncwarp();
-  // ---- four windows by eight pairs a lane
+  // ---- MW windows by eight pairs a lane
   const uint32_t pgs = p8 / 8, wg = lane / pgs, pg = lane - wg * pgs;
-  const bool mine = 4 * wg < Ws;
-  float2 ev[4][4], od[4][4];
+  const bool mine = MW * wg < Ws;
+  float2 ev[MW][4], od[MW][4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < MW; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) ev[i][j] = od[i][j] = make_float2(0.0f, 0.0f);
   if (mine) {
-    const float4 *cp = reinterpret_cast<const float4 *>(o.otile) + 2 * wg;  // windows 4 wg .. + 3 of bin 0
+    const float4 *cp = reinterpret_cast<const float4 *>(o.otile) + MW / 2 * wg;  // windows MW wg .. of bin 0
     const float4 *bp = reinterpret_cast<const float4 *>(bas) + 2 * pg;
     const uint32_t cstep = Ws / 2, bstep = p8 / 4;
-    auto bin = [&](float2(&acc)[4][4]) {
-      const float4 c01 = cp[0], c23 = cp[1], b0 = bp[0], b1 = bp[1];
+    auto bin = [&](float2(&acc)[MW][4]) {
+      float2 c[MW];
+#pragma unroll
+      for (int i = 0; i < MW; i += 2) {
+        const float4 q = cp[i / 2];
+        c[i] = make_float2(q.x, q.y);
+        c[i + 1] = make_float2(q.z, q.w);
+      }
+      const float4 b0 = bp[0], b1 = bp[1];
       cp += cstep;
       bp += bstep;
-      const float2 c[4] = {make_float2(c01.x, c01.y), make_float2(c01.z, c01.w), make_float2(c23.x, c23.y),
-                           make_float2(c23.z, c23.w)};
       const float2 b[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y),
                            make_float2(b1.z, b1.w)};
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < MW; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = __ffma2_rn(c[i], b[j], acc[i][j]);
     };
@@ -529,9 +539,9 @@ __device__ __forceinline__ void shape_pairs(const DecodeParams &p, const UnitSeg
   if (mine) {
     const bool whole = N % 4 == 0 && 8 * pg + 8 <= P;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (4 * wg + i >= dd.step) break;
-      float *const x = reinterpret_cast<float *>(o.otile) + (4 * wg + i) * N;
+    for (int i = 0; i < MW; ++i) {
+      if (MW * wg + i >= dd.step) break;
+      float *const x = reinterpret_cast<float *>(o.otile) + (MW * wg + i) * N;
       float f[8], m[8];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -635,7 +645,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_decode_shape(const DecodePara
         if constexpr (FORMS & kShapeCompiled) done = shape_compiled<TILES, ONE>(p, sg, dd, smem_raw, levels, win, n, o, turn);
         if constexpr (FORMS & kShapeAny)
           if (!done) {
-            shape_pairs(p, sg, dd, smem_raw, levels, win, n, o);
+            shape_pairs<(int)shape_pair_windows(TILES)>(p, sg, dd, smem_raw, levels, win, n, o);
             turn = kAllTiles;
           }
       });

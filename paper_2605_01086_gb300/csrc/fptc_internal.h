@@ -67,7 +67,8 @@ void fill_domain_dev(const fptc_domain &dm, DomainDev *dd);
 // c, and a NaN bound is never <= c).
 void host_zone_bounds(const fptc_domain &d, uint32_t zone, double *bounds);
 
-// One segment, in tile-queue order (segments sorted by domain).
+// One segment, in tile-queue order (by output offset), or in the order of the
+// domains' transforms (fptc_plan segs_form).
 struct SegDev {
   uint64_t word_offset;
   uint64_t n_words;
@@ -83,6 +84,8 @@ struct SegDev {
   uint32_t domain;
   uint32_t caller_index; // position in the caller's segment array
   uint32_t out_aligned;  // bit 0: out_offset % 4 == 0 (16-byte stores), bit 1: % 8 (32-byte), bit 2: % 32 (128-byte rows)
+  uint32_t queue_index;  // position in tile-queue order (seg_bad)
+  uint32_t pad;
 };
 
 // Start of a tile in the SymLen stream: the word holding the tile's first symbol
@@ -141,6 +144,7 @@ struct DecodeParams {
   uint32_t seg_begin, seg_end;    // segment range covering it
   uint32_t lut_cap;               // decode-table entries that fit the shared buffer
   uint32_t coef_cap;              // tile_windows * E capacity of the shared tile buffers
+  uint32_t form_order;            // segs are not in tile-queue order: seg_bad by their queue_index
   uint32_t after_index;           // launched right behind the index kernel: may start before it ends (launch_after)
 };
 

@@ -28,6 +28,11 @@ struct fptc_plan {
   std::vector<fptc_segment> caller_segs;
   std::vector<uint32_t> queue;           // queue position -> caller index
   std::vector<SegDev> segs;              // queue order
+  // The same by the domains' transforms, with tiles numbered in that order, where the
+  // shape kernel serves domains of several: a CTA's range then holds one transform
+  // (mostly), whose code stays in its SM's instruction cache (a batch of four shapes:
+  // 110 us in queue order, warps stalled for instructions; 80 us in this).
+  std::vector<SegDev> segs_form;
   std::vector<DomainDev> dom_dev;
   std::vector<uint64_t> level_off;       // caller order
   uint64_t n_tiles = 0, n_chunks = 0, n_groups = 0, n_levels = 0;
@@ -35,6 +40,7 @@ struct fptc_plan {
   // device memory owned by the plan
   DomainDev *d_domains = nullptr;
   SegDev *d_segs = nullptr;
+  SegDev *d_segs_form = nullptr;
   uint16_t *d_luts = nullptr;
   float *d_basis = nullptr;
   uint32_t *d_chunk_sum = nullptr;
@@ -115,6 +121,7 @@ struct PlanDeleter {
 void free_device(fptc_plan *p) {
   cudaFree(p->d_domains);
   cudaFree(p->d_segs);
+  cudaFree(p->d_segs_form);
   cudaFree(p->d_luts);
   cudaFree(p->d_basis);
   cudaFree(p->d_chunk_sum);
@@ -138,7 +145,7 @@ void free_device(fptc_plan *p) {
 
 void PlanDeleter::operator()(fptc_plan *p) const {
   if (!p) return;
-  if (p->d_domains || p->d_segs || p->d_luts || p->d_basis || p->d_chunk_sum || p->d_chunk_off || p->d_seg_bad ||
+  if (p->d_domains || p->d_segs || p->d_segs_form || p->d_luts || p->d_basis || p->d_chunk_sum || p->d_chunk_off || p->d_seg_bad ||
       p->d_groups || p->d_done || p->d_word_off || p->d_lev_scratch || p->d_tiles || p->d_status || p->up || p->ev_start || p->aux[0] ||
       p->ev[0] || p->evh[0]) {
     DeviceGuard g(p->device);
@@ -261,6 +268,26 @@ void layout_tiles(fptc_plan *p, uint32_t tile_samples) {
     t += s.n_tiles;
   }
   p->n_tiles = t;
+  p->segs_form.clear();
+  if (shape) {
+    auto form = [&](const SegDev &sg) -> uint32_t {
+      const DomainDev &dd = p->dom_dev[sg.domain];
+      const uint32_t f = shape_one_form(dd.N, std::min(dd.E, dd.B2), p->shape_tiles);
+      return f ? f : dd.N;  // compiled forms lie above every N
+    };
+    bool several = false;
+    for (const SegDev &sg : p->segs) several = several || form(sg) != form(p->segs[0]);
+    if (several) {
+      p->segs_form = p->segs;
+      std::stable_sort(p->segs_form.begin(), p->segs_form.end(),
+                       [&](const SegDev &a, const SegDev &b) { return form(a) < form(b); });
+      uint64_t base = 0;
+      for (SegDev &sg : p->segs_form) {
+        sg.tile_base = base;
+        base += sg.n_tiles;
+      }
+    }
+  }
 }
 
 // FPTC_ERR_UNSUPPORTED with the sizes when a kernel's shared memory at `threads`
@@ -463,6 +490,16 @@ fptc_status upload_layout(fptc_plan *p) {
     e = cudaMemcpy(p->d_domains, p->dom_dev.data(), p->dom_dev.size() * sizeof(DomainDev), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(e, "upload domains");
   }
+  if (!p->segs_form.empty()) {
+    const size_t bytes = p->segs_form.size() * sizeof(SegDev);
+    if (!p->d_segs_form) {
+      e = cudaMalloc(&p->d_segs_form, bytes);
+      if (e != cudaSuccess) return cuda_fail(e, "segments by transform");
+      p->device_bytes += bytes;
+    }
+    e = cudaMemcpy(p->d_segs_form, p->segs_form.data(), bytes, cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return cuda_fail(e, "upload segments by transform");
+  }
   if (p->n_tiles > p->tiles_capacity) {
     if (p->d_tiles) {
       cudaFree(p->d_tiles);
@@ -569,6 +606,10 @@ cudaError_t run_range(const fptc_plan *p, const IndexParams &ip0, const DecodePa
   if (p->kind == FPTC_KERNEL_WARP_TILE) {
     WarpParams wp = p->wp;
     if (p->shape) {
+      if (!p->segs_form.empty() && s0 == 0 && s1 == p->segs.size()) {  // the whole plan
+        dp.segs = p->d_segs_form;
+        dp.form_order = 1;
+      }
       ShapeMaps maps;
       std::memset(&maps, 0, sizeof(maps));
       wp.out_tma = encode_out_map(&maps.rows, dp.out, p->out_extent) ? 1u : 0u;
@@ -859,6 +900,7 @@ fptc_status fptc_plan_create(fptc_plan **out, int device, const fptc_domain *dom
       sd.n_windows = (s.n_samples + d.N - 1) / d.N;
       sd.domain = s.domain;
       sd.caller_index = ci;
+      sd.queue_index = (uint32_t)qi;
       sd.out_aligned = ((s.out_offset % 4) == 0 ? 1u : 0u) | ((s.out_offset % 8) == 0 ? 2u : 0u) |
                        ((s.out_offset % 32) == 0 ? 4u : 0u);
       sd.chunk_base = chunk;

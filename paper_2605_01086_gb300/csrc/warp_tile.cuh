@@ -545,7 +545,8 @@ __device__ __forceinline__ void stream_tiles(const DecodeParams &p, uint64_t t0,
   uint32_t s = warp_find_segment(p.segs, p.seg_begin, p.seg_end, t0, lane);
   int64_t base;         // the pass's first word
   int32_t fill = 0;     // symbols in the stage (negative: those of the unit's first word before it)
-  bool ok = p.seg_bad[s] == 0;
+  auto bad_segment = [&](uint32_t i) -> bool { return p.seg_bad[p.form_order ? p.segs[i].queue_index : i] != 0; };
+  bool ok = !bad_segment(s);
   PassWords nx;
   {
     const SegDev &sg = p.segs[s];
@@ -592,7 +593,7 @@ __device__ __forceinline__ void stream_tiles(const DecodeParams &p, uint64_t t0,
       do ++s1; while (t >= p.segs[s1].tile_base + p.segs[s1].n_tiles);  // segments without tiles
       lo1 = (int64_t)p.segs[s1].word_offset;
       hi1 = lo1 + (int64_t)p.segs[s1].n_words;
-      ok1 = p.seg_bad[s1] == 0;
+      ok1 = !bad_segment(s1);
       if (!ok1) hi1 = lo1;
     };
     if (!ok && t < t1) {  // a segment the index rejected: only the next unit's first words
