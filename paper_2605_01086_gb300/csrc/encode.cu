@@ -437,6 +437,7 @@ __device__ __forceinline__ void lv_load_async(const EncParams &p, const LvWin &w
 // that); each group's samples come into shared memory by asynchronous copies while
 // the warp computes the group before.
 __global__ void __launch_bounds__(kLvThreads, 5) k_enc_levels_w32(EncParams p, uint64_t n_windows, uint32_t groups) {
+  dependents_may_start();
   // per warp: two groups' samples (one row per window), and the second tier's
   // work list (window lane, bin), the windows' levels, segments, sample sums
   __shared__ __align__(16) float rows[kLvThreads / 32][2][32 * kRowPitch];
@@ -628,7 +629,9 @@ __global__ void __launch_bounds__(kLvThreads, 5) k_enc_levels_w32(EncParams p, u
 // of a run (256 symbols) on small ones.  With a block's packing done by one
 // thread twice (its reference, then the words) the chain was 16,384 symbols
 // and more: 43 M levels of a mixed batch took 1,112 us for the packing, now
-// 123 us (79 + 2 + 42); one stream of 32,768 levels 677 us, now 30 us.  Runs of
+// 113 us (69 + 2 + 42); one stream of 32,768 levels 677 us, now 24 us.  The loops
+// of k_enc_starts are rolled up: unrolled, its 50 KB of code came from L2 once per
+// SM and cost 10 us more (21 us for one stream, 14 now).  Runs of
 // 2048 symbols by one thread without tables left 5 to 14 % of the blocks
 // unmet, and the scan that walked them took 380 us.
 
@@ -687,54 +690,51 @@ constexpr uint32_t kExitPitch = 68;              // bytes per run: its exits by 
 constexpr uint32_t kSeqPitch = 33;               // bytes per first start: the states its 32 runs are entered in, exit
 constexpr uint32_t kStartWarpBytes = 32 * kExitPitch + 64 * kSeqPitch + 32 * 8;
 
-// The run packed from first starts base .. base + 2 R - 1 on (base a multiple
-// of 16, R <= 8): s[r] ends as the states of first starts base + 2 r and + 1.
-// c2: a level's code length in both halves.
-template <int R, class Len2>
-__device__ __forceinline__ void pack_run(const uint8_t *lv, uint32_t base, const Len2 &c2, uint32_t (&s)[R]) {
-#pragma unroll
-  for (int r = 0; r < R; ++r) s[r] = 0xFFFFFFFFu;  // a full word: the next symbol starts one
-  uint4 cur[4], nxt[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    cur[q] = make_uint4(0u, 0u, 0u, 0u);
-    if (base + 16 * q < kSub) cur[q] = load_run16(lv, base + 16 * q, kSub);
-    nxt[q] = cur[q];
-  }
-  each16(cur[0], [&](int j, uint32_t level) {  // first start j begins at symbol base + j
-    const uint32_t c = c2(level), k = c + kOff16x2;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      if (j >= 2 * r) s[r] = __viaddmax_u16x2(s[r], c, k);
-      if (j == 2 * r) s[r] |= 0xFFFF0000u;
-    }
-  });
-  auto step = [&](const uint4 &v) {
-    each16(v, [&](int, uint32_t level) {
-      const uint32_t c = c2(level), k = c + kOff16x2;
-#pragma unroll
-      for (int r = 0; r < R; ++r) s[r] = __viaddmax_u16x2(s[r], c, k);
-    });
-  };
+// fn(v, levels 16 v .. 16 v + 15) over the run of n at lv, the next three vectors
+// in flight.  One place in the code where levels are loaded: a small batch runs
+// this once per SM, from a cold instruction cache.
+template <class F>
+__device__ __forceinline__ void each_vector(const uint8_t *lv, uint32_t first, uint32_t n, F fn) {
+  const int nv = (int)((n + 15) / 16);
+  uint4 r0, r1, r2, r3;
+  r1 = r2 = r3 = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll 1
-  for (uint32_t i = base; i < kSub; i += 64) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if (i + 64 + 16 * q < kSub) nxt[q] = load_run16(lv, i + 64 + 16 * q, kSub);
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if ((q || i != base) && i + 16 * q < kSub) step(cur[q]);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) cur[q] = nxt[q];
+  for (int v = (int)first - 3; v < nv; ++v) {
+    r0 = r1;
+    r1 = r2;
+    r2 = r3;
+    if (v + 3 < nv) r3 = load_run16(lv, 16 * (uint32_t)(v + 3), n);
+    if (v >= (int)first) fn((uint32_t)v, r0);
   }
 }
 
 // Exits of a run by first start into its row (bytes: the states' low bytes,
-// u - 65 mod 256), for the first starts base .. base + 2 R - 1.
+// u - 65 mod 256), for the first starts base .. base + 2 R - 1 (base a multiple of
+// 16, R <= 8): two packings per instruction, c2 a level's code length in both
+// halves.
 template <int R, class Len2>
 __device__ __forceinline__ void run_exits(const uint8_t *lv, uint32_t base, const Len2 &c2, uint8_t *row) {
   uint32_t s[R];
-  pack_run<R>(lv, base, c2, s);
+#pragma unroll
+  for (int r = 0; r < R; ++r) s[r] = 0xFFFFFFFFu;  // a full word: the next symbol starts one
+  each_vector(lv, base / 16, kSub, [&](uint32_t v, const uint4 &q) {
+    if (v == base / 16) {  // first start j begins at symbol base + j
+      each16(q, [&](int j, uint32_t level) {
+        const uint32_t c = c2(level), k = c + kOff16x2;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          if (j >= 2 * r) s[r] = __viaddmax_u16x2(s[r], c, k);
+          if (j == 2 * r) s[r] |= 0xFFFF0000u;
+        }
+      });
+    } else {
+      each16(q, [&](int, uint32_t level) {
+        const uint32_t c = c2(level), k = c + kOff16x2;
+#pragma unroll
+        for (int r = 0; r < R; ++r) s[r] = __viaddmax_u16x2(s[r], c, k);
+      });
+    }
+  });
   // byte 0 and byte 2 of two states
 #pragma unroll
   for (int r = 0; r < R; r += 2)
@@ -749,7 +749,8 @@ __device__ __forceinline__ uint32_t first_start(uint64_t bounds, uint32_t u) {
 }
 
 template <bool TAB>
-__global__ void __launch_bounds__((kStartWarps + 1) * 32, 3) k_enc_starts(EncParams p) {
+__global__ void __launch_bounds__((kStartWarps + 1) * 32, 4) k_enc_starts(EncParams p) {
+  dependents_may_start();
   extern __shared__ uint32_t starts_smem[];
   // per block: what it is (bit 0: there is one, 1: its stream's first, 2: another follows it, 3: every first start
   // gives one exit), the state it is entered in and which first start that is
@@ -765,6 +766,7 @@ __global__ void __launch_bounds__((kStartWarps + 1) * 32, 3) k_enc_starts(EncPar
       tab_s[i] = entry_len(__ldg(p.code_tab + i)) * 0x10001u;
     __syncthreads();
   }
+  dependency_wait();  // the levels
   const uint64_t b = (uint64_t)blockIdx.x * kStartWarps + wid - 1;  // warp 0: the block before the CTA's (may wrap: none)
   bool have = b < p.n_blocks;
   const uint8_t *lv = p.levels;  // this lane's run
@@ -816,10 +818,8 @@ __global__ void __launch_bounds__((kStartWarps + 1) * 32, 3) k_enc_starts(EncPar
       // as many packings as the warp's runs want (the instance is the warp's)
       if (most - base > 12)
         run_exits<8>(lv, base, c2, row);
-      else if (most - base > 8)
-        run_exits<6>(lv, base, c2, row);
       else
-        run_exits<4>(lv, base, c2, row);
+        run_exits<6>(lv, base, c2, row);
     }
     __syncwarp();
     // ---- the block's: lane = first start, run after run
@@ -866,51 +866,36 @@ __global__ void __launch_bounds__((kStartWarps + 1) * 32, 3) k_enc_starts(EncPar
   }
   __syncthreads();
   if (wid == 0 || !have) return;
-  // ---- the word starts, each lane those of its run
+  // ---- the word starts, each lane those of its run (its bitmap in halfwords over its row of exits)
   uint32_t seen = 0, cnt = 0;
   const uint32_t n = lane * kSub < nb ? (nb - lane * kSub < kSub ? nb - lane * kSub : kSub) : 0u;
   const uint32_t u_in = in_s[wid];
-  uint32_t *const row = p.masks + b * kMaskWords + lane * (kSub / 32);
   if (n) {
-    const uint32_t cand = cand_s[wid];
-    uint32_t s = (lane ? (uint32_t)seq[cand * kSeqPitch + lane] : u_in) + kOff32;
-    uint32_t m[kSub / 32];
-#pragma unroll
-    for (uint32_t q = 0; q < kSub / 32; ++q) m[q] = 0u;
-    uint4 cur[2], nxt[2];
-    cur[0] = load_run16(lv, 0, n);
-    cur[1] = 16u < n ? load_run16(lv, 16, n) : make_uint4(0u, 0u, 0u, 0u);
-    nxt[0] = nxt[1] = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-    for (uint32_t q = 0; q < kSub / 32; ++q) {
-      const uint32_t i = 32 * q;
-      if (i + 32 < n) nxt[0] = load_run16(lv, i + 32, n);
-      if (i + 48 < n) nxt[1] = load_run16(lv, i + 48, n);
-      if (i + 32 <= n) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-          each16(cur[h], [&](int j, uint32_t level) {
-            const uint32_t c = c2(level) & 0xffffu, k = c + kOff32;
-            seen |= c;
-            s = __viaddmax_u32(s, c, k);
-            if (s == k) m[q] |= 1u << (16 * h + j);
-          });
-      } else if (i < n) {
+    uint16_t *const bits = reinterpret_cast<uint16_t *>(exits + lane * kExitPitch);
+    uint32_t s = (lane ? (uint32_t)seq[cand_s[wid] * kSeqPitch + lane] : u_in) + kOff32;
+    auto start = [&](uint32_t level) -> bool {
+      const uint32_t c = c2(level) & 0xffffu, k = c + kOff32;
+      seen |= c;
+      s = __viaddmax_u32(s, c, k);
+      return s == k;
+    };
+    each_vector(lv, 0, n, [&](uint32_t v, const uint4 &q) {
+      uint32_t m = 0;
+      if (16 * v + 16 <= n) {
+        each16(q, [&](int j, uint32_t level) { m |= start(level) ? 1u << j : 0u; });
+      } else {  // the stream's last symbols
 #pragma unroll 1
-        for (uint32_t j = 0; i + j < n; ++j) {
-          const uint32_t c = c2((uint32_t)__ldg(lv + i + j)) & 0xffffu, k = c + kOff32;
-          seen |= c;
-          s = __viaddmax_u32(s, c, k);
-          if (s == k) m[q] |= 1u << j;
-        }
+        for (uint32_t j = 0; 16 * v + j < n; ++j) m |= start((uint32_t)__ldg(lv + 16 * v + j)) ? 1u << j : 0u;
       }
-      cnt += __popc(m[q]);
-      cur[0] = nxt[0];
-      cur[1] = nxt[1];
-    }
+      cnt += __popc(m);
+      bits[v] = (uint16_t)m;
+    });
+    for (uint32_t v = (n + 15) / 16; v < kSub / 16; ++v) bits[v] = 0;
+    const uint32_t *const w = reinterpret_cast<const uint32_t *>(bits);
+    uint4 *const row = reinterpret_cast<uint4 *>(p.masks + b * kMaskWords + lane * (kSub / 32));
     static_assert(kSub == 256, "a run's bitmap is two 16-byte vectors");
-    reinterpret_cast<uint4 *>(row)[0] = make_uint4(m[0], m[1], m[2], m[3]);
-    reinterpret_cast<uint4 *>(row)[1] = make_uint4(m[4], m[5], m[6], m[7]);
+    row[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    row[1] = make_uint4(w[4], w[5], w[6], w[7]);
   }
   cnt = __reduce_add_sync(0xffffffffu, cnt);
   seen = __reduce_or_sync(0xffffffffu, seen);
@@ -974,6 +959,9 @@ __device__ void walk_block(const EncParams &p, const EncSeg &sg, const EncDomain
 // entered in another state than assumed is walked again from the true one;
 // code and room checks; the stream's word count.
 __global__ void __launch_bounds__(128) k_enc_scan(EncParams p) {
+  dependents_may_start();
+  dependency_wait();  // the blocks' records
+  if (blockIdx.x == 0 && threadIdx.x == 0) *p.fb_count = 0;  // the level kernels' list, for the next encode
   const uint64_t s = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint32_t lane = threadIdx.x & 31u;
   if (s >= p.n_segs) return;  // the whole warp
@@ -1070,7 +1058,18 @@ __device__ __forceinline__ bool level_compensated(const EncParams &p, uint64_t g
 #pragma unroll
     for (int n = 0; n < 32; ++n) step(xv[n], cs[n]);
   } else {
-    for (uint32_t n = 0; n < nn; ++n) step(__ldg(src + n), __ldg(ct + (size_t)n * d.E));
+    for (uint32_t n0 = 0; n0 < nn; n0 += 16) {  // sixteen of each requested at once
+      float xv[16];
+      float2 cs[16];
+#pragma unroll
+      for (uint32_t j = 0; j < 16; ++j) {
+        xv[j] = n0 + j < nn ? __ldg(src + n0 + j) : 0.0f;
+        cs[j] = n0 + j < nn ? __ldg(ct + (size_t)(n0 + j) * d.E) : make_float2(0.0f, 0.0f);
+      }
+#pragma unroll
+      for (uint32_t j = 0; j < 16; ++j)
+        if (n0 + j < nn) step(xv[j], cs[j]);
+    }
   }
   const float err2 = s1 * (2.0f / (float)d.N) * 0x1p-34f + 1e-30f;
   const double cd = ((double)hi + (double)lo) * (2.0 / (double)d.N);
@@ -1087,17 +1086,19 @@ __device__ __forceinline__ bool level_compensated(const EncParams &p, uint64_t g
 // copied into shared memory meanwhile.
 //
 // Error of such a sum against the exact one: each of the P fused multiply-adds
-// rounds a partial sum of magnitude at most S = sum |u| (or |v|), the folding
+// (paired: over even and over odd n, added at the end) rounds a partial sum of
+// magnitude at most S = sum |u| (or |v|), and so does that addition, the folding
 // rounds each u to 2^-24 |u| and the cosines (at most 1) are off by at most
-// 2^-25, so (P + 1.5) 2^-24 S and terms of second order; (P + 4) 2^-24 S is
+// 2^-25, so (P + 2.5) 2^-24 S and terms of second order; (P + 4) 2^-24 S is
 // used, and 2^-40 (sum |u| + sum |v|) for the host encoder's own rounding in FP64
 // (N 2^-52 sum |x|, and sum |x| <= sum |u| + sum |v|).  The zone maps are bracketed
 // by that bound as in the window kernel; a bin it does not settle (about one
 // in 200) goes to the list of k_enc_fallback, or, where a tile has many, is
 // settled here by the compensated sum.
 // Bound by instruction issue (about 30 instructions a sample at N = 64, E = 32).
-// 16.8 M samples at N = 64, E = 32: 75 us (one thread per bin with the compensated
-// sum for every bin took 457 us).
+// 16.8 M samples at N = 64, E = 32: 70 us (one thread per bin with the compensated
+// sum for every bin took 457 us; the zone maps behind a branch per bin, and plain
+// multiply-adds, 75).
 constexpr uint32_t kAnyWarps = 4;
 constexpr uint32_t kAnyTile0 = 4;  // zone-0 bins of a window mapped by all lanes together
 
@@ -1129,12 +1130,14 @@ __host__ __device__ constexpr uint32_t any_bytes(uint32_t N, uint32_t E) {
 
 __global__ void __launch_bounds__(kAnyWarps * 32, 4) k_enc_levels_any(EncParams p, uint64_t n_units, uint32_t warp_bytes) {
   extern __shared__ __align__(16) unsigned char any_smem[];
+  dependents_may_start();
   const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
   const uint64_t unit = (uint64_t)blockIdx.x * kAnyWarps + wid;
   if (unit >= n_units) return;  // the whole warp
   const EncUnit un = p.units[unit];
-  const EncSeg &sg = p.segs[un.seg];
-  const EncDomain &d = p.doms[sg.domain];
+  // by value: read through references they are loaded again after every store
+  const EncSeg sg = p.segs[un.seg];
+  const EncDomain d = p.doms[sg.domain];
   const uint32_t N = d.N, E = d.E, B1 = d.B1, B2 = d.B2;
   const uint32_t P = (N + 1) / 2, P4 = any_pairs4(N), tile = any_tile(N, E);
   const uint32_t xp = any_pitch(N), up = any_pitch(P4);
@@ -1225,12 +1228,11 @@ __global__ void __launch_bounds__(kAnyWarps * 32, 4) k_enc_levels_any(EncParams 
         const float *cs[4];
 #pragma unroll
         for (uint32_t j = 0; j < 4; ++j) cs[j] = dots + (k0 + 2 * j < E ? k0 + 2 * j : k0) * P4;
-        float acc[4][4];
+        float2 pair[4][4];  // sums over even and odd n
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
-#pragma unroll 2
+          for (int j = 0; j < 4; ++j) pair[i][j] = make_float2(0.0f, 0.0f);
         for (uint32_t c = 0; c < P4; c += 4) {
           float4 f[4];
 #pragma unroll
@@ -1240,56 +1242,84 @@ __global__ void __launch_bounds__(kAnyWarps * 32, 4) k_enc_levels_any(EncParams 
             const float4 g = __ldg(reinterpret_cast<const float4 *>(cs[j] + c));
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-              acc[i][j] = fmaf(f[i].x, g.x, acc[i][j]);
-              acc[i][j] = fmaf(f[i].y, g.y, acc[i][j]);
-              acc[i][j] = fmaf(f[i].z, g.z, acc[i][j]);
-              acc[i][j] = fmaf(f[i].w, g.w, acc[i][j]);
+              pair[i][j] = __ffma2_rn(make_float2(f[i].x, f[i].y), make_float2(g.x, g.y), pair[i][j]);
+              pair[i][j] = __ffma2_rn(make_float2(f[i].z, f[i].w), make_float2(g.z, g.w), pair[i][j]);
             }
           }
         }
+        float acc[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[i][j] = pair[i][j].x + pair[i][j].y;
+        // bound on |a - a64|, a the unscaled sum (c = a 2 / N), per window
+        float eb[4];
+        bool finite = true;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const uint32_t w = wg + i * wgs;
-          if (w >= nw) continue;
           const float su = sums[w] + sums[tile + w], sv = sums[2 * tile + w] + sums[3 * tile + w];
-          const bool finite = su + sv <= 1.0e38f;
-          // bound on |a - a64|, a the unscaled sum (c = a 2 / N)
-          const float eb = (odd ? sv : su) * ((float)(P + 4) * 0x1p-24f) + (su + sv) * 0x1p-40f + 1e-28f;
+          eb[i] = (odd ? sv : su) * ((float)(P + 4) * 0x1p-24f) + (su + sv) * 0x1p-40f + 1e-28f;
+          finite = finite && (su + sv <= 1.0e38f || w >= nw);
+        }
+        if (d.z1_f32 && B1 <= kAnyTile0 && finite) {
+          // every bin as one of zone 1, branch-free as in tier1_bins_fast; the others
+          // masked (zone 0 is mapped below and written over this)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const uint32_t k = k0 + 2 * j;
-            if (k >= E) continue;
-            if (k < B1 && k < kAnyTile0) {
-              z0[w * kAnyTile0 + k] = acc[i][j];
-              continue;
+          for (int i = 0; i < 4; ++i) {
+            const uint32_t w = wg + i * wgs;
+            const float base = eb[i] + d.u1_slack;
+            uint8_t *const out = lev + w * E + k0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const uint32_t k = k0 + 2 * j;
+              const float ak = fabsf(acc[i][j]);
+              const float m = fmaf(ak, 0x1p-21f, base);
+              const float lo = ak - m, hi = ak + m;
+              const bool dz = hi < d.u1_d1, edge = lo <= d.u1_d1, pos = acc[i][j] > 0.0f;
+              const float kk = pos ? d.u1_kp : d.u1_kn;
+              const int v0 = __float2int_rd(fmaf(fminf(lo, d.u1_A1) - d.u1_d1, kk, 0.5f));
+              const int v1 = __float2int_rd(fmaf(fminf(hi, d.u1_A1) - d.u1_d1, kk, 0.5f));
+              const bool und = !dz && (edge || v0 != v1) && k >= B1 && k < B2 && w < nw;
+              undecided |= und ? 1u << (4 * i + j) : 0u;
+              if (k < E) out[2 * j] = (uint8_t)(dz || k >= B2 ? 128u : und ? 0u : (uint32_t)(pos ? 129 + v0 : 127 - v0));
+              if (j < 2 && k < B1) z0[w * kAnyTile0 + k] = acc[i][j];  // k < 4: j = 0, 1
             }
-            uint32_t L = 128u;
-            bool und = false;
-            if (k < B2) {
-              if (!finite) {
-                und = true;
-              } else if (k < B1) {
-                const float c = acc[i][j] * d.two_over_n;
-                const float m = eb * d.two_over_n + d.slack0 + fabsf(c) * 0x1p-21f;
-                L = zone0_level32(c - m, d);
-                und = L != zone0_level32(c + m, d);
-              } else if (d.z1_f32) {  // as in tier1_bins_fast
-                const float ak = fabsf(acc[i][j]);
-                const float m = eb + d.u1_slack + ak * 0x1p-21f;
-                const float lo = ak - m, hi = ak + m;
-                const bool dz = hi < d.u1_d1, edge = lo <= d.u1_d1, pos = acc[i][j] > 0.0f;
-                const float kk = pos ? d.u1_kp : d.u1_kn;
-                const int v0 = __float2int_rd(fmaf(fminf(lo, d.u1_A1) - d.u1_d1, kk, 0.5f));
-                const int v1 = __float2int_rd(fmaf(fminf(hi, d.u1_A1) - d.u1_d1, kk, 0.5f));
-                und = !dz && (edge || v0 != v1);
-                L = dz ? 128u : (uint32_t)(pos ? 129 + v0 : 127 - v0);
-              } else {
-                const float c = acc[i][j] * d.two_over_n;
-                und = !zone1_decide32(c, eb * d.two_over_n + d.slack1 + fabsf(c) * 0x1p-21f, d, L);
+          }
+        } else {
+#pragma unroll 1
+          for (int i = 0; i < 4; ++i) {
+            const uint32_t w = wg + i * wgs;
+            if (w >= nw) continue;
+            const float su = sums[w] + sums[tile + w], sv = sums[2 * tile + w] + sums[3 * tile + w];
+            const bool fin = su + sv <= 1.0e38f;
+            const float e = i == 0 ? eb[0] : i == 1 ? eb[1] : i == 2 ? eb[2] : eb[3];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const uint32_t k = k0 + 2 * j;
+              if (k >= E) continue;
+              const float a = i == 0 ? acc[0][j] : i == 1 ? acc[1][j] : i == 2 ? acc[2][j] : acc[3][j];
+              if (k < B1 && k < kAnyTile0) {
+                z0[w * kAnyTile0 + k] = a;
+                continue;
               }
+              uint32_t L = 128u;
+              bool und = false;
+              if (k < B2) {
+                const float c = a * d.two_over_n;
+                if (!fin) {
+                  und = true;
+                } else if (k < B1) {
+                  const float m = e * d.two_over_n + d.slack0 + fabsf(c) * 0x1p-21f;
+                  L = zone0_level32(c - m, d);
+                  und = L != zone0_level32(c + m, d);
+                } else {
+                  und = !zone1_decide32(c, e * d.two_over_n + d.slack1 + fabsf(c) * 0x1p-21f, d, L);
+                }
+              }
+              undecided |= und ? 1u << (4 * i + j) : 0u;
+              lev[w * E + k] = (uint8_t)(und ? 0u : L);
             }
-            undecided |= und ? 1u << (4 * i + j) : 0u;
-            lev[w * E + k] = (uint8_t)(und ? 0u : L);
           }
         }
       }
@@ -1359,6 +1389,8 @@ __global__ void __launch_bounds__(kAnyWarps * 32, 4) k_enc_levels_any(EncParams 
 // The listed bins, one per thread: from their compensated FP32 coefficient
 // where its bound settles the level, else from their FP64 coefficient.
 __global__ void __launch_bounds__(256) k_enc_fallback(EncParams p) {
+  dependents_may_start();
+  dependency_wait();  // the list
   const unsigned int n = min(*p.fb_count, p.fb_cap);
   for (unsigned int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const unsigned long long e = p.fb_list[i];
@@ -1392,6 +1424,7 @@ __global__ void __launch_bounds__(kPackWarps * 32) k_enc_pack(EncParams p) {
     for (uint32_t i = threadIdx.x; i < p.n_doms * 256u; i += kPackWarps * 32) code_s[i] = __ldg(p.code_tab + i);
     __syncthreads();
   }
+  dependency_wait();  // the scan
   const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
   const uint64_t item = (uint64_t)blockIdx.x * kPackWarps + wid, b = item / (kPackBlock / kPackPart);
   const uint32_t part = (uint32_t)(item % (kPackBlock / kPackPart));
@@ -1765,6 +1798,10 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
     if (err == cudaSuccess)
       err = cudaFuncSetAttribute(k_enc_starts<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (kStartWarps + 1) * kStartWarpBytes + kTabDomains * 1024u);
+    // four CTAs an SM
+    if (err == cudaSuccess)
+      err = cudaFuncSetAttribute(k_enc_starts<true>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 (int)cudaSharedmemCarveoutMaxShared);
     if (err == cudaSuccess) err = cudaMalloc(&e->d_recs, std::max<uint64_t>(blocks, 1) * sizeof(PackRec));
     if (err == cudaSuccess) err = cudaMalloc(&e->d_masks, std::max<uint64_t>(blocks, 1) * kMaskWords * 4);
     if (err == cudaSuccess) err = cudaMalloc(&e->d_first_word, std::max<uint64_t>(blocks, 1) * 8);
@@ -1824,6 +1861,7 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
     e->fb_cap = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(lv / 16, 4096), uint64_t(1) << 28);
     if (err == cudaSuccess) err = cudaMalloc(&e->d_fb_list, (size_t)e->fb_cap * sizeof(unsigned long long));
     if (err == cudaSuccess) err = cudaMalloc(&e->d_fb_count, sizeof(unsigned int));
+    if (err == cudaSuccess) err = cudaMemset(e->d_fb_count, 0, sizeof(unsigned int));
     if (err == cudaSuccess) {
       const EncStatus s0{0u, 0u, ~0ull};
       err = enc_upload(&e->d_status, &s0, 1);
@@ -1891,48 +1929,37 @@ static fptc_status enc_run(fptc_encoder *enc, const float *d_x, bool levels_give
   EncParams p = enc_params(enc, d_words, d_symlen, d_n_words, lev);
   p.x = d_x;
   cudaError_t e = cudaSuccess;
-  if (!levels_given && enc->n_levels) {
-    e = cudaMemsetAsync(enc->d_fb_count, 0, sizeof(unsigned int), s);
-    if (e == cudaSuccess) {
-      if (enc->w32) {
-        // kLvGroups groups a warp, or as many as leave every warp the chip can hold (20 an SM) one
-        const uint64_t all = (enc->n_windows + 31) / 32, warps = (uint64_t)enc->sm_count * 20u;
-        const uint32_t groups = (uint32_t)std::min<uint64_t>(kLvGroups, (all + warps - 1) / warps);
-        const uint64_t per = (uint64_t)kLvThreads * groups;
-        k_enc_levels_w32<<<(unsigned)((enc->n_windows + per - 1) / per), kLvThreads, 0, s>>>(p, enc->n_windows, groups);
-      } else {
-        k_enc_levels_any<<<(unsigned)((enc->n_units + kAnyWarps - 1) / kAnyWarps), kAnyWarps * 32,
-                           kAnyWarps * enc->any_warp_bytes, s>>>(p, enc->n_units, enc->any_warp_bytes);
-      }
-      e = cudaGetLastError();
+  // each kernel may start beside the one before it and waits for it where its outputs are read
+  auto launch = [&](const void *kernel, uint64_t grid, uint32_t threads, size_t smem, bool overlap) {
+    if (e != cudaSuccess) return;
+    void *args[] = {&p};
+    e = launch_after(kernel, (uint32_t)grid, threads, args, smem, s, overlap);
+  };
+  const bool levels = !levels_given && enc->n_levels;
+  if (levels) {
+    if (enc->w32) {
+      // kLvGroups groups a warp, or as many as leave every warp the chip can hold (20 an SM) one
+      const uint64_t all = (enc->n_windows + 31) / 32, warps = (uint64_t)enc->sm_count * 20u;
+      const uint32_t groups = (uint32_t)std::min<uint64_t>(kLvGroups, (all + warps - 1) / warps);
+      const uint64_t per = (uint64_t)kLvThreads * groups;
+      k_enc_levels_w32<<<(unsigned)((enc->n_windows + per - 1) / per), kLvThreads, 0, s>>>(p, enc->n_windows, groups);
+    } else {
+      k_enc_levels_any<<<(unsigned)((enc->n_units + kAnyWarps - 1) / kAnyWarps), kAnyWarps * 32,
+                         kAnyWarps * enc->any_warp_bytes, s>>>(p, enc->n_units, enc->any_warp_bytes);
     }
-    if (e == cudaSuccess) {
-      k_enc_fallback<<<(unsigned)enc->sm_count * 8u, 256, 0, s>>>(p);
-      e = cudaGetLastError();
-    }
+    e = cudaGetLastError();
+    launch(reinterpret_cast<const void *>(&k_enc_fallback), (uint64_t)enc->sm_count * 8u, 256, 0, true);
   }
   const bool tab = enc->n_doms <= kTabDomains;
-  if (e == cudaSuccess && enc->n_blocks) {
-    const unsigned grid = (unsigned)((enc->n_blocks + kStartWarps - 1) / kStartWarps);
-    const size_t smem = (kStartWarps + 1) * kStartWarpBytes + (tab ? enc->n_doms * 1024u : 0u);
-    if (tab)
-      k_enc_starts<true><<<grid, (kStartWarps + 1) * 32, smem, s>>>(p);
-    else
-      k_enc_starts<false><<<grid, (kStartWarps + 1) * 32, smem, s>>>(p);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) {
-    k_enc_scan<<<(unsigned)((enc->n_segs * 32 + 127) / 128), 128, 0, s>>>(p);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess && enc->n_blocks) {
-    const unsigned grid = (unsigned)((enc->n_blocks * (kPackBlock / kPackPart) + kPackWarps - 1) / kPackWarps);
-    if (tab)
-      k_enc_pack<true><<<grid, kPackWarps * 32, enc->n_doms * 1024u, s>>>(p);
-    else
-      k_enc_pack<false><<<grid, kPackWarps * 32, 0, s>>>(p);
-    e = cudaGetLastError();
-  }
+  if (enc->n_blocks)
+    launch(tab ? reinterpret_cast<const void *>(&k_enc_starts<true>) : reinterpret_cast<const void *>(&k_enc_starts<false>),
+           (enc->n_blocks + kStartWarps - 1) / kStartWarps, (kStartWarps + 1) * 32,
+           (kStartWarps + 1) * kStartWarpBytes + (tab ? enc->n_doms * 1024u : 0u), levels);
+  launch(reinterpret_cast<const void *>(&k_enc_scan), (enc->n_segs * 32 + 127) / 128, 128, 0, enc->n_blocks > 0);
+  if (enc->n_blocks)
+    launch(tab ? reinterpret_cast<const void *>(&k_enc_pack<true>) : reinterpret_cast<const void *>(&k_enc_pack<false>),
+           (enc->n_blocks * (kPackBlock / kPackPart) + kPackWarps - 1) / kPackWarps, kPackWarps * 32,
+           tab ? enc->n_doms * 1024u : 0u, true);
   if (e != cudaSuccess) return enc_cuda_fail(e, "encode launch");
   return FPTC_OK;
 }
