@@ -22,7 +22,7 @@ constexpr uint32_t kChunkWords = 496;
 __host__ __device__ constexpr uint64_t chunks_of(uint64_t n) { return n ? ((n + 15) / 16 + 1 + 30) / 31 : 0; }
 // Chunks a warp of the index kernel takes at once (a group; groups do not cross
 // segments).
-constexpr uint32_t kGroupChunks = 8;
+constexpr uint32_t kGroupChunks = 4;
 __host__ __device__ constexpr uint64_t groups_of(uint64_t chunks) { return (chunks + kGroupChunks - 1) / kGroupChunks; }
 constexpr uint32_t kMaxLmax = 16;
 constexpr uint32_t kChunkBad = 0xFFFFFFFFu;  // chunk sum sentinel: a symlen > 64 was seen
@@ -86,6 +86,7 @@ struct SegDev {
   uint32_t out_aligned;  // bit 0: out_offset % 4 == 0 (16-byte stores), bit 1: % 8 (32-byte), bit 2: % 32 (128-byte rows)
   uint32_t queue_index;  // position in tile-queue order (seg_bad)
   uint32_t pad;
+  uint64_t n_symbols;    // n_windows times the domain's E
 };
 
 // Start of a tile in the SymLen stream: the word holding the tile's first symbol
@@ -102,8 +103,10 @@ struct DevStatus {
   unsigned long long first_bad;  // smallest caller index of a bad segment
 };
 
-// A group of index chunks: its segment (queue index) and first chunk in it.
+// A group of index chunks: its segment (queue index) and first chunk in it, and
+// what its loads need of the segment.
 struct IndexGroup {
+  uint64_t word_offset, n_words;
   uint32_t seg;
   uint32_t chunk;
 };

@@ -1,7 +1,7 @@
 // SymLen segment indexing (Sec. 4.2.1: an exclusive prefix sum over the symlen
 // array gives every compressed word the output position of its first symbol).
 //
-//   1. k_index: a warp per group of 8 chunks of a segment sums each chunk's
+//   1. k_index: a warp per group of 4 chunks of a segment sums each chunk's
 //      symlen (and checks that none exceeds 64); the warp that counts a
 //      segment's last group scans the segment's chunk sums into chunk offsets
 //      and checks the total against W*E.  No CTA waits on another: the last
@@ -12,7 +12,7 @@
 // The decode kernels then start each tile without decoding earlier words.
 //
 // A few MB are read, so k_index is bound by the dependent loads of a warp:
-// group, segment, symlen (eight chunks at once).  Two kernels, one finding its
+// group, then segment and symlen (four chunks) at once.  Two kernels, one finding its
 // segment by a binary search, took 16 us for the 13 M words of a mixed batch and
 // 23 us for 16,384 streams of 370 words; this one 8 and 15 us, and the decode
 // kernel behind it loads its tables meanwhile (launch_after).
@@ -74,7 +74,7 @@ __device__ __forceinline__ void load_group(const IndexParams &p, uint64_t c, uin
 // claims more than 64 symbols: its flag and the plan's status.
 __device__ __forceinline__ void close_segment(const IndexParams &p, uint32_t s, const SegDev &sg, uint64_t total,
                                               bool range_bad, uint32_t lane) {
-  const bool count_bad = total != sg.n_windows * (uint64_t)p.domains[sg.domain].E;
+  const bool count_bad = total != sg.n_symbols;
   if (lane == 0) {
     p.seg_bad[s] = (range_bad || count_bad) ? 1u : 0u;
     if (range_bad) flag_bad(p.status, kFlagSymlenRange, sg.caller_index);
@@ -97,22 +97,25 @@ __global__ void __launch_bounds__(256) k_index(IndexParams p) {
   const uint32_t lane = threadIdx.x & 31;
   const uint64_t g = p.group_begin + (uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (g >= p.group_end) return;  // the whole warp
-  uint32_t s, c0;
+  // the group names its segment's words, so that the symlen and the segment's
+  // record are requested together
+  IndexGroup r;
   if (p.groups) {
-    const IndexGroup r = p.groups[g];
-    s = r.seg;
-    c0 = r.chunk;
+    r = p.groups[g];
   } else {
     const uint32_t b = p.seg_begin;
-    s = b + (uint32_t)warp_last_leq(p.seg_end - b, g, lane, [&](uint64_t i) { return p.segs[b + i].group_base; });
-    c0 = (uint32_t)(g - p.segs[s].group_base) * kGroupChunks;
+    r.seg = b + (uint32_t)warp_last_leq(p.seg_end - b, g, lane, [&](uint64_t i) { return p.segs[b + i].group_base; });
+    r.chunk = (uint32_t)(g - p.segs[r.seg].group_base) * kGroupChunks;
+    r.word_offset = p.segs[r.seg].word_offset;
+    r.n_words = p.segs[r.seg].n_words;
   }
-  const SegDev &sg = p.segs[s];
-  const uint32_t n_chunks = sg.n_chunks, n = n_chunks - c0 < kGroupChunks ? n_chunks - c0 : kGroupChunks;
+  const uint32_t s = r.seg, c0 = r.chunk;
+  const SegDev sg = p.segs[s];
   uint4 v[kGroupChunks];
 #pragma unroll
-  for (uint32_t i = 0; i < kGroupChunks; ++i)
-    v[i] = i < n ? load_block(p.symlen, sg, c0 + i, lane).v : make_uint4(0u, 0u, 0u, 0u);
+  for (uint32_t i = 0; i < kGroupChunks; ++i)  // all zero past the segment's end
+    v[i] = load_block(p.symlen, r.word_offset, r.n_words, c0 + i, lane).v;
+  const uint32_t n_chunks = sg.n_chunks, n = n_chunks - c0 < kGroupChunks ? n_chunks - c0 : kGroupChunks;
   uint32_t sum = 0u, over = 0u;  // lane i: chunk i's sum and whether a word of it claims more than 64
 #pragma unroll
   for (uint32_t i = 0; i < kGroupChunks; ++i) {

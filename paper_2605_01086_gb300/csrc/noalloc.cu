@@ -155,6 +155,7 @@ extern "C" fptc_status fptc_decode_stream_noalloc(const fptc_domain *domain, con
   sg.out_offset = 0;
   sg.level_offset = 0;
   sg.n_windows = W;
+  sg.n_symbols = W * dm.E;
   sg.tile_base = 0;
   sg.n_tiles = (W + dd.tile_windows - 1) / dd.tile_windows;
   sg.chunk_base = 0;

@@ -898,6 +898,7 @@ fptc_status fptc_plan_create(fptc_plan **out, int device, const fptc_domain *dom
       sd.out_offset = s.out_offset;
       sd.level_offset = p->level_off[ci];
       sd.n_windows = (s.n_samples + d.N - 1) / d.N;
+      sd.n_symbols = sd.n_windows * d.E;
       sd.domain = s.domain;
       sd.caller_index = ci;
       sd.queue_index = (uint32_t)qi;
@@ -907,7 +908,7 @@ fptc_status fptc_plan_create(fptc_plan **out, int device, const fptc_domain *dom
       sd.n_chunks = (uint32_t)chunks_of(s.n_words);
       chunk += sd.n_chunks;
       sd.group_base = groups.size();
-      for (uint32_t c = 0; c < sd.n_chunks; c += kGroupChunks) groups.push_back(IndexGroup{(uint32_t)qi, c});
+      for (uint32_t c = 0; c < sd.n_chunks; c += kGroupChunks) groups.push_back(IndexGroup{s.word_offset, s.n_words, (uint32_t)qi, c});
     }
     p->n_chunks = chunk;
     p->n_groups = groups.size();

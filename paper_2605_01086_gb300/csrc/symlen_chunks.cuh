@@ -25,13 +25,14 @@ struct LaneBlock {
   uint64_t word0;
 };
 
-// Block 31 k - 1 + lane of segment sg (lane < 31).
-__device__ __forceinline__ LaneBlock load_block(const uint8_t *symlen, const SegDev &sg, uint64_t k, uint32_t lane) {
+// Block 31 k - 1 + lane (lane < 31) of the segment of n_words words from word_offset on.
+__device__ __forceinline__ LaneBlock load_block(const uint8_t *symlen, uint64_t word_offset, uint64_t n_words,
+                                                uint64_t k, uint32_t lane) {
   LaneBlock r;
-  const uintptr_t a0 = reinterpret_cast<uintptr_t>(symlen + sg.word_offset);
-  const uintptr_t a1 = a0 + sg.n_words;
+  const uintptr_t a0 = reinterpret_cast<uintptr_t>(symlen + word_offset);
+  const uintptr_t a1 = a0 + n_words;
   const uintptr_t blk = ((a0 + 15) & ~uintptr_t(15)) + 16 * (uintptr_t)(31 * k + lane) - 16;
-  r.word0 = sg.word_offset + (uint64_t)(blk - a0);  // wraps below word_offset for block -1 (masked bytes)
+  r.word0 = word_offset + (uint64_t)(blk - a0);  // wraps below word_offset for block -1 (masked bytes)
   if (lane < 31 && blk >= a0 && blk + 16 <= a1) {
     r.v = __ldg(reinterpret_cast<const uint4 *>(blk));
   } else {
@@ -46,6 +47,10 @@ __device__ __forceinline__ LaneBlock load_block(const uint8_t *symlen, const Seg
     r.v = make_uint4(w[0], w[1], w[2], w[3]);
   }
   return r;
+}
+
+__device__ __forceinline__ LaneBlock load_block(const uint8_t *symlen, const SegDev &sg, uint64_t k, uint32_t lane) {
+  return load_block(symlen, sg.word_offset, sg.n_words, k, lane);
 }
 
 __device__ __forceinline__ uint32_t block_sum(const uint4 &v) {
