@@ -25,12 +25,15 @@
 //  * otherwise (shape_pairs): a window's samples as ceil(N / 2) mirrored pairs
 //        x[n] = Ev[n] + Od[n],  x[N - 1 - n] = Ev[n] - Od[n],
 //    Ev / Od the sums over even / odd bins, as a small matrix product per step: the
-//    step's coefficients are dequantized once into shared memory, each twice in a
-//    row, and a lane takes four windows by eight pairs, two pairs per
-//    instruction (fma.f32x2): 16 of those for four 16-byte reads.  One lane per
+//    step's coefficients are dequantized once into shared memory, and a lane takes
+//    four windows by eight pairs, two pairs per instruction (fma.f32x2): 16 of
+//    those for three 16-byte reads.  Bound by shared-memory wavefronts (a 16-byte
+//    read is four of them, whatever it shares).  One lane per
 //    16 pairs of one window, with a basis read for every four multiply-adds and
 //    the coefficients dequantized again by each lane of a window, took 228 us for
-//    33 M samples at N = 100, E = 50; this takes 133 us.
+//    33 M samples at N = 100, E = 50; this form takes 114 us (133 us with each
+//    coefficient stored twice and a lane's windows side by side, when rows of 24,
+//    48 or 64 samples met in the same banks: N = 24, E = 12 took 117 us, now 83).
 #pragma once
 
 #include <cuda.h>
@@ -76,8 +79,8 @@ __host__ __device__ constexpr uint32_t shape_pair_windows(uint32_t tiles) { retu
 
 // Windows per output step.  Compiled forms: 32 lanes, 32 / N windows each for N
 // < 32.  shape_pairs: as many groups of its windows as lanes for their groups
-// of eight pairs, less where the coefficients (twice) or the samples would not
-// fit the warp's output tiles.  Either way at most 2048 symbols.
+// of eight pairs, less where the coefficients or the samples would not fit the
+// warp's output tiles.  Either way at most 2048 symbols.
 __host__ __device__ constexpr uint32_t shape_step(uint32_t N, uint32_t E, uint32_t kz, uint32_t tiles) {
   uint32_t w = 0;
   if (shape_form(N, kz, tiles)) {
@@ -86,7 +89,7 @@ __host__ __device__ constexpr uint32_t shape_step(uint32_t N, uint32_t E, uint32
     const uint32_t bytes = tiles * (uint32_t)kOutTile;
     const uint32_t m = shape_pair_windows(tiles);
     w = 32 / (shape_pairs8(N) / 8) * m;
-    const uint32_t fit_c = bytes / (8 * (kz ? kz : 1)) / 4 * 4, fit_x = bytes / (4 * N) / 4 * 4;
+    const uint32_t fit_c = bytes / (4 * (kz ? kz : 1)) / 4 * 4, fit_x = bytes / (4 * N) / 4 * 4;
     w = w < fit_c ? w : fit_c;
     w = w < fit_x ? w : fit_x;
   }
@@ -146,12 +149,15 @@ __device__ __forceinline__ uint32_t load_shape_tables(const DecodeParams &p, uin
       deq[i] = L < 256u ? (z == 0 ? a0 : a1) * dm.unit[z][L] : 0.0f;
     }
     if (form) continue;
-    // the half basis B[k][n], n < ceil(N / 2), zero up to the next eight
+    // the half basis B[k][n], n < ceil(N / 2), zero up to the next eight; a row holds
+    // the first four of every eight, then the second four (consecutive groups of
+    // pairs in consecutive 16 bytes)
     float *bas = reinterpret_cast<float *>(smem + basis_off);
     const float *g_bas = p.basis + dm.basis_offset;
     const uint32_t pairs = shape_pair_count(N);
     for (uint32_t i = threadIdx.x; i < kz * p8; i += THREADS) {
-      const uint32_t k = i / p8, n = i - k * p8;
+      const uint32_t k = i / p8, r = i - k * p8, h = r < p8 / 2 ? 0u : 1u, q = r - h * (p8 / 2);
+      const uint32_t n = q / 4 * 8 + 4 * h + q % 4;
       bas[i] = n < pairs ? __ldg(g_bas + (size_t)k * N + n) : 0.0f;
     }
   }
@@ -475,19 +481,21 @@ __device__ __forceinline__ void shape_pairs(const DecodeParams &p, const UnitSeg
                                             const unsigned char *smem, const uint8_t *lv0, uint64_t win, uint32_t n,
                                             const ShapeOut &o) {
   const uint32_t lane = o.lane, N = dd.N, P = shape_pair_count(N), p8 = shape_pairs8(N), kz = dd.kz;
-  const uint32_t Ws = (dd.step + 3) / 4 * 4;  // rows of coefficients
+  // lanes' windows lie G apart (rows that are multiples of 32 samples apart would
+  // share their banks): place MW g + i of a bin's coefficients is window g + G i
+  const uint32_t Ws = (dd.step + 3) / 4 * 4, G = Ws / MW;
   const float *deq = reinterpret_cast<const float *>(smem + dd.deq_off);
   const float *bas = reinterpret_cast<const float *>(smem + dd.basis_off);
   if (lane == 0) tma_wait_read_but<0>();  // earlier steps have left the tiles
   __syncwarp();
   // ---- coefficients, lanes along the windows
   {
-    float2 *const cs = reinterpret_cast<float2 *>(o.otile);
+    float *const cs = reinterpret_cast<float *>(o.otile);
     const uint32_t dk = 32 / Ws, dw = 32 - dk * Ws;
     uint32_t k = lane / Ws, w = lane - k * Ws;
     for (uint32_t i = lane; i < kz * Ws; i += 32) {
-      const float c = w < n ? deq[(k < dd.B1 ? 0 : kZStride) + lv0[w * dd.E + k]] : 0.0f;
-      cs[i] = make_float2(c, c);  // i = k Ws + w
+      const uint32_t ww = w / MW + G * (w % MW);
+      cs[i] = ww < n ? deq[(k < dd.B1 ? 0 : kZStride) + lv0[ww * dd.E + k]] : 0.0f;  // i = k Ws + w
       k += dk;
       w += dw;
       if (w >= Ws) {
@@ -499,26 +507,31 @@ __device__ __forceinline__ void shape_pairs(const DecodeParams &p, const UnitSeg
   __syncwarp();
   // ---- MW windows by eight pairs a lane
   const uint32_t pgs = p8 / 8, wg = lane / pgs, pg = lane - wg * pgs;
-  const bool mine = MW * wg < Ws;
+  const bool mine = wg < G;
   float2 ev[MW][4], od[MW][4];
 #pragma unroll
   for (int i = 0; i < MW; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) ev[i][j] = od[i][j] = make_float2(0.0f, 0.0f);
   if (mine) {
-    const float4 *cp = reinterpret_cast<const float4 *>(o.otile) + MW / 2 * wg;  // windows MW wg .. of bin 0
-    const float4 *bp = reinterpret_cast<const float4 *>(bas) + 2 * pg;
-    const uint32_t cstep = Ws / 2, bstep = p8 / 4;
+    const float *cp = reinterpret_cast<const float *>(o.otile) + MW * wg;  // the lane's windows, bin 0
+    const float4 *bp = reinterpret_cast<const float4 *>(bas) + pg;
+    const uint32_t bhalf = p8 / 8, bstep = p8 / 4;
     auto bin = [&](float2(&acc)[MW][4]) {
-      float2 c[MW];
-#pragma unroll
-      for (int i = 0; i < MW; i += 2) {
-        const float4 q = cp[i / 2];
-        c[i] = make_float2(q.x, q.y);
-        c[i + 1] = make_float2(q.z, q.w);
+      float2 c[MW];  // a window's coefficient in both halves
+      if constexpr (MW == 4) {
+        const float4 q = *reinterpret_cast<const float4 *>(cp);
+        c[0] = make_float2(q.x, q.x);
+        c[1] = make_float2(q.y, q.y);
+        c[2] = make_float2(q.z, q.z);
+        c[3] = make_float2(q.w, q.w);
+      } else {
+        const float2 q = *reinterpret_cast<const float2 *>(cp);
+        c[0] = make_float2(q.x, q.x);
+        c[1] = make_float2(q.y, q.y);
       }
-      const float4 b0 = bp[0], b1 = bp[1];
-      cp += cstep;
+      const float4 b0 = bp[0], b1 = bp[bhalf];
+      cp += Ws;
       bp += bstep;
       const float2 b[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y),
                            make_float2(b1.z, b1.w)};
@@ -540,8 +553,8 @@ __device__ __forceinline__ void shape_pairs(const DecodeParams &p, const UnitSeg
     const bool whole = N % 4 == 0 && 8 * pg + 8 <= P;
 #pragma unroll
     for (int i = 0; i < MW; ++i) {
-      if (MW * wg + i >= dd.step) break;
-      float *const x = reinterpret_cast<float *>(o.otile) + (MW * wg + i) * N;
+      if (wg + G * i >= dd.step) break;
+      float *const x = reinterpret_cast<float *>(o.otile) + (wg + G * i) * N;
       float f[8], m[8];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
