@@ -246,9 +246,13 @@ void layout_tiles(fptc_plan *p, uint32_t tile_samples) {
     choose_shape(p);
     for (const auto &dd : p->dom_dev) dearest = std::max(dearest, step_cost(dd));
   }
+  // the three-kernel schedule runs a block per tile: 4096 samples (with a step's 1024
+  // its blocks are four times as many and take 4 % longer)
+  const bool three = p->opts.schedule == FPTC_SCHEDULE_THREE_KERNEL;
+  if (three && p->kind == FPTC_KERNEL_WARP_TILE) tile_samples = std::max(tile_samples, 4096u);
   for (auto &dd : p->dom_dev) {
     dd.tile_windows = shape ? step_of(dd) * std::max<uint32_t>(1u, std::min<uint32_t>(
-                                                dearest / step_cost(dd),
+                                                three ? 4096u / (step_of(dd) * dd.N) : dearest / step_cost(dd),
                                                 std::min(8192u / (step_of(dd) * dd.N), 2048u / (step_of(dd) * dd.E))))
                             : std::max<uint32_t>(1u, tile_samples / dd.N);
     // the block adjoint takes up to 8192 samples and 2048 symbols of a segment's tiles together
@@ -1271,6 +1275,8 @@ fptc_status fptc_plan_autotune(fptc_plan *p, const uint64_t *d_words, const uint
     else if (keep.idct != FPTC_IDCT_FP32)
       for (uint32_t th : {256u, 384u, 512u, 640u, 768u, 896u})
         cands.push_back({FPTC_KERNEL_TENSOR, tc_tile_windows() * 32, th});
+    if (keep.idct == FPTC_IDCT_FP32 && p->shape)  // choose_shape's own count (it may be one that no option names)
+      cands.push_back({FPTC_KERNEL_WARP_TILE, 4096, 0u});
     for (uint32_t th : {128u, 256u, 512u, 768u, 896u, 1024u}) {
       if (keep.idct != FPTC_IDCT_FP32) continue;
       if (th > 512) {
