@@ -113,10 +113,9 @@ typedef enum fptc_kernel {
                                   else generic */
   FPTC_KERNEL_GENERIC = 1,     /* any N, E: one block per tile, basis through L1 */
   FPTC_KERNEL_BLOCK_TILE = 2,  /* N = 32, E = 16: one block per tile, pipelined */
-  FPTC_KERNEL_WARP_TILE = 3,   /* one warp per tile, no block barriers: N = 32, E = 16 (128-window tiles),
-                                  or any N in [4, 128] in every domain (several N in one batch; N not a
-                                  power of two stores with the lanes instead of TMA), any E <= N (tiles
-                                  of about 2048 symbols); at most 8 domains */
+  FPTC_KERNEL_WARP_TILE = 3,   /* a range of tiles per warp, no block barriers: N = 32, E = 16,
+                                  or any N in [4, 128] in every domain (several N in one batch), any
+                                  E <= N; at most 8 domains */
   FPTC_KERNEL_TENSOR = 4       /* tensor-core transform, chosen by idct != FPTC_IDCT_FP32: N = 32, E = 16
                                   in every domain, or one (N, E) in {(32, 32), (64, 32), (128, 32),
                                   (128, 64)} shared by every domain */
@@ -127,16 +126,16 @@ typedef struct fptc_plan_options {
   uint32_t schedule;      /* fptc_schedule */
   uint32_t tile_samples;  /* target output samples per tile (whole windows) of the block-tile and generic
                              kernels; 0 = 8192 for the block-tile kernel, else 4096.  The warp-tile and
-                             tensor-core kernels fix their tiles: 128 windows at N = 32, E = 16; at other
-                             shapes about 2048 symbols in whole 1024-sample steps (at most 8) */
+                             tensor-core kernels fix their tiles */
   uint32_t threads;       /* threads per CTA: 128, 256 or 512 (also 768, 896, 1024 for the warp-tile kernel
                              at N = 32, E = 16; 256, 512 or 768 for it at other shapes; 384, 640, 768 or
                              896 for the tensor-core kernel at N = 32, E = 16, whose other shapes fix their
                              own); 0 = 256, or for the warp-tile kernel 896 where its shared memory fits
-                             (28 warps, no register spills), else the most that fit (at most 512 at other
-                             shapes), and for the tensor-core kernel the most that fit shared and tensor
-                             memory (896; 640 for its 3xTF32 form); a count that does not fit is refused
-                             with FPTC_ERR_UNSUPPORTED */
+                             (28 warps, no register spills), else the most that fit (at other shapes 512,
+                             384 for several transforms in one plan or N = 128, else less), and for the
+                             tensor-core kernel the most that fit shared and tensor memory (896; 640 for
+                             its 3xTF32 form); a count that does not fit is refused with
+                             FPTC_ERR_UNSUPPORTED */
   uint32_t ctas_per_sm;   /* persistent CTAs per SM; 0 = as many as fit */
   uint32_t kernel;        /* fptc_kernel: which decode kernel; 0 = choose */
   uint32_t reserved[2];   /* must be 0 */

@@ -14,7 +14,7 @@
 // A few MB are read, so k_index is bound by the dependent loads of a warp:
 // group, then segment and symlen (four chunks) at once.  Two kernels, one finding its
 // segment by a binary search, took 16 us for the 13 M words of a mixed batch and
-// 23 us for 16,384 streams of 370 words; this one 8 and 15 us, and the decode
+// 23 us for 16,384 streams of 370 words; this one 8 and 12 us, and the decode
 // kernel behind it loads its tables meanwhile (launch_after).
 // k_tile_index runs one warp per chunk over a contiguous chunk range per warp
 // (the segment cursor advances with the chunk index), with the next chunks'

@@ -1,13 +1,14 @@
-// Shared machinery of the warp-tile decode kernels (FP32 transform in
-// decode_warp.cu, tensor-core transform in decode_tc.cu), for the Table 1 shape
-// N = 32, E = 16: tile constants, per-domain tables in shared memory, the
-// SymLen word decoder, tile contexts and their asynchronous prefetch, the
-// per-window dequantization, and the TMA store of 32-window output tiles.
-//
-// Each warp decodes a contiguous range of tiles.  The first tile of the range
-// is located from the index's chunk offsets (symbol_word); every later tile of
-// a segment starts at the word where the tile before it ended, which the SymLen
-// decode of that tile finds anyway, so no record per tile is read.
+// Shared machinery of the warp-tile kernels: tile constants and the per-window
+// dequantization of the Table 1 shape N = 32, E = 16, per-domain tables in
+// shared memory, the SymLen word decoder, the TMA store of 32-window output
+// tiles, and two ways for a warp to decode its contiguous range of tiles:
+//   * stream_tiles (decode_warp.cu, decode_shape.cuh): the range as one stream of
+//     passes; a step of the transform runs whenever its symbols are there;
+//   * decode_tile with its contexts and their asynchronous prefetch
+//     (decode_tc.cu, decode_tcs.cu, backward_warp.cu): one tile after the other,
+//     each starting at the word where the one before it ended.
+// Either way the first tile of the range is located from the index's chunk
+// offsets (symbol_word), and no record per tile is read.
 #pragma once
 
 #include <cuda.h>
