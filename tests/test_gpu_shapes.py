@@ -79,6 +79,22 @@ def test_shape_thread_counts(threads):
     compare_with_oracle(plan, b, out, lv)
 
 
+@pytest.mark.parametrize("N,Es", [(64, [32, 7]), (24, [12, 5]), (128, [128, 64])])
+def test_shape_tuned_and_three_kernel(N, Es):
+    """A tuned plan's options make a plan again, and the three-kernel schedule's tiles
+    (several of the shape kernel's steps) cover ragged streams: both within the
+    bounds of every other plan."""
+    from paper_2605_01086_gb300.tune_cache import plan_kwargs
+    b = _random_batch(N, Es, seed=11)
+    plan = make_plan(b, out_align=32)
+    w, s = plan.to_device(b.words, b.symlen)
+    best, _ = plan.autotune(w, s, plan.empty_out(), trials=1)
+    for p in (plan, make_plan(b, out_align=32, **plan_kwargs(best)),
+              make_plan(b, out_align=32, schedule="three_kernel")):
+        _, _, out, lv = gpu_decode(p, b)
+        compare_with_oracle(p, b, out, lv)
+
+
 def test_shape_default_choice():
     """Plans whose domains all have a power-of-two N get the warp-tile kernel by
     default, several N in one plan included, window sizes that are not a power
