@@ -11,15 +11,17 @@
 // memory, from where consecutive lanes write consecutive values and form
 // g_C * unit_z(level), added per lane and zone as an FP32 pair (two-sum) and per
 // warp in FP64, one atomic per warp, domain and zone.
-// Bound by instruction issue.  One thread per (window, bin) with an N-term dot
-// product from shared memory took 183 us for 16.8 M samples at N = 64, E = 32:
-// 89 us here.
+// Bound by latency with 16 warps per SM.  One thread per (window, bin) with an
+// N-term dot product from shared memory took 183 us for 16.8 M samples at N = 64,
+// E = 32; this took 89 us with a level loaded at a time (the largest stall by far),
+// and takes 65 us with eight of them in flight.
 #include "device_util.cuh"
 
 namespace fptc {
 namespace {
 
 constexpr uint32_t kBwWarps = 8;
+constexpr uint32_t kBwLevels = 8;  // of a lane's levels, loaded together
 
 __host__ __device__ constexpr uint32_t bw_pitch(uint32_t n) { return ((n + 3) / 4 | 1u) * 4; }  // odd number of 16-byte pieces
 __host__ __device__ constexpr uint32_t bw_pairs4(uint32_t N) { return ((N + 1) / 2 + 3) / 4 * 4; }
@@ -235,15 +237,21 @@ __global__ void __launch_bounds__(kBwWarps * 32, 2) k_backward_any(const Backwar
       }
       uint32_t k = lane % E;
       const uint32_t dk = 32 % E;
-      for (uint32_t i = lane; i < total; i += 32) {
-        const float g = gc[i];
-        const uint32_t L = __ldg(lv + i);
-        if (k < B1)
-          sum0.add(g, unit_tab[L]);
-        else if (k < B2)
-          sum1.add(g, unit_tab[256 + L]);
-        k += dk;
-        if (k >= E) k -= E;
+      for (uint32_t i0 = lane; i0 < total; i0 += 32 * kBwLevels) {
+        uint32_t L[kBwLevels];
+#pragma unroll
+        for (uint32_t j = 0; j < kBwLevels; ++j) L[j] = i0 + 32 * j < total ? __ldg(lv + i0 + 32 * j) : 0u;
+#pragma unroll
+        for (uint32_t j = 0; j < kBwLevels; ++j) {
+          if (i0 + 32 * j >= total) break;
+          const float g = gc[i0 + 32 * j];
+          if (k < B1)
+            sum0.add(g, unit_tab[L[j]]);
+          else if (k < B2)
+            sum1.add(g, unit_tab[256 + L[j]]);
+          k += dk;
+          if (k >= E) k -= E;
+        }
       }
       __syncwarp();
     }
