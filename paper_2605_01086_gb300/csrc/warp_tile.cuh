@@ -536,7 +536,8 @@ __device__ __forceinline__ uint32_t decode_pair(const PassWords &c, uint32_t n0,
 // step_windows(dd): windows of a whole step, whose symbols and a word's 64 are at
 // most CAP.
 // Barriers: step is entered with the levels visible to the warp; they are
-// rewritten only after a warp barrier.
+// rewritten only after a warp barrier of stream_tiles itself, so a step needs
+// none of its own behind its reads.
 template <int CAP, class Dom, class Geo, class Step>
 __device__ __forceinline__ void stream_tiles(const DecodeParams &p, uint64_t t0, uint64_t t1, const Dom *doms,
                                              const unsigned char *smem, uint8_t *stage, uint32_t lane, const Geo &geo,
@@ -657,6 +658,7 @@ __device__ __forceinline__ void stream_tiles(const DecodeParams &p, uint64_t t0,
       }
       more = !last;
       if (more && off) {  // the symbols left, to the front
+        __syncwarp();  // over levels the step has just read: not every step ends with a barrier (lane stores)
         const int32_t r = fill - off;  // fewer than a step's, so the two places do not overlap
         if ((off & 15) == 0) {
           for (int32_t at = 16 * (int32_t)lane; at < r; at += 512)

@@ -1,0 +1,31 @@
+"""Ordering rules of the CUDA sources whose violation no run on a GPU shows reliably
+(a race between lanes, a cached load), checked on the source text."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2605_01086_gb300", "csrc")
+
+
+def _source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def _body(src, head):
+    """Text of the brace block that follows the first match of `head`."""
+    at = src.index("{", re.search(head, src).end())
+    depth = 0
+    for i in range(at, len(src)):
+        depth += {"{": 1, "}": -1}.get(src[i], 0)
+        if depth == 0:
+            return src[at:i + 1]
+    raise AssertionError(head)
+
+
+def test_levels_are_rewritten_behind_a_barrier():
+    """stream_tiles moves the symbols left over the levels that the lanes of a step
+    read: a warp barrier lies between the last step and the first of those stores."""
+    body = _body(_source("warp_tile.cuh"), r"void stream_tiles\(")
+    after = body[body.rindex("step(sg, dd,"):]
+    first_store = min(m.start() for m in re.finditer(r"stage\s*\+\s*at\)\s*=[^=]|stage\[at\]\s*=[^=]", after))
+    assert "__syncwarp()" in after[:first_store]
