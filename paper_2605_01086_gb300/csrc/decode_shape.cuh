@@ -77,6 +77,11 @@ __host__ __device__ constexpr uint32_t shape_form(uint32_t N, uint32_t kz, uint3
 // 24 warps: 80 registers a thread, half of them accumulators at two).
 __host__ __device__ constexpr uint32_t shape_pair_windows(uint32_t tiles) { return tiles > 1 ? 4 : 2; }
 
+// Places a bin's coefficients take in shape_pairs for a step of `step` windows, m a
+// lane: whole lanes' worth (m is the width of their read), and no more: m times
+// the lane groups of a step, of which a warp has 32 / (groups of eight pairs).
+__host__ __device__ constexpr uint32_t shape_pair_places(uint32_t step, uint32_t m) { return (step + m - 1) / m * m; }
+
 // Windows per output step.  Compiled forms: 32 lanes, 32 / N windows each for N
 // < 32.  shape_pairs: as many groups of its windows as lanes for their groups
 // of eight pairs, less where the coefficients or the samples would not fit the
@@ -104,6 +109,33 @@ __host__ __device__ constexpr uint32_t shape_step(uint32_t N, uint32_t E, uint32
   }
   return w / q * q ? w / q * q : w;
 }
+
+// Whether every (window of a step, group of eight pairs) of shape_pairs has a lane,
+// and the step's coefficients and samples their place in the warp's output
+// tiles, for the window sizes [lo, hi] (a range the compiler evaluates at once).
+constexpr bool shape_pairs_covered(uint32_t tiles, uint32_t lo, uint32_t hi) {
+  for (uint32_t N = lo; N <= hi; ++N)
+    for (uint32_t E = 1; E <= N; ++E)
+      for (uint32_t kz = E; kz; kz /= 2) {
+        if (shape_form(N, kz, tiles)) continue;
+        const uint32_t m = shape_pair_windows(tiles), step = shape_step(N, E, kz, tiles);
+        const uint32_t places = shape_pair_places(step, m), bytes = tiles * (uint32_t)kOutTile;
+        if (step == 0 || places / m * (shape_pairs8(N) / 8) > 32) return false;
+        if (4 * kz * places > bytes || 4 * N * step > bytes) return false;
+      }
+  return true;
+}
+template <uint32_t LO, uint32_t HI>
+struct ShapePairsCheck {
+  static_assert(shape_pairs_covered(1, LO, HI), "a window's pairs without a lane");
+  static_assert(shape_pairs_covered(2, LO, HI), "a window's pairs without a lane");
+};
+template struct ShapePairsCheck<4, 48>;
+template struct ShapePairsCheck<49, 68>;
+template struct ShapePairsCheck<69, 84>;
+template struct ShapePairsCheck<85, 100>;
+template struct ShapePairsCheck<101, 115>;
+template struct ShapePairsCheck<116, 128>;
 
 // Symbols a warp's stage holds (stream_tiles): a step's and a pass's.
 __host__ __device__ constexpr int shape_cap(int tiles) { return tiles > 1 ? kTS + 1024 : kMiscBytes - stream_bytes(0); }
@@ -474,8 +506,9 @@ __device__ __forceinline__ void bulk_store(float *dst, const void *src, uint32_t
   asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
-// The pair form, any N: a step of n windows (at most dd.step), MW a lane.  The warp's output tiles hold the step's coefficients ([bin][window],
-// each twice) and then its samples (as they lie in the output).
+// The pair form, any N: a step of n windows (at most dd.step), MW a lane.  The
+// warp's output tiles hold the step's coefficients ([bin][place], each once) and
+// then its samples (as they lie in the output).
 template <int MW>
 __device__ __forceinline__ void shape_pairs(const DecodeParams &p, const UnitSeg &sg, const DomS &dd,
                                             const unsigned char *smem, const uint8_t *lv0, uint64_t win, uint32_t n,
@@ -483,7 +516,7 @@ __device__ __forceinline__ void shape_pairs(const DecodeParams &p, const UnitSeg
   const uint32_t lane = o.lane, N = dd.N, P = shape_pair_count(N), p8 = shape_pairs8(N), kz = dd.kz;
   // lanes' windows lie G apart (rows that are multiples of 32 samples apart would
   // share their banks): place MW g + i of a bin's coefficients is window g + G i
-  const uint32_t Ws = (dd.step + 3) / 4 * 4, G = Ws / MW;
+  const uint32_t Ws = shape_pair_places(dd.step, MW), G = Ws / MW;
   const float *deq = reinterpret_cast<const float *>(smem + dd.deq_off);
   const float *bas = reinterpret_cast<const float *>(smem + dd.basis_off);
   if (lane == 0) tma_wait_read_but<0>();  // earlier steps have left the tiles

@@ -291,3 +291,33 @@ def test_long_and_short_words(N, E):
         _, _, out, lv = gpu_decode(plan, b, out_fill=float("nan"))
         assert plan.device_status()[0] == 0
         compare_with_oracle(plan, b, out, lv)
+
+
+@pytest.mark.parametrize("N,Es", [(12, [5, 8]), (24, [9, 24]), (48, [7, 40]), (52, [13, 48]), (72, [8, 71]), (81, [41, 8]),
+                                  (84, [40, 81]), (85, [85, 48]), (88, [88, 33]), (96, [95, 16]), (100, [50, 33]),
+                                  (127, [64, 127])])
+@pytest.mark.parametrize("align", [32, 1])
+def test_pair_form_thread_counts(N, Es, align):
+    """The pair form with one to eight groups of eight pairs a window, with two output
+    tiles per warp (four windows a lane) and with one (two windows a lane: 768
+    threads, and other counts where two tiles do not fit): every window of a step,
+    every pair of it, bins of either parity last."""
+    b = _random_batch(N, Es, seed=N + align)
+    for threads in (0, 256, 512, 768):
+        plan = make_plan(b, out_align=align, out_base=0 if align == 32 else 3, kernel="warp_tile", threads=threads)
+        _, _, out, lv = gpu_decode(plan, b, out_fill=float("nan"))
+        compare_with_oracle(plan, b, out, lv)
+        assert plan.device_status()[0] == 0
+
+
+@pytest.mark.parametrize("N,E,n", [(84, 40, 3), (84, 40, 4), (81, 41, 3), (100, 50, 3), (127, 127, 2)])
+def test_pair_form_of_many_domains(N, E, n):
+    """Plans whose tables leave the default no room for two output tiles per warp."""
+    b = _random_batch(N, [E] * n, seed=N + n)
+    for d in b.domains:
+        d.lmax = 12  # decode tables of 8 KB a domain, the same codewords
+    plan = make_plan(b, out_align=32)
+    assert plan.info["kernel"] == WARP_TILE
+    _, _, out, lv = gpu_decode(plan, b, out_fill=float("nan"))
+    compare_with_oracle(plan, b, out, lv)
+    assert plan.device_status()[0] == 0
