@@ -145,8 +145,13 @@ __device__ __forceinline__ void dependents_may_start() { asm volatile("griddepco
 
 // cudaLaunchKernel, or, with overlap, a launch that may begin before the kernel
 // in front of it in the stream has ended: that must be a kernel of this library
-// which itself began after everything before it, and the launched kernel calls
-// dependency_wait before it touches anything but the plan's own tables.
+// which itself began after everything before it (or waited for what did), and the
+// launched kernel calls dependency_wait before it touches anything that a kernel
+// of the chain writes: before it, the plan's own tables and the caller's inputs
+// (words, symbol counts, samples, scales), which were complete before the chain
+// began.  What a kernel of the chain writes is never read through the read-only
+// path (__ldg): it is not read-only for as long as the reading kernel runs, nor
+// need such a load stay behind the wait.
 inline cudaError_t launch_after(const void *kernel, uint32_t grid, uint32_t threads, void **args, size_t smem,
                                 cudaStream_t stream, bool overlap) {
   if (!overlap) return cudaLaunchKernel(kernel, dim3(grid), dim3(threads), args, smem, stream);

@@ -656,21 +656,22 @@ constexpr uint32_t kTabDomains = 16;
 // 16 levels from i (a multiple of 16, i < n) of the run of n at lv, zero past
 // n: one vector load where the run is 16-byte aligned, else aligned 4-byte
 // words put together (bytes at the run's ends, where a word would reach
-// outside it).
+// outside it).  Here and below levels are read by plain loads: the grids
+// before may still be writing them when this one starts (launch_after).
 __device__ __forceinline__ uint4 load_run16(const uint8_t *lv, uint32_t i, uint32_t n) {
   const uintptr_t a = reinterpret_cast<uintptr_t>(lv + i);
-  if ((a & 15u) == 0 && i + 16 <= n) return __ldg(reinterpret_cast<const uint4 *>(a));
+  if ((a & 15u) == 0 && i + 16 <= n) return *reinterpret_cast<const uint4 *>(a);
   if (i != 0 && i + 20 <= n) {
     const uint32_t *w = reinterpret_cast<const uint32_t *>(a & ~uintptr_t(3));
     const uint32_t s = (uint32_t)(a & 3u) * 8u;
-    const uint32_t w0 = __ldg(w), w1 = __ldg(w + 1), w2 = __ldg(w + 2), w3 = __ldg(w + 3), w4 = __ldg(w + 4);
+    const uint32_t w0 = w[0], w1 = w[1], w2 = w[2], w3 = w[3], w4 = w[4];
     return make_uint4(__funnelshift_r(w0, w1, s), __funnelshift_r(w1, w2, s), __funnelshift_r(w2, w3, s),
                       __funnelshift_r(w3, w4, s));
   }
   uint32_t t[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
   for (int r = 0; r < 16; ++r)
-    if (i + r < n) t[r >> 2] |= (uint32_t)__ldg(lv + i + r) << (8 * (r & 3));
+    if (i + r < n) t[r >> 2] |= (uint32_t)lv[i + r] << (8 * (r & 3));
   return make_uint4(t[0], t[1], t[2], t[3]);
 }
 
@@ -885,7 +886,7 @@ __global__ void __launch_bounds__((kStartWarps + 1) * 32, 4) k_enc_starts(EncPar
         each16(q, [&](int j, uint32_t level) { m |= start(level) ? 1u << j : 0u; });
       } else {  // the stream's last symbols
 #pragma unroll 1
-        for (uint32_t j = 0; 16 * v + j < n; ++j) m |= start((uint32_t)__ldg(lv + 16 * v + j)) ? 1u << j : 0u;
+        for (uint32_t j = 0; 16 * v + j < n; ++j) m |= start((uint32_t)lv[16 * v + j]) ? 1u << j : 0u;
       }
       cnt += __popc(m);
       bits[v] = (uint16_t)m;
@@ -932,7 +933,7 @@ __device__ void walk_block(const EncParams &p, const EncSeg &sg, const EncDomain
   const uint8_t *lv = p.levels + sg.level_offset + i0;
   const uint32_t *tab = p.code_tab + sg.domain * 256u;
   uint32_t *row = p.masks + b * kMaskWords;
-  auto fetch = [&](uint32_t at) -> uint32_t { return at + lane < nb ? (uint32_t)__ldg(lv + at + lane) : 0u; };
+  auto fetch = [&](uint32_t at) -> uint32_t { return at + lane < nb ? (uint32_t)lv[at + lane] : 0u; };
   uint32_t cur = fetch(0), v = 64u - u;
   for (uint32_t at = 0; at < nb; at += 32) {
     const uint32_t nxt = fetch(at + 32);
@@ -1448,12 +1449,12 @@ __global__ void __launch_bounds__(kPackWarps * 32) k_enc_pack(EncParams p) {
     const uintptr_t a = a0 - sh + c;
     uint4 q = make_uint4(0u, 0u, 0u, 0u);
     if (a >= lo && a + 16 <= hi) {
-      q = __ldg(reinterpret_cast<const uint4 *>(a));
+      q = *reinterpret_cast<const uint4 *>(a);
     } else {  // the stream's ends: nothing outside it is read
       uint32_t t[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
       for (int r = 0; r < 16; ++r)
-        if (a + r >= lo && a + r < hi) t[r >> 2] |= (uint32_t)__ldg(reinterpret_cast<const uint8_t *>(a + r)) << (8 * (r & 3));
+        if (a + r >= lo && a + r < hi) t[r >> 2] |= (uint32_t)*reinterpret_cast<const uint8_t *>(a + r) << (8 * (r & 3));
       q = make_uint4(t[0], t[1], t[2], t[3]);
     }
     *reinterpret_cast<uint4 *>(stage + c) = q;

@@ -29,3 +29,14 @@ def test_levels_are_rewritten_behind_a_barrier():
     after = body[body.rindex("step(sg, dd,"):]
     first_store = min(m.start() for m in re.finditer(r"stage\s*\+\s*at\)\s*=[^=]|stage\[at\]\s*=[^=]", after))
     assert "__syncwarp()" in after[:first_store]
+
+
+def test_levels_of_overlapped_encoder_kernels_are_plain_loads():
+    """k_enc_starts, k_enc_scan and k_enc_pack may start while the level kernels
+    still write: what they read through the read-only path is the code table and
+    nothing else."""
+    src = _source("encode.cu")
+    table = re.compile(r"__ldg\((p\.code_tab|gt|tab)\b")
+    for head in (r"uint4 load_run16\(", r"k_enc_starts\(", r"void walk_block\(", r"k_enc_scan\(", r"k_enc_pack\("):
+        body = _body(src, head)
+        assert len(re.findall(r"__ldg\(", body)) == len(table.findall(body)), head
