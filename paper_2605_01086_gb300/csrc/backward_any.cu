@@ -11,6 +11,12 @@
 // memory, from where consecutive lanes write consecutive values and form
 // g_C * unit_z(level), added per lane and zone as an FP32 pair (two-sum) and per
 // warp in FP64, one atomic per warp, domain and zone.
+// A batch with fewer tiles than the chip has warps is split into parts of tiles
+// (backward_any_split), and a CTA loads the tables of its own segments' domains
+// only: with whole tiles per warp and every domain's tables per CTA, 40,000
+// samples of eight domains (64, 64) took 60 us, longer than the 18 us of the
+// block kernel (backward.cu) that this one replaced; now 17.  (One domain
+// (64, 64): 33 us, the block kernel 21, now 19.)
 // Bound by latency with 16 warps per SM.  One thread per (window, bin) with an
 // N-term dot product from shared memory took 183 us for 16.8 M samples at N = 64,
 // E = 32; this took 89 us with a level loaded at a time (the largest stall by far),
@@ -22,6 +28,7 @@ namespace {
 
 constexpr uint32_t kBwWarps = 8;
 constexpr uint32_t kBwLevels = 8;  // of a lane's levels, loaded together
+constexpr uint32_t kBwMaxDomains = 128;  // more do not fit: a domain's unit rows are 2 KB
 
 __host__ __device__ constexpr uint32_t bw_pitch(uint32_t n) { return ((n + 3) / 4 | 1u) * 4; }  // odd number of 16-byte pieces
 __host__ __device__ constexpr uint32_t bw_pairs4(uint32_t N) { return ((N + 1) / 2 + 3) / 4 * 4; }
@@ -60,41 +67,65 @@ struct PairSum {
   }
 };
 
+// A place among the tiles: a tile and a part of it (split parts a tile).
+struct BwPlace {
+  uint64_t tile;
+  uint32_t part;
+  __device__ BwPlace(const DecodeParams &p, uint32_t split, uint64_t unit, uint64_t units) {
+    const uint64_t at = (p.tile_end - p.tile_begin) * split * unit / units;
+    tile = p.tile_begin + at / split;
+    part = (uint32_t)(at % split);
+  }
+  __device__ bool before(const BwPlace &o) const { return tile < o.tile || (tile == o.tile && part < o.part); }
+};
+
 __global__ void __launch_bounds__(kBwWarps * 32, 2) k_backward_any(const BackwardParams bp, uint32_t n_domains,
-                                                                  uint32_t warp_bytes) {
+                                                                  uint32_t warp_bytes, uint32_t split) {
   extern __shared__ __align__(16) unsigned char bw_smem[];
   const DecodeParams &p = bp.d;
   const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
-  // ---- every domain's unit rows (zeroed for a zone that is off) and basis rows of bw_pairs4(N)
-  float *const tabs = reinterpret_cast<float *>(bw_smem);
+  uint32_t tab_bytes = 0;
+  for (uint32_t d = 0; d < n_domains; ++d) tab_bytes += (512u + p.domains[d].E * bw_pairs4(p.domains[d].N)) * 4;
+  float *const tabs = reinterpret_cast<float *>(bw_smem), *const xs = tabs + (tab_bytes + wid * warp_bytes) / 4;
+  const uint64_t units = (uint64_t)gridDim.x * kBwWarps, unit = (uint64_t)blockIdx.x * kBwWarps + wid;
+  BwPlace at(p, split, unit, units);
+  const BwPlace to(p, split, unit + 1, units);
+  uint32_t s = 0;
+  if (at.before(to)) s = warp_find_segment(p.segs, p.seg_begin, p.seg_end, at.tile, lane);
+  // ---- the domains of the CTA's segments, a bit each (in the first warp's buffers)
+  uint32_t *const used = reinterpret_cast<uint32_t *>(bw_smem + tab_bytes);
+  if (n_domains > 1) {
+    if (threadIdx.x < kBwMaxDomains / 32) used[threadIdx.x] = 0u;
+    __syncthreads();
+    if (at.before(to)) {
+      const uint64_t end = to.tile + (to.part ? 1u : 0u);
+      for (uint32_t i = s + lane; i < p.seg_end && p.segs[i].tile_base < end; i += 32)
+        atomicOr(used + p.segs[i].domain / 32u, 1u << (p.segs[i].domain & 31u));
+    }
+    __syncthreads();
+  }
+  // ---- those domains' unit rows (zeroed for a zone that is off) and basis rows of bw_pairs4(N)
   {
     uint32_t off = 0;
     for (uint32_t d = 0; d < n_domains; ++d) {
       const DomainDev &dm = p.domains[d];
-      const float a0 = p.scale ? p.scale[d * 3 + 0] : dm.scale[0];
-      const float a1 = p.scale ? p.scale[d * 3 + 1] : dm.scale[1];
-      for (uint32_t i = threadIdx.x; i < 512u; i += kBwWarps * 32)
-        tabs[off + i] = (i < 256u ? a0 : a1) > 1e-30f ? dm.unit[i >> 8][i & 255u] : 0.0f;
-      off += 512u;
       const uint32_t P = (dm.N + 1) / 2, p4 = bw_pairs4(dm.N);
-      for (uint32_t i = threadIdx.x; i < dm.E * p4; i += kBwWarps * 32) {
-        const uint32_t k = i / p4, n = i - k * p4;
-        tabs[off + i] = n < P ? __ldg(p.basis + dm.basis_offset + (size_t)k * dm.N + n) : 0.0f;
+      if (n_domains == 1 || (used[d / 32u] >> (d & 31u) & 1u)) {
+        const float a0 = p.scale ? p.scale[d * 3 + 0] : dm.scale[0];
+        const float a1 = p.scale ? p.scale[d * 3 + 1] : dm.scale[1];
+        for (uint32_t i = threadIdx.x; i < 512u; i += kBwWarps * 32)
+          tabs[off + i] = (i < 256u ? a0 : a1) > 1e-30f ? dm.unit[i >> 8][i & 255u] : 0.0f;
+#pragma unroll 8
+        for (uint32_t i = threadIdx.x; i < dm.E * p4; i += kBwWarps * 32) {
+          const uint32_t k = i / p4, n = i - k * p4;
+          tabs[off + 512u + i] = n < P ? __ldg(p.basis + dm.basis_offset + (size_t)k * dm.N + n) : 0.0f;
+        }
       }
-      off += dm.E * p4;
+      off += 512u + dm.E * p4;
     }
   }
   __syncthreads();
-  uint32_t tab_bytes = 0;
-  for (uint32_t d = 0; d < n_domains; ++d) tab_bytes += (512u + p.domains[d].E * bw_pairs4(p.domains[d].N)) * 4;
-  float *const xs = reinterpret_cast<float *>(bw_smem + tab_bytes + (size_t)wid * warp_bytes);
-
-  const uint64_t units = (uint64_t)gridDim.x * kBwWarps, unit = (uint64_t)blockIdx.x * kBwWarps + wid;
-  const uint64_t n_all = p.tile_end - p.tile_begin;
-  const uint64_t t1 = p.tile_begin + n_all * (unit + 1) / units;
-  uint64_t t = p.tile_begin + n_all * unit / units;
-  if (t >= t1) return;
-  uint32_t s = warp_find_segment(p.segs, p.seg_begin, p.seg_end, t, lane);
+  if (!at.before(to)) return;
 
   PairSum sum0, sum1;
   uint32_t dom = 0xFFFFFFFFu;
@@ -112,19 +143,27 @@ __global__ void __launch_bounds__(kBwWarps * 32, 2) k_backward_any(const Backwar
     sum0 = sum1 = PairSum{};
   };
 
-  for (; t < t1; ++s) {
+  for (; at.before(to); ++s) {
     const SegDev &sg = p.segs[s];
     const uint64_t seg_end = sg.tile_base + sg.n_tiles;
-    if (t >= seg_end) continue;
+    if (at.tile >= seg_end) continue;
     const DomainDev &dm = p.domains[sg.domain];
     const uint32_t N = dm.N, E = dm.E, B1 = dm.B1, B2 = dm.B2;
     if (sg.domain != dom) {
       flush();
       dom = sg.domain;
     }
-    const uint64_t win0 = (t - sg.tile_base) * dm.tile_windows;
-    const uint64_t wend = t1 < seg_end ? (t1 - sg.tile_base) * dm.tile_windows : sg.n_windows;
-    t = t1 < seg_end ? t1 : seg_end;
+    auto window = [&](const BwPlace &x) -> uint64_t {
+      return (x.tile - sg.tile_base) * dm.tile_windows + dm.tile_windows * x.part / split;
+    };
+    const uint64_t win0 = window(at);
+    const uint64_t wend = to.tile < seg_end ? min(window(to), sg.n_windows) : sg.n_windows;
+    at = to;
+    if (to.tile >= seg_end) {  // the range goes on, or ends, behind this segment
+      at.tile = seg_end;
+      at.part = 0;
+    }
+    if (win0 >= wend) continue;  // a part past the end of the segment's last tile
     const float *unit_tab = tabs;
     for (uint32_t d = 0; d < sg.domain; ++d) unit_tab += 512u + p.domains[d].E * bw_pairs4(p.domains[d].N);
     const float *const basis = unit_tab + 512;
@@ -280,10 +319,21 @@ cudaError_t backward_any_config(size_t smem, int *ctas_per_sm) {
   return e;
 }
 
-cudaError_t launch_backward_any(const BackwardParams &p, uint32_t n_domains, uint32_t warp_bytes, uint32_t grid,
-                                size_t smem, cudaStream_t stream) {
+// Parts a tile is split in: until every warp of `ctas` has one, or a part is one
+// of the kernel's own tiles (bw_tile).
+uint32_t backward_any_split(uint64_t n_tiles, uint64_t ctas, const DomainDev *dd, uint32_t n_domains) {
+  uint32_t most = 1;
+  for (uint32_t d = 0; d < n_domains; ++d) {
+    const uint32_t t = bw_tile(dd[d].N, dd[d].E);
+    most = std::max(most, (dd[d].tile_windows + t - 1) / t);
+  }
+  return n_tiles ? (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(most, ctas * kBwWarps / n_tiles)) : 1u;
+}
+
+cudaError_t launch_backward_any(const BackwardParams &p, uint32_t n_domains, uint32_t warp_bytes, uint32_t split,
+                                uint32_t grid, size_t smem, cudaStream_t stream) {
   if (p.d.tile_end <= p.d.tile_begin || grid == 0) return cudaSuccess;
-  k_backward_any<<<grid, kBwWarps * 32, smem, stream>>>(p, n_domains, warp_bytes);
+  k_backward_any<<<grid, kBwWarps * 32, smem, stream>>>(p, n_domains, warp_bytes, split);
   return cudaGetLastError();
 }
 

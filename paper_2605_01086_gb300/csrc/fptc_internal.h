@@ -273,8 +273,9 @@ cudaError_t launch_backward_warp(const BackwardParams &p, const WarpParams &wp, 
 // adjoint from saved levels for any shape (backward_any.cu)
 size_t backward_any_smem(const uint32_t *N, const uint32_t *E, uint32_t n_domains, uint32_t *warp_bytes);
 cudaError_t backward_any_config(size_t smem, int *ctas_per_sm);
-cudaError_t launch_backward_any(const BackwardParams &p, uint32_t n_domains, uint32_t warp_bytes, uint32_t grid,
-                                size_t smem, cudaStream_t stream);
+uint32_t backward_any_split(uint64_t n_tiles, uint64_t ctas, const DomainDev *dd, uint32_t n_domains);
+cudaError_t launch_backward_any(const BackwardParams &p, uint32_t n_domains, uint32_t warp_bytes, uint32_t split,
+                                uint32_t grid, size_t smem, cudaStream_t stream);
 
 cudaError_t launch_backward(const BackwardParams &p, uint32_t threads, uint32_t grid, size_t smem,
                             cudaStream_t stream);

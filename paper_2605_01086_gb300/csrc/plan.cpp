@@ -69,7 +69,7 @@ struct fptc_plan {
   uint32_t b_threads = 256, b_grid = 0;
   size_t b_smem = 0;
   bool b_warp = false;    // backward on the warp-tile adjoint kernel
-  uint32_t b_any_grid = 0, b_any_warp_bytes = 0;  // backward from saved levels on backward_any.cu (grid 0: not)
+  uint32_t b_any_grid = 0, b_any_warp_bytes = 0, b_any_split = 1;  // backward from saved levels on backward_any.cu (grid 0: not)
   size_t b_any_smem = 0;
   WarpParams b_wp{};
   static constexpr int kAux = 4;        // copy-back streams of the end-to-end decode
@@ -468,8 +468,11 @@ fptc_status configure_launch(fptc_plan *p) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     p->b_any_smem = backward_any_smem(ns.data(), es.data(), (uint32_t)ns.size(), &p->b_any_warp_bytes);
-    if (p->b_any_smem <= (size_t)optin && backward_any_config(p->b_any_smem, &aocc) == cudaSuccess && aocc > 0)
-      p->b_any_grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)p->sm_count * aocc, p->n_tiles));
+    if (p->b_any_smem <= (size_t)optin && backward_any_config(p->b_any_smem, &aocc) == cudaSuccess && aocc > 0) {
+      const uint64_t most = (uint64_t)p->sm_count * aocc;
+      p->b_any_split = backward_any_split(p->n_tiles, most, p->dom_dev.data(), (uint32_t)ns.size());
+      p->b_any_grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(most, p->n_tiles * p->b_any_split));
+    }
   }
   p->b_threads = (threads == 128 || threads == 256 || threads == 512) ? threads : 256u;  // backward variants
   p->b_smem = backward_smem_bytes(p->b_threads, p->lut_cap, p->coef_cap, p->gx_cap, p->basis_cap);
@@ -1123,7 +1126,8 @@ fptc_status fptc_decode_backward(fptc_plan *p, const uint64_t *d_words, const ui
     wp.out_tma = encode_out_map(&map, const_cast<float *>(d_grad_out), p->out_extent) ? 1u : 0u;
     e = launch_backward_warp(bp, wp, map, p->b_threads, p->b_grid, p->b_smem, s);
   } else if (!redecode && p->b_any_grid) {
-    e = launch_backward_any(bp, (uint32_t)p->domains.size(), p->b_any_warp_bytes, p->b_any_grid, p->b_any_smem, s);
+    e = launch_backward_any(bp, (uint32_t)p->domains.size(), p->b_any_warp_bytes, p->b_any_split, p->b_any_grid,
+                            p->b_any_smem, s);
   } else {
     e = launch_backward(bp, p->b_threads, p->b_grid, p->b_smem, s);
   }

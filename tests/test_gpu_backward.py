@@ -259,3 +259,89 @@ def test_backward_from_levels_any_shape(N, E, B1, B2):
             for z in range(2):
                 want = 0.0 if (z == 0 and d == 1) else gA[d, z]
                 assert abs(g[d, z] - want) <= slack[d, z], (d, z, g[d, z], want)
+
+
+def _two_routes(doms, lens, idx, seed, gx=None):
+    """dL/dC and dL/dA from the saved levels and with the levels decoded again (the
+    block kernel, where the domains are not N = 32, E = 16), and what they were made of."""
+    from gpu_util import crafted_batch
+    rng = np.random.default_rng(seed)
+    levels = [rng.integers(0, 256, size=doms[j].windows(S) * doms[j].E).astype(np.uint8) for S, j in zip(lens, idx)]
+    b = crafted_batch(doms, levels, lens, idx)
+    plan = make_plan(b, out_align=4)
+    w, s, _, lv = gpu_decode(plan, b)
+    if gx is None:
+        gx = torch.randn(plan.info["out_extent"], generator=torch.Generator().manual_seed(seed))
+    gx = gx.to(plan.device)
+    gco = torch.full((plan.info["n_levels_total"],), float("nan"), device=plan.device)
+    gco2 = torch.full_like(gco, float("nan"))
+    gsc, _ = plan.backward(gx, levels=lv, grad_coeffs=gco)
+    gsc2, _ = plan.backward(gx, words=w, symlen=s, grad_coeffs=gco2)
+    assert plan.device_status()[0] == 0
+    return plan, gx.cpu().numpy(), gsc.cpu().numpy(), gco.cpu().numpy(), gsc2.cpu().numpy(), gco2.cpu().numpy()
+
+
+@pytest.mark.parametrize("N,E", [(4, 4), (16, 8), (24, 12), (64, 64), (81, 41), (127, 64), (128, 128)])
+@pytest.mark.parametrize("n", [1, 3, 12])
+def test_backward_batch_sizes(N, E, n):
+    """Batches of a few tiles (split into parts, most warps idle) and of more than the
+    chip holds at once, of one domain, several (a CTA loads the tables of those its
+    segments have) and more than the warp-tile kernel takes: both routes agree.
+
+    Either route's coefficient is a sum of at most N products: within (N + 5) 2^-24
+    of sum |g| of its window (|basis| <= 1), and the scale gradients within the sum
+    of that over their bins (|unit| <= 1) and (4 + 2048) 2^-24 of the sum of
+    |g_C unit| <= sum |g| E (the block kernel's partial sums are FP32 over at most
+    2048 products a thread)."""
+    cl = np.full(256, 8, np.uint8)
+    doms = [oracle.Domain(N, E, min(2, E - 1), E - (d % 2), 30.0, 0.02, (3.0, 1.5, 0.0), 8, cl) for d in range(n)]
+    for lens in ([1, N, 7 * N + 1, 16 * N, 33 * N + N // 2, 5000],
+                 [30000 + 11 * i for i in range(max(n, 40))]):
+        idx = [i % n for i in range(len(lens))] if len(lens) >= n else [(3 * i) % n for i in range(len(lens))]
+        plan, g, sa, ca, sb, cb = _two_routes(doms, lens, idx, N + n)
+        slack = np.zeros((n, 3))
+        for i, S in enumerate(lens):
+            a, o = int(plan.level_offsets[i]), int(plan.segments[i]["out_offset"])
+            W = doms[idx[i]].windows(S)
+            x = np.zeros(W * N)
+            x[:S] = np.abs(g[o:o + S].astype(np.float64))
+            x = x.reshape(W, N).sum(1)
+            bound = 2 * (N + 5) * 2.0 ** -24 * x
+            d = np.abs(ca[a:a + W * E].astype(np.float64) - cb[a:a + W * E]).reshape(W, E)
+            assert np.all(d <= bound[:, None]), (i, d.max())  # a NaN is no bound's
+            slack[idx[i]] += (bound.sum() + 2052 * 2.0 ** -24 * x.sum()) * E
+        assert np.all(np.abs(sa - sb) <= slack)
+        assert np.all(sa[np.unique(idx), 1] != 0)
+
+
+@pytest.mark.parametrize("N,E,n", [(64, 64, 8), (128, 64, 4)])
+def test_small_batches_of_many_domains_are_quick(N, E, n):
+    """From saved levels a few short streams of several domains take no longer than
+    with the levels decoded again, which is the same work and more (they took
+    twice as long while every block loaded every domain's tables)."""
+    from gpu_util import crafted_batch
+    cl = np.full(256, 8, np.uint8)
+    doms = [oracle.Domain(N, E, 2, E, 30.0, 0.02, (3.0, 1.5, 0.0), 8, cl) for _ in range(n)]
+    lens = [5000] * n
+    rng = np.random.default_rng(1)
+    levels = [rng.integers(0, 256, size=doms[i].windows(S) * E).astype(np.uint8) for i, S in enumerate(lens)]
+    b = crafted_batch(doms, levels, lens, list(range(n)))
+    plan = make_plan(b)
+    w, s, _, lv = gpu_decode(plan, b)
+    g = torch.randn(plan.info["out_extent"], device=plan.device)
+    gc = torch.empty(plan.info["n_levels_total"], device=plan.device)
+
+    def quickest(call):
+        times = []
+        for _ in range(20):
+            a, z = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            call()
+            z.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(z))
+        return min(times)
+
+    saved = quickest(lambda: plan.backward(g, levels=lv, grad_coeffs=gc))
+    again = quickest(lambda: plan.backward(g, words=w, symlen=s, grad_coeffs=gc))
+    assert saved <= 1.2 * again, (saved, again)
