@@ -3,8 +3,11 @@
 //
 // As in the encoder's level kernel for other shapes, a window of gradients is
 // folded once, u[n] = g[n] + g[N-1-n] and v[n] = g[n] - g[N-1-n] for n < P =
-// ceil(N / 2) (the middle sample of an odd N alone in u), because
+// ceil(N / 2) (the middle sample of an odd N as it is in both: its basis value is
+// 0 to rounding for odd k), because
 //   g_C[k] = sum_n g[n] B[k][n] = sum_{n < P} (k even ? u : v)[n] B[k][n].
+// Where that is not finite (an infinity or NaN among the gradients, or two whose
+// sum overflows) the plain sum over n is taken instead, as in the block kernel.
 // A lane then has four windows and four bins of one parity: 32 paired multiply-
 // adds (fma.f32x2, pairs along n, the halves added at the end) for four 16-byte
 // reads of the folded windows and four of the basis.  g_C is staged in shared
@@ -56,9 +59,10 @@ __device__ __forceinline__ void cp4z(void *dst, const void *src, uint32_t bytes)
                : "memory");
 }
 
-// An FP32 sum with its rounding errors.
+// An FP32 sum with its rounding errors (which are NaN where the sum is infinite).
 struct PairSum {
   float s = 0.0f, c = 0.0f;
+  __device__ __forceinline__ double total() const { return isfinite(s) ? (double)s + (double)c : (double)s; }
   __device__ __forceinline__ void add(float a, float b) {  // + a * b
     const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
     const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
@@ -130,7 +134,7 @@ __global__ void __launch_bounds__(kBwWarps * 32, 2) k_backward_any(const Backwar
   PairSum sum0, sum1;
   uint32_t dom = 0xFFFFFFFFu;
   auto flush = [&]() {
-    double a0 = (double)sum0.s + (double)sum0.c, a1 = (double)sum1.s + (double)sum1.c;
+    double a0 = sum0.total(), a1 = sum1.total();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       a0 += __shfl_xor_sync(0xffffffffu, a0, o);
@@ -217,7 +221,7 @@ __global__ void __launch_bounds__(kBwWarps * 32, 2) k_backward_any(const Backwar
           for (uint32_t j = 0; j < 4; ++j) {
             const bool in = c + j < P, mid = 2 * (c + j) + 1 == N;
             u[j] = in ? (mid ? a[j] : a[j] + b[j]) : 0.0f;
-            v[j] = in && !mid ? a[j] - b[j] : 0.0f;
+            v[j] = in ? (mid ? a[j] : a[j] - b[j]) : 0.0f;
           }
           *reinterpret_cast<float4 *>(us + w * up + c) = make_float4(u[0], u[1], u[2], u[3]);
           *reinterpret_cast<float4 *>(vs + w * up + c) = make_float4(v[0], v[1], v[2], v[3]);
@@ -227,6 +231,7 @@ __global__ void __launch_bounds__(kBwWarps * 32, 2) k_backward_any(const Backwar
       if (w0 + tile < wend) load(w0 + tile);
       // ---- g_C, four windows x four bins a lane and round
       const uint32_t wgs = tile / 4, items = wgs * (ge + go);
+      float off = 0.0f;  // 0 while every g_C is finite, else NaN
       for (uint32_t item = lane; item < items; item += 32) {
         const uint32_t bg = item / wgs, wg = item - bg * wgs;
         const bool odd = bg >= ge;
@@ -257,10 +262,26 @@ __global__ void __launch_bounds__(kBwWarps * 32, 2) k_backward_any(const Backwar
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (uint32_t j = 0; j < 4; ++j)
-            if (k0 + 2 * j < E) gc[(wg + i * wgs) * E + k0 + 2 * j] = acc[i][j].x + acc[i][j].y;
+          for (uint32_t j = 0; j < 4; ++j) {
+            const float r = acc[i][j].x + acc[i][j].y;
+            off += r - r;
+            if (k0 + 2 * j < E) gc[(wg + i * wgs) * E + k0 + 2 * j] = r;
+          }
       }
       __syncwarp();
+      if (__any_sync(0xffffffffu, off != 0.0f)) {
+        const float *const src = src0 + w0 * N;
+        const uint64_t left = sg.n_samples - w0 * N;
+        for (uint32_t i = lane; i < nw * E; i += 32) {
+          if (isfinite(gc[i])) continue;
+          const uint32_t w = i / E;
+          const float *const row = p.basis + dm.basis_offset + (size_t)(i - w * E) * N;
+          float acc = 0.0f;
+          for (uint32_t n = 0; n < N; ++n) acc = fmaf(w * N + n < left ? src[w * N + n] : 0.0f, row[n], acc);
+          gc[i] = acc;
+        }
+        __syncwarp();
+      }
       // ---- out, and with the levels into the scale gradients
       const uint32_t total = nw * E;
       const uint64_t at = sg.level_offset + w0 * E;

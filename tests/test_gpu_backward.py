@@ -345,3 +345,28 @@ def test_small_batches_of_many_domains_are_quick(N, E, n):
     saved = quickest(lambda: plan.backward(g, levels=lv, grad_coeffs=gc))
     again = quickest(lambda: plan.backward(g, words=w, symlen=s, grad_coeffs=gc))
     assert saved <= 1.2 * again, (saved, again)
+
+
+@pytest.mark.parametrize("N,E", [(64, 32), (24, 12), (81, 41), (5, 5), (127, 127)])
+def test_backward_infinite_and_nan_gradients(N, E):
+    """Infinities and NaN in the incoming gradient (either half of a window, both
+    mirrored samples, the middle one of an odd N): dL/dC and dL/dA are infinite, of
+    the same sign, and NaN where the block kernel's sums are."""
+    cl = np.full(256, 8, np.uint8)
+    inf, nan = float("inf"), float("nan")
+    places = [[(0, inf)], [(N - 1, -inf)], [(N // 2, inf)], [((N - 1) // 2, nan)], [(1, inf), (N - 2, inf)],
+              [(1, inf), (N - 2, -inf)], [(2, nan)], [(N // 2 + 1, -inf)], []]
+    doms = [oracle.Domain(N, E, 1, E, 30.0, 0.02, (3.0, 1.5, 0.0), 8, cl) for _ in range(len(places))]
+    lens = [40 * N] * len(places)
+    off = np.zeros(len(places) + 1, np.int64)
+    off[1:] = np.cumsum([-(-S // 4) * 4 for S in lens])
+    gx = torch.randn(int(off[-1]), generator=torch.Generator().manual_seed(N))
+    for i, at in enumerate(places):
+        for n, v in at:
+            gx[off[i] + 17 * N + n] = v
+    plan, _, sa, ca, sb, cb = _two_routes(doms, lens, list(range(len(places))), N, gx)
+    assert [int(x["out_offset"]) for x in plan.segments] == list(off[:-1])
+    assert np.isinf(sb[:, 0]).any() and np.isnan(sb).any() and np.isfinite(sb[-1]).all()
+    for a, b in ((ca, cb), (sa, sb)):
+        np.testing.assert_array_equal(np.isnan(a), np.isnan(b))
+        np.testing.assert_array_equal(np.where(np.isinf(a), a, 0.0), np.where(np.isinf(b), b, 0.0))
