@@ -461,16 +461,19 @@ fptc_status configure_launch(fptc_plan *p) {
       }
     }
   }
-  // from saved levels: the kernel of backward_any.cu where its tables and windows fit
+  // from saved levels: the kernel of backward_any.cu where its tables and windows fit; the
+  // block kernel where that fills no more than an SM each and a window's bins take a warp two
+  // turns there (E > 64: (128, 128), 128 tiles, 31 us against 36; 256 tiles, 48 against 38)
   p->b_any_grid = 0;
   {
     std::vector<uint32_t> es;
     for (const auto &d : p->domains) es.push_back(d.E);
+    const bool few = p->n_tiles <= (uint64_t)p->sm_count && *std::max_element(es.begin(), es.end()) > 64;
     int dev = 0, optin = 0, aocc = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     p->b_any_smem = backward_any_smem(ns.data(), es.data(), (uint32_t)ns.size(), &p->b_any_warp_bytes);
-    if (p->b_any_smem <= (size_t)optin && backward_any_config(p->b_any_smem, &aocc) == cudaSuccess && aocc > 0) {
+    if (!few && p->b_any_smem <= (size_t)optin && backward_any_config(p->b_any_smem, &aocc) == cudaSuccess && aocc > 0) {
       const uint64_t most = (uint64_t)p->sm_count * aocc;
       p->b_any_split = backward_any_split(p->n_tiles, most, p->dom_dev.data(), (uint32_t)ns.size());
       p->b_any_grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(most, p->n_tiles * p->b_any_split));
