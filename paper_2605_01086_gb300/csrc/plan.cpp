@@ -512,18 +512,6 @@ fptc_status upload_layout(fptc_plan *p) {
     e = cudaMemcpy(p->d_segs_form, p->segs_form.data(), bytes, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(e, "upload segments by transform");
   }
-  if (p->n_tiles > p->tiles_capacity) {
-    if (p->d_tiles) {
-      cudaFree(p->d_tiles);
-      p->device_bytes -= p->tiles_capacity * sizeof(TileRec);
-      p->d_tiles = nullptr;
-    }
-    const uint64_t cap = std::max<uint64_t>(p->n_tiles, 1);
-    e = cudaMalloc(&p->d_tiles, cap * sizeof(TileRec));
-    if (e != cudaSuccess) return cuda_fail(e, "tile table");
-    p->tiles_capacity = cap;
-    p->device_bytes += cap * sizeof(TileRec);
-  }
   return FPTC_OK;
 }
 
@@ -556,6 +544,23 @@ IndexParams index_params(const fptc_plan *p, const uint8_t *d_symlen, bool recor
 bool needs_records(const fptc_plan *p) {
   return !(p->kind == FPTC_KERNEL_WARP_TILE || p->kind == FPTC_KERNEL_TENSOR) ||
          p->opts.schedule == FPTC_SCHEDULE_THREE_KERNEL;
+}
+
+// Room for the records of a configured plan, where anything reads them: its forward
+// decode, or its adjoint with the levels decoded again (not the warp-tile one).
+fptc_status reserve_records(fptc_plan *p) {
+  if ((!needs_records(p) && p->b_warp) || p->n_tiles <= p->tiles_capacity) return FPTC_OK;
+  if (p->d_tiles) {
+    cudaFree(p->d_tiles);
+    p->device_bytes -= p->tiles_capacity * sizeof(TileRec);
+    p->d_tiles = nullptr;
+    p->tiles_capacity = 0;
+  }
+  cudaError_t e = cudaMalloc(&p->d_tiles, p->n_tiles * sizeof(TileRec));
+  if (e != cudaSuccess) return cuda_fail(e, "tile table");
+  p->tiles_capacity = p->n_tiles;
+  p->device_bytes += p->n_tiles * sizeof(TileRec);
+  return FPTC_OK;
 }
 
 DecodeParams decode_params(const fptc_plan *p, const uint64_t *d_words, const uint8_t *d_symlen, float *d_out,
@@ -971,6 +976,7 @@ fptc_status fptc_plan_create(fptc_plan **out, int device, const fptc_domain *dom
       p->device_bytes = b;
       if (st == FPTC_OK) st = upload_layout(p);
       if (st == FPTC_OK) st = configure_launch(p);
+      if (st == FPTC_OK) st = reserve_records(p);
       if (st == FPTC_OK) {
         for (auto &a : p->aux)
           if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&a, cudaStreamNonBlocking);
@@ -1316,7 +1322,7 @@ fptc_status fptc_plan_autotune(fptc_plan *p, const uint64_t *d_words, const uint
       p->opts.ctas_per_sm = 0;
       p->kind = (int)c.kernel;
       layout_tiles(p, c.tile_samples);
-      if (upload_layout(p) != FPTC_OK || configure_launch(p) != FPTC_OK) continue;
+      if (upload_layout(p) != FPTC_OK || configure_launch(p) != FPTC_OK || reserve_records(p) != FPTC_OK) continue;
       if (fptc_decode_batch(p, d_words, d_symlen, d_out, nullptr, nullptr, stream) != FPTC_OK) continue;
       std::vector<float> ms;
       for (uint32_t t = 0; t < trials; ++t) {
@@ -1343,6 +1349,7 @@ fptc_status fptc_plan_autotune(fptc_plan *p, const uint64_t *d_words, const uint
     layout_tiles(p, win.tile_samples);
     st = upload_layout(p);
     if (st == FPTC_OK) st = configure_launch(p);
+    if (st == FPTC_OK) st = reserve_records(p);
     if (st != FPTC_OK) return st;
     if (best) *best = win;
     if (best_ms) *best_ms = win_ms;

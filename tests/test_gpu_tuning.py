@@ -57,3 +57,26 @@ def test_fit_zone_scales_matches_oracle(kernel):
     xh = np.concatenate([oracle.reconstruct(lv, xi.size, doms[b.domain_idx[i]])
                          for i, (lv, xi) in enumerate(zip(lvs, xs))])
     assert abs(rep["prd_after"] - oracle.prd(x_all, xh)) <= 1e-4 * oracle.prd(x_all, xh)
+
+
+def test_tile_records_only_where_they_are_read():
+    """A plan of the warp-tile kernel and its adjoint holds no record per tile (they read
+    none); the kernels that do get theirs, also when the tuner has tried both."""
+    from gpu_util import compare_with_oracle, crafted_batch, gpu_decode
+    d = oracle.Domain(32, 16, 2, 16, 30.0, 0.02, (3.0, 1.5, 0.0), 8, np.full(256, 8, np.uint8))
+    S = 1 << 22
+    b = crafted_batch([d], [np.random.default_rng(3).integers(0, 256, size=S // 2).astype(np.uint8)], [S], [0])
+    plan = make_plan(b)
+    assert plan.info["device_bytes"] < 16 * plan.info["n_tiles"]
+    w, s, out, lv = gpu_decode(plan, b)
+    g = torch.randn(plan.info["out_extent"], device=plan.device)
+    a = [plan.backward(g, words=w, symlen=s)[0], plan.backward(g, levels=lv)[0]]
+    assert torch.allclose(a[0], a[1], rtol=1e-12, atol=0)
+    plan.autotune(w, s, out, trials=1)
+    for p in (plan, make_plan(b, kernel="block_tile"), make_plan(b, kernel="generic"),
+              make_plan(b, schedule="three_kernel")):
+        _, _, out, lv = gpu_decode(p, b)
+        compare_with_oracle(p, b, out, lv)
+        # 2^21 products of random sign: their sum is about 2^-10.5 of the sum of their magnitudes,
+        # to which some 70 roundings of 2^-24 (N terms a product, FP32 partial sums) are relative
+        assert torch.allclose(p.backward(g, words=w, symlen=s)[0], a[0], rtol=1e-2, atol=0)
