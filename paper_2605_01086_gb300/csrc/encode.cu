@@ -397,7 +397,9 @@ __device__ __forceinline__ LvWin lv_window(const EncParams &p, uint64_t gw, uint
 // samples: consecutive lanes copy consecutive 16 bytes (4 where the stream does
 // not start on a 16-byte boundary, as in a batch of ragged lengths).  Where
 // windows of several streams or a stream's end meet, each lane copies its own
-// window (zero past the stream's end; no window: zeros).
+// window, a whole one on a 16-byte boundary in 16-byte pieces (zero past the
+// stream's end; no window: zeros).  That is every group of a batch of short
+// streams: 50,000 of 600 samples take 80 us, 145 in 4-byte pieces alone.
 // Each lane its own row for every group made a ragged batch of 86 M samples
 // take 317 us (50 M of the 70 M shared-memory wavefronts bank conflicts, 32
 // lines a copy); consecutive lanes take 122 us.
@@ -419,6 +421,11 @@ __device__ __forceinline__ void lv_load_async(const EncParams &p, const LvWin &w
     return;
   }
   float *const row = rows + lane * kRowPitch;
+  if (wn.avail >= 32 && (reinterpret_cast<uintptr_t>(wn.src) & 15u) == 0) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) cp_async_16(row + 4 * j, wn.src + 4 * j);
+    return;
+  }
   const float *base = wn.avail ? wn.src : p.x;  // a valid address where nothing is read
 #pragma unroll 8
   for (int j = 0; j < 32; ++j)

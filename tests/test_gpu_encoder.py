@@ -298,3 +298,33 @@ def test_encode_shapes_match_host(N, E, B1):
             np.testing.assert_array_equal(s_g, s_h, err_msg=f"symlen of stream {i}")
             if r == 0:
                 again[o:o + S] = oracle.decode_stream(w_h, s_h, S, od)[0].astype(np.float32)
+
+
+def _host_words(dom, x, offs, lens):
+    """Words, symbol counts and levels of every stream by the host encoder."""
+    from paper_2605_01086_gb300 import codec
+    return [codec.encode_stream(dom, x[int(o):int(o) + int(S)]) for o, S in zip(offs, lens)]
+
+
+@pytest.mark.parametrize("lens_of", ["aligned", "ragged"])
+def test_encode_many_short_streams(lens_of):
+    """Groups of windows from several streams each (16-byte copies where a window
+    starts on such a boundary, 4-byte ones elsewhere, zeros past a stream's end):
+    levels, words and counts equal the host encoder's."""
+    from paper_2605_01086_gb300 import Encoder
+    rng = np.random.default_rng(17)
+    lens = rng.choice([4, 32, 36, 64, 600] if lens_of == "aligned" else [1, 31, 33, 600, 605], size=400)
+    offs = np.zeros(len(lens), np.int64)
+    offs[1:] = np.cumsum(lens[:-1])
+    d = product_domain(oracle_domains()[0])
+    x = (rng.standard_normal(int(lens.sum())) * d.scale[0] * 0.2).astype(np.float32)
+    enc = Encoder([d], lens, np.zeros(len(lens), np.int64))
+    lv = torch.empty(enc.n_levels, dtype=torch.uint8, device=enc.device)
+    words, symlen, n_words = enc.encode(torch.from_numpy(x).to(enc.device), levels=lv)
+    assert enc.status()[0] == 0
+    wh, sh, nh, lh = words.cpu().numpy().view(np.uint64), symlen.cpu().numpy(), n_words.cpu().numpy(), lv.cpu().numpy()
+    for i, (w, s, l) in enumerate(_host_words(d, x, offs, lens)):
+        np.testing.assert_array_equal(lh[int(enc.level_offsets[i]):int(enc.level_offsets[i]) + l.size], l)
+        w_g, s_g = _room_words(enc, wh, sh, nh, i)
+        np.testing.assert_array_equal(w_g, w)
+        np.testing.assert_array_equal(s_g, s)
