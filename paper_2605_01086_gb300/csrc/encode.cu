@@ -15,6 +15,8 @@
 //                 computes again in FP64 (products and sums rounded
 //                 separately, in sample order, then scaled by 2/N, as the host
 //                 encoder does), one bin per lane, and quantizes from that.
+//   k_enc_short  one lane per short stream, where there are very many: its
+//                 words, one after the other.  The other streams:
 //   k_enc_starts  one warp per packing block of kPackBlock symbols: where
 //                 words start in it (Alg. 1), as a bitmap of its symbols.
 //   k_enc_scan    one warp per stream: the words before each block; the
@@ -69,7 +71,7 @@ struct EncSeg {
   uint64_t room;
   uint64_t level_offset;
   uint64_t n_windows;
-  uint64_t block_base;  // first global packing block
+  uint64_t block_base;  // first global packing block (not of a stream k_enc_short packs)
   uint32_t domain;
   uint32_t pad;
 };
@@ -98,6 +100,10 @@ struct EncParams {
   uint64_t *first_word;  // per packing block: the stream's words that start before it
   const uint32_t *block_seg;  // per packing block: its segment
   const uint32_t *code_tab;   // per domain, 256 entries: codeword << (32 - length) | length, 0: no codeword
+  const uint32_t *short_seg;  // k_enc_short: its streams
+  uint64_t n_short;
+  const uint32_t *scan_seg;   // k_enc_scan: the others, or null: every stream
+  uint64_t n_scan;
   const EncUnit *units;       // k_enc_levels_any: the windows of each warp
   const float *dots;          // and its cosines
   const uint32_t *lv_seg;     // k_enc_levels_w32: the segment of each warp's first window
@@ -970,9 +976,10 @@ __global__ void __launch_bounds__(128) k_enc_scan(EncParams p) {
   dependents_may_start();
   dependency_wait();  // the blocks' records
   if (blockIdx.x == 0 && threadIdx.x == 0) *p.fb_count = 0;  // the level kernels' list, for the next encode
-  const uint64_t s = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const uint64_t i = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint32_t lane = threadIdx.x & 31u;
-  if (s >= p.n_segs) return;  // the whole warp
+  if (i >= p.n_scan) return;  // the whole warp
+  const uint64_t s = p.scan_seg ? p.scan_seg[i] : i;
   const EncSeg sg = p.segs[s];
   const EncDomain &d = p.doms[sg.domain];
   const uint64_t L = sg.n_windows * d.E;
@@ -1524,6 +1531,80 @@ __global__ void __launch_bounds__(kPackWarps * 32) k_enc_pack(EncParams p) {
   }
 }
 
+// k_enc_short: one lane per stream, by Alg. 1 as it stands, twice: the words
+// counted (and the code and room checks), then put together and written.  Bound
+// by a lane's chain, 63 ns a symbol for both, until some 20,000 streams fill the
+// chip.  A warp per block (and four in k_enc_pack) takes about 10 ns a block of any
+// size: 50,000 streams of 304 symbols took 463 us so (43 us when every block was
+// a lane's), and take 41 us here.
+constexpr uint32_t kShortThreads = 64;
+
+template <bool TAB>
+__global__ void __launch_bounds__(kShortThreads) k_enc_short(EncParams p) {
+  dependents_may_start();
+  extern __shared__ uint32_t short_s[];  // TAB: [n_domains][256] table entries
+  if (TAB) {
+    for (uint32_t i = threadIdx.x; i < p.n_doms * 256u; i += kShortThreads) short_s[i] = __ldg(p.code_tab + i);
+    __syncthreads();
+  }
+  dependency_wait();  // the levels
+  if (blockIdx.x == 0 && threadIdx.x == 0) *p.fb_count = 0;  // as in k_enc_scan
+  const uint64_t i = (uint64_t)blockIdx.x * kShortThreads + threadIdx.x;
+  if (i >= p.n_short) return;
+  const uint32_t s = p.short_seg[i];
+  const EncSeg &sg = p.segs[s];
+  const uint32_t L = (uint32_t)(sg.n_windows * p.doms[sg.domain].E);
+  const uint8_t *const lv = p.levels + sg.level_offset;
+  const uint32_t *const tab = TAB ? short_s + sg.domain * 256u : p.code_tab + sg.domain * 256u;
+  auto entry = [&](uint32_t level) -> uint32_t { return TAB ? tab[level] : __ldg(tab + level); };
+  // fn(level) for the stream's levels in order
+  auto each = [&](auto fn) {
+    each_vector(lv, 0, L, [&](uint32_t v, const uint4 &q) {
+      if (16 * v + 16 <= L) {
+        each16(q, [&](int, uint32_t level) { fn(level); });
+      } else {
+#pragma unroll 1
+        for (uint32_t j = 16 * v; j < L; ++j) fn((uint32_t)lv[j]);
+      }
+    });
+  };
+  uint32_t state = 0xFFFFFFFFu, words = 0, seen = 0;  // a full word: the first symbol starts one
+  each([&](uint32_t level) {
+    const uint32_t c = entry_len(entry(level)), k = c + kOff32;
+    seen |= c;
+    state = __viaddmax_u32(state, c, k);
+    words += state == k ? 1u : 0u;
+  });
+  bool bad = seen >> 6;
+  if (bad) enc_flag(p.status, FPTC_ENC_FLAG_NO_CODE, s);
+  if (!bad && words > sg.room) {
+    enc_flag(p.status, FPTC_ENC_FLAG_ROOM, s);
+    bad = true;
+  }
+  p.seg_bad[s] = bad ? 1u : 0u;
+  p.n_words[s] = bad ? 0u : words;
+  if (bad || L == 0) return;
+  uint64_t *w = p.words + sg.word_offset;
+  uint8_t *n = p.symlen + sg.word_offset;
+  uint32_t h = 0, l = 0, used = 0, count = 0;
+  auto put = [&]() {
+    *w++ = ((uint64_t)h << 32 | l) << (64u - used);
+    *n++ = (uint8_t)count;
+  };
+  each([&](uint32_t level) {
+    const uint32_t e = entry(level), c = e & 31u;
+    if (used + c > 64u) {
+      put();
+      h = l = used = count = 0u;
+    }
+    h = __funnelshift_l(l, h, e);
+    l = __funnelshift_l(e, l, e);
+    used += c;
+    ++count;
+  });
+  put();
+}
+
 struct DevGuard {
   int prev = -1;
   bool ok = true;
@@ -1558,6 +1639,9 @@ struct fptc_encoder {
   uint32_t *d_masks = nullptr;              // [n_blocks][kMaskWords]
   uint64_t *d_first_word = nullptr;         // [n_blocks]
   uint32_t *d_block_seg = nullptr;          // [n_blocks]
+  uint32_t *d_short_seg = nullptr;          // [n_short]
+  uint32_t *d_scan_seg = nullptr;           // [n_scan], null where n_short is 0
+  uint64_t n_short = 0, n_scan = 0;
   uint32_t *d_code_tab = nullptr;           // [n_domains][256]
   uint32_t *d_lv_seg = nullptr;             // [warps of k_enc_levels_w32]
   long long *d_bound_keys = nullptr;        // [n_domains][2][255]
@@ -1588,6 +1672,8 @@ void enc_free(fptc_encoder *e) {
   cudaFree(e->d_masks);
   cudaFree(e->d_first_word);
   cudaFree(e->d_block_seg);
+  cudaFree(e->d_short_seg);
+  cudaFree(e->d_scan_seg);
   cudaFree(e->d_code_tab);
   cudaFree(e->d_lv_seg);
   cudaFree(e->d_units);
@@ -1630,6 +1716,10 @@ EncParams enc_params(const fptc_encoder *e, uint64_t *d_words, uint8_t *d_symlen
   p.first_word = e->d_first_word;
   p.n_doms = e->n_doms;
   p.block_seg = e->d_block_seg;
+  p.short_seg = e->d_short_seg;
+  p.n_short = e->n_short;
+  p.scan_seg = e->d_scan_seg;
+  p.n_scan = e->n_scan;
   p.code_tab = e->d_code_tab;
   p.lv_seg = e->d_lv_seg;
   p.units = e->d_units;
@@ -1644,6 +1734,35 @@ EncParams enc_params(const fptc_encoder *e, uint64_t *d_words, uint8_t *d_symlen
   p.n_segs = e->n_segs;
   p.n_levels = e->n_levels;
   return p;
+}
+
+// The streams that k_enc_short packs: those of at most X symbols, X such that it
+// gains most over a warp for each of their blocks, if it gains anything.  In
+// nanoseconds, measured: 10 a block and 0.001 a symbol there; here the longest
+// stream's 63 a symbol or, of very many, 0.003 for each (16,384 streams of 2048
+// symbols: 180 us there, 132 here; 4000 of them 57 and 131; 1000 of 304 symbols 23
+// and 23, 4000 of them 52 and 23).
+std::vector<uint32_t> choose_short(const std::vector<EncSeg> &segs, const std::vector<EncDomain> &doms) {
+  std::vector<std::pair<uint32_t, uint32_t>> single;  // (symbols, segment)
+  for (size_t i = 0; i < segs.size(); ++i) {
+    const uint64_t L = segs[i].n_windows * doms[segs[i].domain].E;
+    if (L <= kPackBlock) single.push_back({(uint32_t)L, (uint32_t)i});
+  }
+  std::sort(single.begin(), single.end());
+  double best = 0.0, symbols = 0.0;
+  size_t take = 0;
+  for (size_t i = 0; i < single.size(); ++i) {
+    symbols += single[i].first;
+    if (i + 1 < single.size() && single[i + 1].first == single[i].first) continue;
+    const double gain = 10.0 * (double)(i + 1) + 0.001 * symbols - std::max(6000.0 + 63.0 * single[i].first, 0.003 * symbols);
+    if (gain > best) {
+      best = gain;
+      take = i + 1;
+    }
+  }
+  std::vector<uint32_t> r(take);  // neighbours in a warp are as long as one another
+  for (size_t i = 0; i < take; ++i) r[i] = single[i].second;
+  return r;
 }
 
 bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
@@ -1747,7 +1866,7 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
     std::vector<EncSeg> segs(n_segments);
     std::vector<uint64_t> level_off(n_segments);
     std::vector<std::pair<uint64_t, uint64_t>> rooms;
-    std::vector<uint32_t> block_seg;
+    std::vector<uint32_t> block_seg, scan_seg;
     uint64_t win = 0, lv = 0, blocks = 0;
     for (uint64_t i = 0; i < n_segments; ++i) {
       const fptc_segment &s = segments[i];
@@ -1763,16 +1882,25 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
       e.room = s.n_words;
       e.level_offset = lv;
       e.n_windows = (s.n_samples + dm.N - 1) / dm.N;
-      e.block_base = blocks;
       e.domain = s.domain;
       e.pad = 0;
       level_off[i] = lv;
       win += e.n_windows;
       lv += e.n_windows * dm.E;
-      const uint64_t nb = (e.n_windows * dm.E + kPackBlock - 1) / kPackBlock;
-      blocks += nb;
-      block_seg.insert(block_seg.end(), nb, (uint32_t)i);
       if (s.n_words) rooms.push_back({s.word_offset, s.word_offset + s.n_words});
+    }
+    const std::vector<uint32_t> short_seg = choose_short(segs, doms);
+    {
+      std::vector<bool> is_short(n_segments);
+      for (uint32_t i : short_seg) is_short[i] = true;
+      for (uint64_t i = 0; i < n_segments; ++i) {
+        segs[i].block_base = blocks;
+        if (is_short[i]) continue;
+        const uint64_t nb = (segs[i].n_windows * doms[segs[i].domain].E + kPackBlock - 1) / kPackBlock;
+        blocks += nb;
+        block_seg.insert(block_seg.end(), nb, (uint32_t)i);
+        if (!short_seg.empty()) scan_seg.push_back((uint32_t)i);
+      }
     }
     std::sort(rooms.begin(), rooms.end());
     for (size_t i = 1; i < rooms.size(); ++i)
@@ -1797,6 +1925,8 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
     e->n_doms = n_domains;
     e->n_levels = lv;
     e->n_blocks = blocks;
+    e->n_short = short_seg.size();
+    e->n_scan = n_segments - short_seg.size();
     e->level_off = level_off;
     cudaError_t err = cudaDeviceGetAttribute(&e->sm_count, cudaDevAttrMultiProcessorCount, device);
     if (err == cudaSuccess) err = enc_upload(&e->d_segs, segs.data(), segs.size());
@@ -1814,6 +1944,10 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
     if (err == cudaSuccess) err = cudaMalloc(&e->d_masks, std::max<uint64_t>(blocks, 1) * kMaskWords * 4);
     if (err == cudaSuccess) err = cudaMalloc(&e->d_first_word, std::max<uint64_t>(blocks, 1) * 8);
     if (err == cudaSuccess) err = enc_upload(&e->d_block_seg, block_seg.data(), block_seg.size());
+    if (err == cudaSuccess && e->n_short) {
+      err = enc_upload(&e->d_short_seg, short_seg.data(), short_seg.size());
+      if (err == cudaSuccess) err = enc_upload(&e->d_scan_seg, scan_seg.data(), scan_seg.size());
+    }
     if (err == cudaSuccess) err = enc_upload(&e->d_code_tab, code_tab.data(), code_tab.size());
     for (size_t i = 0; i < bounds.size(); ++i) {  // order keys (see order_key); a NaN bound: no level reached
       long long b;
@@ -1959,11 +2093,19 @@ static fptc_status enc_run(fptc_encoder *enc, const float *d_x, bool levels_give
     launch(reinterpret_cast<const void *>(&k_enc_fallback), (uint64_t)enc->sm_count * 8u, 256, 0, true);
   }
   const bool tab = enc->n_doms <= kTabDomains;
-  if (enc->n_blocks)
+  bool chained = levels;  // a kernel of this call is in front
+  if (enc->n_short) {
+    launch(tab ? reinterpret_cast<const void *>(&k_enc_short<true>) : reinterpret_cast<const void *>(&k_enc_short<false>),
+           (enc->n_short + kShortThreads - 1) / kShortThreads, kShortThreads, tab ? enc->n_doms * 1024u : 0u, chained);
+    chained = true;
+  }
+  if (enc->n_blocks) {
     launch(tab ? reinterpret_cast<const void *>(&k_enc_starts<true>) : reinterpret_cast<const void *>(&k_enc_starts<false>),
            (enc->n_blocks + kStartWarps - 1) / kStartWarps, (kStartWarps + 1) * 32,
-           (kStartWarps + 1) * kStartWarpBytes + (tab ? enc->n_doms * 1024u : 0u), levels);
-  launch(reinterpret_cast<const void *>(&k_enc_scan), (enc->n_segs * 32 + 127) / 128, 128, 0, enc->n_blocks > 0);
+           (kStartWarps + 1) * kStartWarpBytes + (tab ? enc->n_doms * 1024u : 0u), chained);
+    chained = true;
+  }
+  if (enc->n_scan) launch(reinterpret_cast<const void *>(&k_enc_scan), (enc->n_scan * 32 + 127) / 128, 128, 0, chained);
   if (enc->n_blocks)
     launch(tab ? reinterpret_cast<const void *>(&k_enc_pack<true>) : reinterpret_cast<const void *>(&k_enc_pack<false>),
            (enc->n_blocks * (kPackBlock / kPackPart) + kPackWarps - 1) / kPackWarps, kPackWarps * 32,

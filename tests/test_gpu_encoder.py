@@ -328,3 +328,70 @@ def test_encode_many_short_streams(lens_of):
         w_g, s_g = _room_words(enc, wh, sh, nh, i)
         np.testing.assert_array_equal(w_g, w)
         np.testing.assert_array_equal(s_g, s)
+
+
+@pytest.mark.parametrize("n_doms", [1, 20])
+def test_pack_very_many_short_streams(n_doms):
+    """6,000 streams of 0 to 75 symbols (a lane each) among longer ones (warps for their
+    blocks), at every alignment, with few and with more domains than the tables in
+    shared memory hold; one whose room is too small and one with a level that has no
+    codeword are flagged and get no words; all others equal Alg. 1's."""
+    from paper_2605_01086_gb300 import Encoder, _lib
+    rng = np.random.default_rng(31 + n_doms)
+    doms = []
+    for k in range(n_doms):
+        cl = np.full(256, 13, np.uint8)
+        cl[100:130], cl[130], cl[131], cl[7] = 6, 2 + k % 3, 3, 0
+        doms.append(oracle.Domain(16, 5, 2, 5, 50.0, 0.004, (1.0, 1.0, 0.0), 13, cl))
+    W = np.concatenate([rng.integers(0, 16, size=6000), [400, 1700, 3, 5000]])
+    W = rng.permutation(W)
+    idx = rng.integers(0, n_doms, size=len(W))
+    pool = np.r_[np.arange(8, 256), np.full(300, 130), np.full(100, 131)]
+    levels = [rng.choice(pool, size=int(w) * 5).astype(np.uint8) for w in W]
+    tight, bad = np.flatnonzero(W == 9)[[3, 7]]
+    levels[bad][17] = 7
+    room = [max(1, int(w) * 5) for w in W]
+    room[tight] = 1
+    enc = Encoder([product_domain(d) for d in doms], W * 16, idx, room=room)
+    lv = torch.from_numpy(np.concatenate(levels)).to(enc.device)
+    words, symlen, n_words = enc.buffers()
+    words.fill_(-1)
+    enc.pack(lv, words, symlen, n_words)
+    st, flags, first = enc.status()
+    assert st == _lib.CORRUPT_STREAM and flags == _lib.ENC_FLAG_ROOM | _lib.ENC_FLAG_NO_CODE and first == min(tight, bad)
+    wh, sh, nh = words.cpu().numpy().view(np.uint64), symlen.cpu().numpy(), n_words.cpu().numpy()
+    used = np.zeros(wh.size, bool)
+    for i, L in enumerate(levels):
+        if i in (tight, bad):
+            assert nh[i] == 0
+            continue
+        d = doms[idx[i]]
+        w_o, s_o = oracle.pack_symlen(L, oracle.canonical_codes(d.code_len, d.lmax), d.code_len) if L.size else \
+            (np.zeros(0, np.uint64), np.zeros(0, np.uint8))
+        w_g, s_g = _room_words(enc, wh, sh, nh, i)
+        np.testing.assert_array_equal(w_g, w_o)
+        np.testing.assert_array_equal(s_g, s_o)
+        used[int(enc.room_offsets[i]):int(enc.room_offsets[i]) + len(w_o)] = True
+    assert np.all(wh[~used] == np.uint64(2 ** 64 - 1))  # nothing else is written
+
+
+def test_short_streams_cost_what_long_ones_do():
+    """Encoding 50,000 streams of 600 samples takes at most three times as long as the same
+    samples in streams of 65,536 (one warp for each stream's few symbols took five times)."""
+    from paper_2605_01086_gb300 import Encoder
+    d = product_domain(oracle_domains()[0])
+    x = torch.randn(30_000_000, device="cuda") * d.scale[0] * 0.2
+    best = []
+    for n, S in ((50000, 600), (457, 65536)):
+        enc = Encoder([d], [S] * n, [0] * n)
+        bufs = enc.buffers()
+        times = []
+        for _ in range(8):
+            a, z = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            enc.encode(x, *bufs)
+            z.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(z))
+        best.append(min(times))
+    assert best[0] <= 3.0 * best[1], best
