@@ -8,7 +8,9 @@
 //   k_enc_levels_any  (other shapes) a warp per tile of windows, folded once
 //                 by the mirror symmetry of the basis: four windows by four
 //                 bins per lane in FP32 with a bound on the sums' error.
-//                 In both, every zone map is monotone in the coefficient, so
+//   k_enc_levels_bins  (other shapes, streams of a window or a few bins, where
+//                 there are many or no others) one thread per bin.
+//                 In all, every zone map is monotone in the coefficient, so
 //                 when the levels at c - err and c + err agree the FP64
 //                 coefficient (which lies between) has that level too;
 //                 otherwise the bin goes to a list that k_enc_fallback
@@ -84,6 +86,7 @@ struct EncStatus {
 
 struct PackRec;
 struct EncUnit;
+struct EncBins;
 
 struct EncParams {
   const float *x;
@@ -106,6 +109,9 @@ struct EncParams {
   uint64_t n_scan;
   const EncUnit *units;       // k_enc_levels_any: the windows of each warp
   const float *dots;          // and its cosines
+  const EncBins *bins;        // k_enc_levels_bins: its streams
+  const uint32_t *bin_first;  // and of every 32 of their bins the first one's entry
+  uint32_t n_bin_segs, n_bins;
   const uint32_t *lv_seg;     // k_enc_levels_w32: the segment of each warp's first window
   const long long *bound_keys;  // per domain: zone 0's, then zone 1's 255 level boundaries (order keys)
   uint32_t n_doms;
@@ -1034,7 +1040,9 @@ __global__ void __launch_bounds__(128) k_enc_scan(EncParams p) {
 // products by FMA, exact sums by two-sum: error O((N u)^2 sum |x|) + u |c|; the
 // bound 2^-34 (2/N) sum |x| also covers the cosines' representation and the
 // FP64 evaluation's own rounding for N <= 128); false when that bound cannot
-// settle it.
+// settle it.  AHEAD: sixteen samples and cosines are requested at once, for
+// kernels with few bins in flight (and registers for it).
+template <bool AHEAD = true>
 __device__ __forceinline__ bool level_compensated(const EncParams &p, uint64_t g, uint64_t s, uint32_t &L) {
   const EncSeg sg = p.segs[s];
   const EncDomain d = p.doms[sg.domain];
@@ -1055,7 +1063,9 @@ __device__ __forceinline__ bool level_compensated(const EncParams &p, uint64_t g
     hi = t;
     s1 += fabsf(xv);
   };
-  if (d.N == 32 && nn == 32 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
+  if (!AHEAD) {
+    for (uint32_t n = 0; n < nn; ++n) step(__ldg(src + n), __ldg(ct + (size_t)n * d.E));
+  } else if (d.N == 32 && nn == 32 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
     // a whole window: its samples and cosines requested at once, the same
     // operations in the same order as below
     float xv[32];
@@ -1193,8 +1203,8 @@ __global__ void __launch_bounds__(kAnyWarps * 32, 4) k_enc_levels_any(EncParams 
     cp_async_wait_group<0>();
     __syncwarp();
     // ---- fold: lane (or lanes' turn t) = window and every other piece of four pairs
-    for (uint32_t t = lane; t < 2 * tile; t += 32) {
-      const uint32_t w = t % tile, h = t / tile;
+    for (uint32_t t = lane; t < 2 * nw; t += 32) {
+      const uint32_t h = t < nw ? 0u : 1u, w = t - h * nw;
       const float *x = xs + w * xp;
       float su = 0.0f, sv = 0.0f;
       for (uint32_t c = 4 * h; c < P4; c += 8) {
@@ -1228,9 +1238,10 @@ __global__ void __launch_bounds__(kAnyWarps * 32, 4) k_enc_levels_any(EncParams 
     }
     __syncwarp();
     if (w0 + tile < un.n) load(w0 + tile);
-    // ---- bins, four windows x four bins a lane and round
+    // ---- bins, four windows x four bins a lane and round (a tile that is not full
+    // takes fewer rounds; what its last lanes' windows past nw hold is not used)
     const uint64_t win = un.win + w0;
-    const uint32_t wgs = tile / 4, items = wgs * (ge + go);
+    const uint32_t wgs = (nw + 3) / 4, items = wgs * (ge + go);
     for (uint32_t i0 = 0; i0 < items; i0 += 32) {
       const uint32_t item = i0 + lane;
       uint32_t undecided = 0, wg = 0, k0 = 0;
@@ -1399,6 +1410,38 @@ __global__ void __launch_bounds__(kAnyWarps * 32, 4) k_enc_levels_any(EncParams 
     }
     __syncwarp();
   }
+}
+
+// A stream whose bins take a thread each, and how many such bins come before it.
+struct EncBins {
+  uint32_t seg;
+  uint32_t base;
+};
+// Streams of one window or of at most a warp's bins: a warp of k_enc_levels_any
+// takes 2 ns (N = 4) to 11 ns (N = E = 128) for one however few windows it has, as
+// compensated sums a thread each they take 0.2 to 5.  200,000 streams of four samples
+// at N = 4: 427 us there, 37 here; of twenty at (24, 12) 480 and 102; of forty at
+// (128, 128) 2190 and 1013; of 100 at (64, 32), two windows, 660 there.
+__host__ __device__ constexpr bool few_bins(uint64_t n_windows, uint32_t E) { return n_windows == 1 || n_windows * E <= 32; }
+
+__global__ void __launch_bounds__(256) k_enc_levels_bins(EncParams p) {
+  dependents_may_start();
+  dependency_wait();  // k_enc_fallback, behind this kernel, waits for this one only
+  const uint32_t b = blockIdx.x * 256u + threadIdx.x;
+  if (b >= p.n_bins) return;
+  uint32_t i = p.bin_first[b >> 5];
+  while (i + 1 < p.n_bin_segs && p.bins[i + 1].base <= b) ++i;
+  const uint64_t s = p.bins[i].seg, g = p.segs[s].level_offset + (b - p.bins[i].base);
+  uint32_t L;
+  if (!level_compensated<false>(p, g, s, L)) {
+    const unsigned int slot = fb_slot(p);
+    if (slot != ~0u) {
+      p.fb_list[slot] = fb_entry(g, s);
+      return;  // k_enc_fallback writes the level
+    }
+    L = level_fp64_seg(p, g, s);
+  }
+  p.levels[g] = (uint8_t)L;
 }
 
 // The listed bins, one per thread: from their compensated FP32 coefficient
@@ -1647,7 +1690,10 @@ struct fptc_encoder {
   long long *d_bound_keys = nullptr;        // [n_domains][2][255]
   EncUnit *d_units = nullptr;               // [n_units] (k_enc_levels_any)
   float *d_dots = nullptr;                  // its cosines
+  EncBins *d_bins = nullptr;                // [n_bin_segs] (k_enc_levels_bins)
+  uint32_t *d_bin_first = nullptr;          // [(n_bins + 31) / 32]
   uint64_t n_units = 0;
+  uint32_t n_bin_segs = 0, n_bins = 0;
   uint32_t any_warp_bytes = 0;              // its shared memory per warp
   bool w32 = false;               // every domain N = 32, E = 16: the window-per-thread level kernel
   uint32_t *d_seg_bad = nullptr;
@@ -1678,6 +1724,8 @@ void enc_free(fptc_encoder *e) {
   cudaFree(e->d_lv_seg);
   cudaFree(e->d_units);
   cudaFree(e->d_dots);
+  cudaFree(e->d_bins);
+  cudaFree(e->d_bin_first);
   cudaFree(e->d_bound_keys);
   cudaFree(e->d_seg_bad);
   cudaFree(e->d_fb_list);
@@ -1724,6 +1772,10 @@ EncParams enc_params(const fptc_encoder *e, uint64_t *d_words, uint8_t *d_symlen
   p.lv_seg = e->d_lv_seg;
   p.units = e->d_units;
   p.dots = e->d_dots;
+  p.bins = e->d_bins;
+  p.bin_first = e->d_bin_first;
+  p.n_bin_segs = e->n_bin_segs;
+  p.n_bins = e->n_bins;
   p.bound_keys = e->d_bound_keys;
   p.seg_bad = e->d_seg_bad;
   p.fb_list = e->d_fb_list;
@@ -1978,20 +2030,41 @@ fptc_status fptc_encoder_create(fptc_encoder **enc, int device, const fptc_domai
           for (uint32_t n = 0; n < p4; ++n)
             dots.push_back(n < pairs ? (float)cosv[doms[d].cos_off + (size_t)k * N + n] : 0.0f);
       }
+      // streams of few bins: a kernel more, so where it saves the time of one or is the only one
+      uint64_t some = 0, tiny = 0;
+      for (const EncSeg &sg : segs) {
+        some += sg.n_windows ? 1u : 0u;
+        tiny += sg.n_windows && few_bins(sg.n_windows, doms[sg.domain].E) ? 1u : 0u;
+      }
+      const bool by_bins = tiny && (tiny == some || tiny >= 2048);
+      auto binned = [&](const EncSeg &sg) { return by_bins && few_bins(sg.n_windows, doms[sg.domain].E); };
+      std::vector<EncBins> bins;
+      std::vector<uint32_t> bin_first;
+      for (uint64_t i = 0; i < n_segments; ++i) {
+        if (!segs[i].n_windows || !binned(segs[i])) continue;
+        bins.push_back(EncBins{(uint32_t)i, e->n_bins});
+        e->n_bins += (uint32_t)segs[i].n_windows * doms[segs[i].domain].E;  // 2^24 streams of 128 at most
+        while (bin_first.size() * 32u < e->n_bins) bin_first.push_back((uint32_t)bins.size() - 1);
+      }
+      e->n_bin_segs = (uint32_t)bins.size();
+      if (e->n_bins) err = enc_upload(&e->d_bins, bins.data(), bins.size());
+      if (err == cudaSuccess && e->n_bins) err = enc_upload(&e->d_bin_first, bin_first.data(), bin_first.size());
       uint64_t tiles = 0;
       for (const EncSeg &sg : segs) {
+        if (binned(sg)) continue;
         const uint32_t t = any_tile(doms[sg.domain].N, doms[sg.domain].E);
         tiles += (sg.n_windows + t - 1) / t;
       }
       const uint64_t per = std::min<uint64_t>(8, std::max<uint64_t>(1, tiles / ((uint64_t)e->sm_count * 32u)));
       std::vector<EncUnit> units;
       for (uint64_t i = 0; i < n_segments; ++i) {
+        if (binned(segs[i])) continue;
         const uint64_t step = per * any_tile(doms[segs[i].domain].N, doms[segs[i].domain].E);
         for (uint64_t w = 0; w < segs[i].n_windows; w += step)
           units.push_back(EncUnit{w, (uint32_t)i, (uint32_t)std::min<uint64_t>(step, segs[i].n_windows - w)});
       }
       e->n_units = units.size();
-      err = enc_upload(&e->d_units, units.data(), units.size());
+      if (err == cudaSuccess) err = enc_upload(&e->d_units, units.data(), units.size());
       if (err == cudaSuccess) err = enc_upload(&e->d_dots, dots.data(), dots.size());
       if (err == cudaSuccess)
         err = set_dynamic_smem_limit(reinterpret_cast<const void *>(&k_enc_levels_any), kAnyWarps * e->any_warp_bytes);
@@ -2085,11 +2158,13 @@ static fptc_status enc_run(fptc_encoder *enc, const float *d_x, bool levels_give
       const uint32_t groups = (uint32_t)std::min<uint64_t>(kLvGroups, (all + warps - 1) / warps);
       const uint64_t per = (uint64_t)kLvThreads * groups;
       k_enc_levels_w32<<<(unsigned)((enc->n_windows + per - 1) / per), kLvThreads, 0, s>>>(p, enc->n_windows, groups);
-    } else {
+    } else if (enc->n_units) {
       k_enc_levels_any<<<(unsigned)((enc->n_units + kAnyWarps - 1) / kAnyWarps), kAnyWarps * 32,
                          kAnyWarps * enc->any_warp_bytes, s>>>(p, enc->n_units, enc->any_warp_bytes);
     }
     e = cudaGetLastError();
+    if (enc->n_bins)
+      launch(reinterpret_cast<const void *>(&k_enc_levels_bins), (enc->n_bins + 255) / 256, 256, 0, enc->n_units > 0);
     launch(reinterpret_cast<const void *>(&k_enc_fallback), (uint64_t)enc->sm_count * 8u, 256, 0, true);
   }
   const bool tab = enc->n_doms <= kTabDomains;

@@ -395,3 +395,56 @@ def test_short_streams_cost_what_long_ones_do():
             times.append(a.elapsed_time(z))
         best.append(min(times))
     assert best[0] <= 3.0 * best[1], best
+
+
+@pytest.mark.parametrize("N,E", [(4, 4), (5, 3), (24, 12), (64, 32), (100, 50), (128, 128)])
+@pytest.mark.parametrize("n", [1, 7, 3000])
+def test_encode_tiny_streams_match_host(N, E, n):
+    """Streams of one window or a few bins, alone and (3,000 of them) among longer ones
+    and empty ones, tiles of every number of windows, values that are not finite or
+    near the largest float: levels and words equal the host encoder's."""
+    from paper_2605_01086_gb300 import Encoder
+    rng = np.random.default_rng(N * 7 + n)
+    lens = rng.integers(1, N + 1, size=n)
+    if n == 3000:
+        lens = rng.permutation(np.r_[lens, np.arange(1, 20) * N, 2 * N + 1, 40 * N + 3, 0, 0])
+    offs = np.zeros(len(lens), np.int64)
+    offs[1:] = np.cumsum(lens[:-1])
+    d = oracle.Domain(N, E, min(2, E), max(min(2, E), E - 1), 50.0, 0.004, (3.0, 1.0, 0.0), 8, np.full(256, 8, np.uint8))
+    pd = product_domain(d)
+    x = rng.standard_normal(max(1, int(lens.sum()))).astype(np.float32)
+    if n == 3000:
+        x[rng.integers(0, x.size, size=40)] = np.repeat(np.float32([np.inf, -np.inf, np.nan, 3e38]), 10)
+    enc = Encoder([pd], lens, np.zeros(len(lens), np.int64))
+    lv = torch.full((max(1, enc.n_levels),), 77, dtype=torch.uint8, device=enc.device)
+    words, symlen, n_words = enc.encode(torch.from_numpy(x).to(enc.device), levels=lv)
+    assert enc.status()[0] == 0
+    wh, sh, nh, lh = words.cpu().numpy().view(np.uint64), symlen.cpu().numpy(), n_words.cpu().numpy(), lv.cpu().numpy()
+    for i, (w, s, l) in enumerate(_host_words(pd, x, offs, lens)):
+        np.testing.assert_array_equal(lh[int(enc.level_offsets[i]):int(enc.level_offsets[i]) + l.size], l, err_msg=str(i))
+        w_g, s_g = _room_words(enc, wh, sh, nh, i)
+        np.testing.assert_array_equal(w_g, w)
+        np.testing.assert_array_equal(s_g, s)
+
+
+def test_single_window_streams_cost_what_more_do():
+    """Encoding 200,000 streams of one window of N = 4 takes no longer than 100,000 of ten
+    each, five times the samples (with a warp per stream it took twice as long)."""
+    from paper_2605_01086_gb300 import Encoder
+    pd = product_domain(oracle.Domain(4, 4, 2, 4, 50.0, 0.004, (3.0, 1.0, 0.0), 8, np.full(256, 8, np.uint8)))
+    x = torch.randn(1_200_000, device="cuda")
+    best = []
+    for n, S in ((200000, 4), (100000, 40)):
+        enc = Encoder([pd], [S] * n, [0] * n)
+        bufs = enc.buffers()
+        xs = x if n * S <= x.numel() else x.repeat(4)[:n * S].contiguous()
+        times = []
+        for _ in range(8):
+            a, z = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            enc.encode(xs, *bufs)
+            z.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(z))
+        best.append(min(times))
+    assert best[0] <= best[1], best
