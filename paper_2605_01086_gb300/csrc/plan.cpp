@@ -463,12 +463,16 @@ fptc_status configure_launch(fptc_plan *p) {
   }
   // from saved levels: the kernel of backward_any.cu where its tables and windows fit; the
   // block kernel where that fills no more than an SM each and a window's bins take a warp two
-  // turns there (E > 64: (128, 128), 128 tiles, 31 us against 36; 256 tiles, 48 against 38)
+  // turns there (E > 64: (128, 128), 128 tiles, 31 us against 36; 256 tiles, 48 against 38),
+  // and for a few windows in all (ten streams of three at (100, 50): 16 us against 20)
   p->b_any_grid = 0;
   {
     std::vector<uint32_t> es;
     for (const auto &d : p->domains) es.push_back(d.E);
-    const bool few = p->n_tiles <= (uint64_t)p->sm_count && *std::max_element(es.begin(), es.end()) > 64;
+    uint64_t windows = 0;
+    for (const SegDev &sg : p->segs) windows += sg.n_windows;
+    const bool few = windows <= 32 ||
+                     (p->n_tiles <= (uint64_t)p->sm_count && *std::max_element(es.begin(), es.end()) > 64);
     int dev = 0, optin = 0, aocc = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
