@@ -645,8 +645,9 @@ struct GeoS {
 // 16 warps leave 128 registers a thread; with several compiled forms in one
 // kernel some of the stream's state was spilled around the larger ones, and
 // spills go to L2 (shared memory leaves L1 little): (64, 32), 67 M samples, took
-// 130 us in that kernel and 88 us in its own.  Plans of several forms
-// run 12 warps, where nothing is spilled.
+// 130 us in that kernel and 88 us in its own.  Plans of several forms run 12
+// warps, where 44 bytes a thread are (432 at 16 warps), and the instance of (128, 64)
+// alone 24; the 24-warp one (threads = 768) 132.
 template <int WARPS, int TILES, int FORMS, uint32_t ONE = 0>
 __global__ void __launch_bounds__(WARPS * 32, 1) k_decode_shape(const DecodeParams p, const WarpParams wp,
                                                                 const __grid_constant__ ShapeMaps maps) {

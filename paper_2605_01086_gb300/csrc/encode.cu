@@ -233,20 +233,6 @@ __device__ __forceinline__ bool zone1_decide32(float c, float m, const EncDomain
   return true;
 }
 
-// Index i of the last entry with base(i) <= g over n ascending entries.
-template <class F>
-__device__ __forceinline__ uint64_t last_leq(uint64_t n, uint64_t g, F base) {
-  uint64_t lo = 0, hi = n;
-  while (hi - lo > 1) {
-    const uint64_t mid = lo + (hi - lo) / 2;
-    if (base(mid) <= g)
-      lo = mid;
-    else
-      hi = mid;
-  }
-  return lo;
-}
-
 // Level of bin g (global level index) of segment s from the FP64 coefficient,
 // computed as the host encoder does: products and sums rounded separately, in
 // sample order, then scaled by 2/N.
@@ -1120,7 +1106,9 @@ __device__ __forceinline__ bool level_compensated(const EncParams &p, uint64_t g
 // by that bound as in the window kernel; a bin it does not settle (about one
 // in 200) goes to the list of k_enc_fallback, or, where a tile has many, is
 // settled here by the compensated sum.
-// Bound by instruction issue (about 30 instructions a sample at N = 64, E = 32).
+// Bound by instruction issue (about 30 instructions a sample at N = 64, E = 32); at
+// 128 registers 64 bytes a thread are spilled, around the branch for samples that
+// are not finite and zones that the fast map does not take.
 // 16.8 M samples at N = 64, E = 32: 70 us (one thread per bin with the compensated
 // sum for every bin took 457 us; the zone maps behind a branch per bin, and plain
 // multiply-adds, 75).

@@ -235,8 +235,10 @@ void layout_tiles(fptc_plan *p, uint32_t tile_samples) {
   p->gx_cap = 0;
   const bool shape = p->kind == FPTC_KERNEL_WARP_TILE && p->shape;
   // the shape kernel splits its work by tiles, so a domain's tile is as many of its
-  // steps as cost about what the dearest step of the plan does (instructions: 14 a
-  // symbol, 10 a sample)
+  // steps as cost about what the dearest step of the plan does: 25 a symbol, and 10 a
+  // sample, 20 at N = 128, whose transform keeps the fewest warps.  With these the warps
+  // of a batch of four shapes end within 1.2 of one another (1.5 with the instructions
+  // counted, 14 and 10)
   auto step_of = [&](const DomainDev &dd) {
     return shape_step_windows(dd.N, dd.E, std::min(dd.E, dd.B2), p->shape_tiles);
   };
