@@ -31,7 +31,7 @@
 //    read is four of them, whatever it shares).  One lane per
 //    16 pairs of one window, with a basis read for every four multiply-adds and
 //    the coefficients dequantized again by each lane of a window, took 228 us for
-//    33 M samples at N = 100, E = 50; this form takes 114 us (133 us with each
+//    33 M samples at N = 100, E = 50; this form takes 111 us (133 us with each
 //    coefficient stored twice and a lane's windows side by side, when rows of 24,
 //    48 or 64 samples met in the same banks: N = 24, E = 12 took 117 us, now 83).
 #pragma once
@@ -516,7 +516,9 @@ __device__ __forceinline__ void shape_pairs(const DecodeParams &p, const UnitSeg
   const uint32_t lane = o.lane, N = dd.N, P = shape_pair_count(N), p8 = shape_pairs8(N), kz = dd.kz;
   // lanes' windows lie G apart (rows that are multiples of 32 samples apart would
   // share their banks): place MW g + i of a bin's coefficients is window g + G i
-  const uint32_t Ws = shape_pair_places(dd.step, MW), G = Ws / MW;
+  // (places for the step's own windows: a stream's last step, or only one, has fewer;
+  // with a whole step's 200,000 streams of one window of (128, 128) took 1880 us, 1375 so)
+  const uint32_t Ws = shape_pair_places(n, MW), G = Ws / MW;
   const float *deq = reinterpret_cast<const float *>(smem + dd.deq_off);
   const float *bas = reinterpret_cast<const float *>(smem + dd.basis_off);
   if (lane == 0) tma_wait_read_but<0>();  // earlier steps have left the tiles
@@ -586,7 +588,7 @@ __device__ __forceinline__ void shape_pairs(const DecodeParams &p, const UnitSeg
     const bool whole = N % 4 == 0 && 8 * pg + 8 <= P;
 #pragma unroll
     for (int i = 0; i < MW; ++i) {
-      if (wg + G * i >= dd.step) break;
+      if (wg + G * i >= n) break;
       float *const x = reinterpret_cast<float *>(o.otile) + (wg + G * i) * N;
       float f[8], m[8];
 #pragma unroll
@@ -646,8 +648,8 @@ struct GeoS {
 // kernel some of the stream's state was spilled around the larger ones, and
 // spills go to L2 (shared memory leaves L1 little): (64, 32), 67 M samples, took
 // 130 us in that kernel and 88 us in its own.  Plans of several forms run 12
-// warps, where 44 bytes a thread are (432 at 16 warps), and the instance of (128, 64)
-// alone 24; the 24-warp one (threads = 768) 132.
+// warps, where 44 bytes a thread are (416 at 16 warps); the instance of (128, 64)
+// alone spills 24, that of the pair form alone 16, the 24-warp one (threads = 768) 132.
 template <int WARPS, int TILES, int FORMS, uint32_t ONE = 0>
 __global__ void __launch_bounds__(WARPS * 32, 1) k_decode_shape(const DecodeParams p, const WarpParams wp,
                                                                 const __grid_constant__ ShapeMaps maps) {
