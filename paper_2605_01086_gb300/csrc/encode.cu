@@ -1191,8 +1191,8 @@ __global__ void __launch_bounds__(kAnyWarps * 32, 4) k_enc_levels_any(EncParams 
     cp_async_wait_group<0>();
     __syncwarp();
     // ---- fold: lane (or lanes' turn t) = window and every other piece of four pairs
-    for (uint32_t t = lane; t < 2 * nw; t += 32) {
-      const uint32_t h = t < nw ? 0u : 1u, w = t - h * nw;
+    for (uint32_t t = lane; t < 2 * tile; t += 32) {
+      const uint32_t w = t % tile, h = t / tile;
       const float *x = xs + w * xp;
       float su = 0.0f, sv = 0.0f;
       for (uint32_t c = 4 * h; c < P4; c += 8) {
@@ -1226,10 +1226,9 @@ __global__ void __launch_bounds__(kAnyWarps * 32, 4) k_enc_levels_any(EncParams 
     }
     __syncwarp();
     if (w0 + tile < un.n) load(w0 + tile);
-    // ---- bins, four windows x four bins a lane and round (a tile that is not full
-    // takes fewer rounds; what its last lanes' windows past nw hold is not used)
+    // ---- bins, four windows x four bins a lane and round
     const uint64_t win = un.win + w0;
-    const uint32_t wgs = (nw + 3) / 4, items = wgs * (ge + go);
+    const uint32_t wgs = tile / 4, items = wgs * (ge + go);
     for (uint32_t i0 = 0; i0 < items; i0 += 32) {
       const uint32_t item = i0 + lane;
       uint32_t undecided = 0, wg = 0, k0 = 0;
@@ -1406,10 +1405,10 @@ struct EncBins {
   uint32_t base;
 };
 // Streams of one window or of at most a warp's bins: a warp of k_enc_levels_any
-// takes 2 ns (N = 4) to 11 ns (N = E = 128) for one however few windows it has, as
+// takes 2.3 ns (N = 4) to 18 ns (N = E = 128) for one however few windows it has, as
 // compensated sums a thread each they take 0.2 to 5.  200,000 streams of four samples
-// at N = 4: 427 us there, 37 here; of twenty at (24, 12) 480 and 102; of forty at
-// (128, 128) 2190 and 1013; of 100 at (64, 32), two windows, 660 there.
+// at N = 4: 466 us there, 36 here, of 32 475 and 254; of twenty at (24, 12) 501 and
+// 102; of forty at (64, 32) 638 and 270, at (128, 128) 3645 and 1013.
 __host__ __device__ constexpr bool few_bins(uint64_t n_windows, uint32_t E) { return n_windows == 1 || n_windows * E <= 32; }
 
 __global__ void __launch_bounds__(256) k_enc_levels_bins(EncParams p) {
